@@ -38,25 +38,6 @@ namespace fqt {
 // ---------------------------------------------------------------------------
 // Split-K reduction (int64) and the grad_W / raw epilogues
 // ---------------------------------------------------------------------------
-struct ReduceArgs {
-  const int32_t *part;
-  int splits;
-  int64_t M, N;
-  int64_t *out_i64;  // raw sums (debug)
-  float *out_f32;    // grad_W
-  // grad_W = inv_s1 inv_sx sum_n (a_nc + z'_1)(x_nd + z'_x)
-  int64_t Kn;        // rows N of dH / X
-  int oa, ob;
-  // an implicit im2col X~: its padding entered the product as code 2^(bx-1);
-  // P += (code(0) - ob) pad_a[c][tap(d)], pad_a = the A carriers summed over
-  // the rows whose tap reads padding (C x taps), tap(d) = d / cin
-  const int32_t *pad_a, *code_zero;
-  int taps, cin;
-  const int32_t *cs_a, *cs_b;  // column sums of Q_b1 codes (M) and X~ codes (N)
-  const float *inv_a, *zero_a, *inv_b, *zero_b;
-  int vec;  // four outputs per thread (N % 4 == 0, 16-byte aligned buffers)
-};
-
 // A thread sums four consecutive outputs of one row over all splits (one
 // 16-byte load per split, coalesced across the warp, two splits in flight)
 // and dequantizes them (r.vec; else one output per thread).
@@ -231,11 +212,14 @@ struct SplitPlan {
   int64_t ks_blocks, kb_total;
 };
 
+// pair: super tiles of 256 x 256 for CTA pairs.
 static SplitPlan plan_splits(int64_t M, int64_t N, int64_t K, int a_bits,
-                             int b_bits, int num_sms, bool allow_split) {
+                             int b_bits, int num_sms, bool allow_split, bool pair = false) {
   SplitPlan p;
-  p.m_tiles = (int)((M + BM - 1) / BM);
-  p.n_tiles = (int)((N + BN - 1) / BN);
+  const int64_t tm = pair ? 2 * BM : BM, tn = pair ? 2 * BN : BN;
+  if (pair) num_sms /= 2;
+  p.m_tiles = (int)((M + tm - 1) / tm);
+  p.n_tiles = (int)((N + tn - 1) / tn);
   p.kb_total = (K + BK - 1) / BK;
   if (p.kb_total < 1) p.kb_total = 1;
   int splits = 1;
@@ -284,8 +268,12 @@ size_t gemm_workspace_bytes(int64_t N, int64_t C, int64_t D) {
     int64_t sp = use_gradw(w, nsm) ? w.splits : plan_splits(C, D, N, b, 8, nsm, true).splits;
     // an implicit im2col operand pads each image's output rows to blocks of
     // 64 slots: at most 2.4 N slots (ow = 9 in blocks of 4 rows of 16)
-    const int64_t sc = plan_splits(C, D, (N * 5 + 1) / 2, b, 8, nsm, true).splits;
+    const int64_t Kp = (N * 5 + 1) / 2;
+    const int64_t sc = plan_splits(C, D, Kp, b, 8, nsm, true).splits;
     if (sc > sp) sp = sc;
+    // CTA pairs (more than 128 rows of grad_W)
+    const int64_t s2 = C > BM ? plan_splits(C, D, Kp, b, 8, nsm, true, true).splits : 0;
+    if (s2 > sp) sp = s2;
     if (sp > splits) splits = sp;
   }
   // + the padding table of an implicit im2col X~ (C x taps, taps <= D)
@@ -293,7 +281,21 @@ size_t gemm_workspace_bytes(int64_t N, int64_t C, int64_t D) {
   return (bytes + 255) & ~(size_t)255;
 }
 
-typedef void (*GemmKernel)(CUtensorMap, CUtensorMap, CUtensorMap, GemmArgs);
+// Whether a contraction takes CTA pairs: p the plan of single CTAs, q that of
+// pairs.  A K block takes about the same time in either (0.41 us for a CTA's
+// 128 x 128, 0.42-0.49 us for a pair's 256 x 256, measured on reductions of
+// 1024 to 8192), so the one with clearly fewer K blocks in its longest chain
+// of waves is taken (three more per item for its start and end).  Measured,
+// 8192 tokens 1024 <-> 4096: grad_X 92 -> 57 us and 86 -> 54 us, forward 86
+// -> 55 us, grad_W 119 -> 63 us with its reduction fused.  Fewer than four K
+// blocks are bound by the output's stores, where the pair has nothing to
+// give.
+static bool pair_faster(const SplitPlan &p, const SplitPlan &q, int num_sms) {
+  const int64_t one = ((int64_t)p.m_tiles * p.n_tiles * p.splits + num_sms - 1) / num_sms;
+  const int64_t two =
+      ((int64_t)q.m_tiles * q.n_tiles * q.splits + num_sms / 2 - 1) / (num_sms / 2);
+  return q.kb_total >= 4 && 10 * two * (q.ks_blocks + 3) < 9 * one * (p.ks_blocks + 3);
+}
 
 // The kernel instance of a mode, BHQ block size (1 = no reflection) and
 // product representation (fp32-exact or int32).
@@ -346,7 +348,7 @@ static GemmKernel gemm_kernel(int mode, int nb, int form) {
 static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *Bm,
                            int b_kmajor, int b_bits, int64_t M, int64_t N, int64_t K,
                            const SplitPlan &p, GemmArgs &g, void *out, int mode, int nb,
-                           int form, cudaStream_t st) {
+                           int form, cudaStream_t st, bool pair = false) {
   const bool partial = mode == MODE_PARTIAL;
   // byte operands (g.u8): split-K partials of MN-major operands only
   if (g.u8 && (!partial || a_kmajor || b_kmajor)) return FQT_EUNSUPPORTED;
@@ -374,10 +376,20 @@ static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *
                                      (uint64_t)p.splits)
                       : make_map_out(&to, out, false, (uint64_t)M, (uint64_t)N, 1));
   if (!ok) return cuda_fail(cudaErrorInvalidValue, "tensor map encode");
-  GemmKernel kern = gemm_kernel(mode, nb, form);
+  GemmKernel kern = pair ? gemm_pair_kernel(mode, nb, form) : gemm_kernel(mode, nb, form);
   if (!kern) return FQT_EUNSUPPORTED;
   const bool four = !partial && form == 2;  // GemmLayout: four epilogue sets
-  const int threads = four ? GemmLayout<0, 2>::threads : GemmLayout<0, 0>::threads;
+  using LP = GemmLayout<1, 0, 1, true>;
+  const int threads = partial && pair ? LP::threads
+                      : four          ? GemmLayout<0, 2>::threads
+                                      : GemmLayout<0, 0>::threads;
+  if (partial && pair) {  // the register split, as below
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess) return cuda_fail(e, "gemm attributes");
+    if (fa.numRegs * LP::threads < 128 * LP::regs_ctl + 256 * LP::regs_epi)
+      return FQT_EUNSUPPORTED;
+  }
   if (four) {
     // the register split needs the launch's registers per thread: with fewer,
     // setmaxnreg.inc would wait for registers that do not exist
@@ -392,7 +404,8 @@ static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *
   }
   // the fp32 form: four epilogue sets for tiles bound by their output, three
   // for long reductions; the code bits for the final pass over raw tiles
-  g.sets = (four && (K + BK - 1) / BK <= 2) ? 4 : 3;
+  // (a pair's accumulators change over two at a time: all four sets)
+  g.sets = (four && (pair || (K + BK - 1) / BK <= 2)) ? 4 : 3;
   g.bw = a_bits;
   g.b2 = b_bits;
   g.small_p = (K << (a_bits + b_bits - 2)) < ((int64_t)1 << 22);
@@ -443,6 +456,27 @@ static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (ea != cudaSuccess) return cuda_fail(ea, "gemm shared-memory attribute");
   const int nsm = device_sm_count();
+  if (pair) {
+    int64_t pairs = g.n_items < nsm / 2 ? g.n_items : nsm / 2;
+    if (pairs < 1) pairs = 1;
+    // two tiles per super tile
+    if (!partial && 2 * ((g.n_items + pairs - 1) / pairs) > kMaxLocalTiles)
+      return FQT_EUNSUPPORTED;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cuda_fail(cudaLaunchKernelEx(&cfg, kern, ta, tb, to, g), "gemm pair launch");
+  }
   int64_t grid = g.n_items < nsm ? g.n_items : nsm;
   if (grid < 1) grid = 1;
   // the raw-tile bits of a CTA cover kMaxLocalTiles of its tiles
@@ -912,8 +946,11 @@ fqt_status linear_forward(const fqt_qtensor *qx, const fqt_qtensor *qw, float *H
   g.zero_w = qw->zero;
   g.flt_mmax = flt ? (float)mmax : -1.0f;
   g.i32_mmax = int32_form_mmax(D, qw->bits, qx->bits, 1);
-  return run_gemm(qw->codes_f16, 1, qw->bits, qx->codes_f16, 1, qx->bits, C, Nr, D, p, g, H,
-                  MODE_GRADX, 1, epilogue_form(flt, mmax, qx->bits), st);
+  const SplitPlan pp = plan_splits(C, Nr, D, qw->bits, qx->bits, nsm, false, true);
+  const bool pair = flt && pair_faster(p, pp, nsm);
+  return run_gemm(qw->codes_f16, 1, qw->bits, qx->codes_f16, 1, qx->bits, C, Nr, D,
+                  pair ? pp : p, g, H, MODE_GRADX, 1, epilogue_form(flt, mmax, qx->bits), st,
+                  pair);
 }
 
 // ---------------------------------------------------------------------------
@@ -1380,9 +1417,12 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
       g.perm = q_b2->perm;
       g.gsize = q_b2->gsize;
       g.raw_mmax = (float)mmax;
+      const SplitPlan pp = plan_splits(D, Nr, C, qw->bits, q_b2->bits, nsm, false, true);
+      const int form = adapt ? 2 : epilogue_form(flt, mmax, q_b2->bits);
+      const bool pair = C <= kc_terms && gemm_pair_kernel(MODE_GRADX, nb, form) &&
+                        pair_faster(p, pp, nsm);
       fqt_status s = run_gemm(qw->codes_f16, 0, qw->bits, q_b2->codes_f16, 1, q_b2->bits,
-                              D, Nr, C, p, g, grad_X, MODE_GRADX, nb,
-                              adapt ? 2 : epilogue_form(flt, mmax, q_b2->bits), st);
+                              D, Nr, C, pair ? pp : p, g, grad_X, MODE_GRADX, nb, form, st, pair);
       if (s != FQT_OK) return s;
       if (adapt) {
         FixArgs f;
@@ -1489,7 +1529,7 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
       }
     }
     const bool conv_tile = cpw > 0;
-    const SplitPlan p = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true);
+    SplitPlan p = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true);
     const WPlan wp = Nr > 0 ? gradw_plan(Nr, C, D, a_bits, x_bits, nsm) : WPlan{};
     // k_gradw serves the implicit im2col operand with wider output rows (4-D
     // boxes of 32 pixels of one row, ow % 32 == 0); plain matrices take the
@@ -1498,6 +1538,17 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
     // operands
     const bool w_ok = use_gradw(wp, nsm) && conv && !conv_tile;
     if (conv && Nr > 0 && !w_ok && !conv_tile) return FQT_EUNSUPPORTED;
+    // CTA pairs where their plan is faster and its partials fit the workspace
+    const int64_t pad_bytes = conv ? C * qx->conv[4] * qx->conv[5] * 4 : 0;
+    bool pair = false;
+    if (Nr > 0 && !w_ok && !bytes && C > BM) {
+      const SplitPlan pp = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true, true);
+      pair = pair_faster(p, pp, nsm) &&
+             (int64_t)kGemmOffset + pp.splits * C * D * 4 + pad_bytes <= (int64_t)ws_bytes;
+      if (pair) p = pp;
+    }
+    // one split: the pair's epilogue dequantizes, no partials and no reduction
+    const bool fuse = pair && p.splits == 1 && !conv && aligned16(grad_W);
     const int splits = w_ok ? wp.splits : p.splits;
     const size_t pbytes = (size_t)splits * (size_t)C * (size_t)D * 4;
     const int taps = conv ? qx->conv[4] * qx->conv[5] : 0;
@@ -1529,6 +1580,29 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
         if (e != cudaSuccess) return cuda_fail(e, "padding sums launch");
       }
     }
+    ReduceArgs r;
+    memset(&r, 0, sizeof(r));
+    r.part = part;
+    r.splits = Nr > 0 ? splits : 1;
+    r.M = C;
+    r.N = D;
+    r.out_f32 = grad_W;
+    r.Kn = Nr;
+    // shifted codes are their own carriers (offset 0, zero point 0)
+    r.oa = shifted ? 0 : 1 << (qa->bits - 1);
+    r.ob = 1 << (qx->bits - 1);
+    r.cs_a = shifted ? qa->shift_col_sum : qa->col_sum;
+    r.cs_b = qx->col_sum;
+    if (conv) {
+      r.pad_a = pad_a;
+      r.code_zero = qx->col_sum + D;
+      r.taps = taps;
+      r.cin = qx->conv[3];
+    }
+    r.inv_a = shifted ? qa->shift_scale : qa->inv_s;
+    r.zero_a = shifted ? qa->shift_scale + 1 : qa->zero;
+    r.inv_b = qx->inv_s;
+    r.zero_b = qx->zero;
     if (Nr > 0 && w_ok) {
       fqt_status s = run_gradw(qx->codes_f16, static_cast<const uint16_t *>(A16), Nr, (int)C,
                                (int)D, wp, part, status, st, conv ? qx->conv : nullptr);
@@ -1553,36 +1627,16 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
         g.coh = cv[1] + 2 * cv[6] - cv[4] + 1;
         g.cow = cv[2] + 2 * cv[6] - cv[5] + 1;
       }
+      g.fuse = fuse ? 1 : 0;
+      g.red = r;
       fqt_status s = run_gemm(A16, 0, a_bits, X16, 0, qx->bits, C, D, Kt, p, g,
-                              part, MODE_PARTIAL, 1, false, st);
+                              fuse ? (void *)grad_W : (void *)part, MODE_PARTIAL, 1, 0, st, pair);
       if (s != FQT_OK) return s;
+      if (fuse) return FQT_OK;
     } else {
       const cudaError_t e = cudaMemsetAsync(part, 0, (size_t)C * D * 4, st);
       if (e != cudaSuccess) return cuda_fail(e, "partial clear");
     }
-    ReduceArgs r;
-    memset(&r, 0, sizeof(r));
-    r.part = part;
-    r.splits = Nr > 0 ? splits : 1;
-    r.M = C;
-    r.N = D;
-    r.out_f32 = grad_W;
-    r.Kn = Nr;
-    // shifted codes are their own carriers (offset 0, zero point 0)
-    r.oa = shifted ? 0 : 1 << (qa->bits - 1);
-    r.ob = 1 << (qx->bits - 1);
-    r.cs_a = shifted ? qa->shift_col_sum : qa->col_sum;
-    r.cs_b = qx->col_sum;
-    if (conv) {
-      r.pad_a = pad_a;
-      r.code_zero = qx->col_sum + D;
-      r.taps = taps;
-      r.cin = qx->conv[3];
-    }
-    r.inv_a = shifted ? qa->shift_scale : qa->inv_s;
-    r.zero_a = shifted ? qa->shift_scale + 1 : qa->zero;
-    r.inv_b = qx->inv_s;
-    r.zero_b = qx->zero;
     launch_reduce(r, st);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "split-K reduce launch");

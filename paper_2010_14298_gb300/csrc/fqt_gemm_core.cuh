@@ -37,14 +37,16 @@ constexpr int kPartialEpiWarps = 8;
 // Otherwise three sets at 128 registers; split-K partials use the first
 // eight epilogue warps.
 constexpr int kGemmWarpPar = 2, kGemmWarpEpi0 = 4;
-template <int MODE, int FORM, int NB = 16>
+// A pair's partials (PAIR, MODE 1) keep their int32 running sums in the
+// registers of two sets (128 columns each, 128 sums per thread).
+template <int MODE, int FORM, int NB = 16, bool PAIR = false>
 struct GemmLayout {
-  static constexpr int sets = (MODE == 0 && FORM == 2) ? 4 : 3;  // MODE 0: grad_X
+  static constexpr int sets = (MODE == 0 && FORM == 2) ? 4 : (MODE == 1 && PAIR) ? 2 : 3;
   static constexpr int threads = 32 * (kGemmWarpEpi0 + 4 * sets);
   // registers per thread of the launch, and the split (0: no setmaxnreg)
   static constexpr int launch_regs = ((65536 / threads) / 8) * 8;
-  static constexpr int regs_ctl = sets == 4 ? (NB <= 16 ? 80 : 64) : 0;
-  static constexpr int regs_epi = sets == 4 ? (NB <= 16 ? 96 : 104) : 0;
+  static constexpr int regs_ctl = sets == 4 ? (NB <= 16 ? 80 : 64) : sets == 2 ? 80 : 0;
+  static constexpr int regs_epi = sets == 4 ? (NB <= 16 ? 96 : 104) : sets == 2 ? 208 : 0;
   static_assert(regs_ctl == 0 || 128 * regs_ctl + 32 * 4 * sets * regs_epi <= threads * launch_regs,
                 "register split above the launch's registers");
 };
@@ -91,6 +93,27 @@ __host__ __device__ constexpr size_t gemm_smem_bytes(int stages, int ring, int u
 // dequantizing epilogue.  MODE_PARTIAL: raw int32 split-K partials.
 enum { MODE_GRADX = 0, MODE_PARTIAL = 1 };
 
+// Dequantization of grad_W's integer products (k_reduce, and the epilogue of
+// a pair's partials when one split covers the reduction).
+struct ReduceArgs {
+  const int32_t *part;
+  int splits;
+  int64_t M, N;
+  int64_t *out_i64;  // raw sums (debug)
+  float *out_f32;    // grad_W
+  // grad_W = inv_s1 inv_sx sum_n (a_nc + z'_1)(x_nd + z'_x)
+  int64_t Kn;        // rows N of dH / X
+  int oa, ob;
+  // an implicit im2col X~: its padding entered the product as code 2^(bx-1);
+  // P += (code(0) - ob) pad_a[c][tap(d)], pad_a = the A carriers summed over
+  // the rows whose tap reads padding (C x taps), tap(d) = d / cin
+  const int32_t *pad_a, *code_zero;
+  int taps, cin;
+  const int32_t *cs_a, *cs_b;  // column sums of Q_b1 codes (M) and X~ codes (N)
+  const float *inv_a, *zero_a, *inv_b, *zero_b;
+  int vec;  // four outputs per thread (N % 4 == 0, 16-byte aligned buffers)
+};
+
 struct GemmArgs {
   int64_t M, N, K;            // out is M x N, reduction over K
   int a_kmajor, b_kmajor;     // operand storage (see fqt_debug_int_gemm)
@@ -128,6 +151,9 @@ struct GemmArgs {
   // read as 4-D boxes of (64 channels, pw, rpb, 1)
   int conv, cpw, crpb, cybi, coh, cih, cin, ckw, cpad, cow, ciw;
   int64_t cnimg;
+  // a pair's partials with one split: grad_W itself (red) instead of partials
+  int fuse;
+  ReduceArgs red;
   int *status;
 };
 
@@ -153,6 +179,47 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, i
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3),
       "r"(smem_u32(bar))
       : "memory");
+}
+
+// The same loads issued by either CTA of a pair (cta_group::2): dst is this
+// CTA's shared memory, bar the cluster address of the barrier that counts
+// the bytes (the leader's).
+__device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, int32_t c0,
+                                                 int32_t c1, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
+      : "memory");
+}
+
+__device__ __forceinline__ void tma_load_4d_pair(void *dst, const CUtensorMap *map, int32_t c0,
+                                                 int32_t c1, int32_t c2, int32_t c3,
+                                                 uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+      : "memory");
+}
+
+// Cluster address of a shared-memory object of the pair's leader (rank 0).
+__device__ __forceinline__ uint32_t leader_addr(const void *p) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(p)));
+  return r;
+}
+
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar)
+               : "memory");
+}
+
+// Barrier of both CTAs of a pair (every thread of both reaches it).
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile(
+      "barrier.cluster.arrive.release.aligned;\n\t"
+      "barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int32_t c0,
@@ -225,12 +292,12 @@ __device__ __forceinline__ uint64_t sw128_desc_mn(uint32_t saddr, uint32_t lbo,
   return d;
 }
 
-// Instruction descriptor of kind::f16: A, B fp16, D fp32, M = 128, N = 128;
+// Instruction descriptor of kind::f16: A, B fp16, D fp32, M x N (128 x 128);
 // bit 15 / 16 select MN-major A / B.
-__host__ __device__ constexpr uint32_t make_idesc(bool a_mn, bool b_mn) {
+__host__ __device__ constexpr uint32_t make_idesc(bool a_mn, bool b_mn, int m = BM,
+                                                  int n = BN) {
   return (1u << 4) | (0u << 7) | (0u << 10) | ((a_mn ? 1u : 0u) << 15) |
-         ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(BN >> 3) << 17) |
-         ((uint32_t)(BM >> 4) << 24);
+         ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t a_desc,
@@ -241,6 +308,27 @@ __device__ __forceinline__ void umma_f16(uint32_t tmem_d, uint64_t a_desc,
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// M = 256 over the two CTAs of a pair (each CTA's shared memory holds its
+// 128 rows of A and its half of B's columns, at the same offsets).
+__device__ __forceinline__ void umma_f16_pair(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc,
+                                              uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// Arrives on the barrier at this offset in both CTAs of the pair.
+__device__ __forceinline__ void umma_commit_pair(uint64_t *bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;" ::"r"(smem_u32(bar)),
+      "h"((uint16_t)3)
       : "memory");
 }
 
@@ -393,6 +481,36 @@ __device__ __forceinline__ Item decode_item(const GemmArgs &g, int64_t it) {
   r.kb0 = (int64_t)r.split * g.ks_blocks;
   r.kb1 = min(g.kb_total, r.kb0 + g.ks_blocks);
   return r;
+}
+
+// The tiles of a CTA in its order.  A CTA on its own takes items blockIdx.x +
+// local gridDim.x.  The CTAs of a pair (PAIR) take super tiles of 256 x 256,
+// every (gridDim.x / 2)-th one: each CTA the 128 output rows M of its rank,
+// as two tiles of 128 columns N (local = 2 super + half).  Returns false
+// past the last.
+template <bool PAIR>
+__device__ __forceinline__ bool cta_item(const GemmArgs &g, int64_t local, Item &t) {
+  if constexpr (PAIR) {
+    const int64_t it = (int64_t)(blockIdx.x >> 1) + (local >> 1) * (int64_t)(gridDim.x >> 1);
+    if (it >= g.n_items) return false;
+    t = decode_item(g, it);
+    t.m0 = 2 * t.m0 + (int64_t)(blockIdx.x & 1) * BM;
+    t.n0 = 2 * t.n0 + (local & 1) * BN;
+    return true;
+  } else {
+    const int64_t it = (int64_t)blockIdx.x + local * (int64_t)gridDim.x;
+    if (it >= g.n_items) return false;
+    t = decode_item(g, it);
+    return true;
+  }
+}
+
+// The accumulator's consumer is done with it: the pair's MMA issuer (the
+// leader) counts the arrivals of both CTAs.
+template <bool PAIR>
+__device__ __forceinline__ void acc_release(uint64_t *bar) {
+  if constexpr (PAIR) mbar_arrive_cluster(leader_addr(bar));
+  else mbar_arrive(bar);
 }
 
 // The items of one step of a CTA's schedule: item it, and with pairs the
@@ -576,7 +694,7 @@ __device__ __forceinline__ void box_small(const Ints &I, const int (&Ip)[leads_p
 // rows (a box, or one block of NB > 32 rows spanning several boxes).  raw: a
 // tile outside both forms, whose row terms are units (m = 0, so I = P): its
 // exact products P are stored as int32 bit patterns for gradx_raw_fix.
-template <int NB>
+template <int NB, bool PAIR>
 __device__ __forceinline__ void gradx_tile(const GemmArgs &g, const Item &t, uint32_t acc,
                                            uint32_t ints, bool multi, const float4 *kp,
                                            const int *leads, const HhConst &hc, float cwc,
@@ -618,7 +736,7 @@ __device__ __forceinline__ void gradx_tile(const GemmArgs &g, const Item &t, uin
       if (r0 + 32 == BN) {  // the accumulator has been read in full
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(acce_set);
+        if (lane == 0) acc_release<PAIR>(acce_set);
       }
       if (raw) {
         w.st32(reinterpret_cast<const float (&)[32]>(I.v));
@@ -670,7 +788,7 @@ __device__ __forceinline__ float reflect_f(float P, const float4 &kq, float cwc,
 // |m| <= mmax).  Block sums S = sum P + CWc sum m, I_p = P_p + m_p CWc.
 // raw: a tile outside the fp32 form, whose row terms are units (1, 0, 0, 0):
 // no block is transformed, so the stores are its exact products P.
-template <int NB>
+template <int NB, bool PAIR>
 __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, uint32_t acc,
                                              const float4 *kp, const int *leads,
                                              const int *msum, const HhConst &hc, float cwc,
@@ -700,7 +818,7 @@ __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, u
       if (r0 + CH == BN) {  // the accumulator has been read in full
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(acce_set);
+        if (lane == 0) acc_release<PAIR>(acce_set);
       }
       const int64_t row0 = t.n0 + r0;
       const int64_t left = g.N - row0;
@@ -813,7 +931,7 @@ __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, u
       if (r0 + 32 == BN) {  // the accumulator has been read in full
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(acce_set);
+        if (lane == 0) acc_release<PAIR>(acce_set);
       }
       // every output of the box is formed in registers before the first
       // store, so the per-row loads from shared memory need not wait for
@@ -950,7 +1068,7 @@ __device__ __forceinline__ void tile_loads(const GemmArgs &g, const Item &t, int
 // order, the per-row terms of its rows and the column sums of its columns go
 // into a parameter stage ahead of the epilogue warps that use them.  The
 // global loads of the next tile are in flight while this tile's are used.
-template <int NB, int FORM>
+template <int NB, int FORM, bool PAIR>
 __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, uint64_t *pfull,
                                              uint64_t *pempty, volatile int *abort_flag,
                                              int lane) {
@@ -959,15 +1077,15 @@ __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, u
   const ff y = two_sum((float)g.ow, zw);
   const int Cn = (int)g.K;
   TileLoads cur, nxt;
-  if ((int64_t)blockIdx.x < g.n_items) tile_loads<NB>(g, decode_item(g, blockIdx.x), lane, cur);
-  int64_t local = 0;
-  for (int64_t it = blockIdx.x; it < g.n_items && !*abort_flag; it += gridDim.x, ++local) {
-    if (it + gridDim.x < g.n_items) tile_loads<NB>(g, decode_item(g, it + gridDim.x), lane, nxt);
+  Item t;
+  if (cta_item<PAIR>(g, 0, t)) tile_loads<NB>(g, t, lane, cur);
+  for (int64_t local = 0; cta_item<PAIR>(g, local, t) && !*abort_flag; ++local) {
+    Item tn;
+    if (cta_item<PAIR>(g, local + 1, tn)) tile_loads<NB>(g, tn, lane, nxt);
     const int s = (int)(local % kParStages);
     const uint32_t wrap = (uint32_t)(local / kParStages);
     const bool got = mbar_wait(&pempty[s], (wrap & 1u) ^ 1u, g.status);
     if (!__all_sync(0xffffffffu, got)) { *abort_flag = 1; break; }
-    const Item t = decode_item(g, it);
     uint8_t *P = smem + kOffPar + (size_t)s * kParBytes;
     float4 *kp = reinterpret_cast<float4 *>(P);
     int *leads = reinterpret_cast<int *>(P + kParLeads);
@@ -1064,7 +1182,7 @@ __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, u
   }
 }
 
-template <int NB, int FORM>
+template <int NB, int FORM, bool PAIR>
 __device__ __forceinline__ void gradx_epilogue(const GemmArgs &g, uint8_t *smem,
                                                uint8_t *ring, uint64_t *accf,
                                                uint64_t *acce, uint64_t *pfull,
@@ -1081,11 +1199,10 @@ __device__ __forceinline__ void gradx_epilogue(const GemmArgs &g, uint8_t *smem,
   HhConst hc = {{0.0f, 0.0f}, {0.0f, 0.0f}};
   if (NB > 1) hc = hh_const(NB);
   bool ok = true;
-  // this CTA's tiles local = set, set + g.sets, ... (item blockIdx.x + local * grid)
+  // this CTA's tiles local = set, set + g.sets, ...
   for (int64_t local = set; set < g.sets; local += g.sets) {
-    const int64_t it = (int64_t)blockIdx.x + local * (int64_t)gridDim.x;
-    if (it >= g.n_items || *abort_flag) break;
-    const Item t = decode_item(g, it);
+    Item t;
+    if (!cta_item<PAIR>(g, local, t) || *abort_flag) break;
     const int buf = (int)(local & (g.nacc - 1));
     const uint32_t acc = lane_base + (uint32_t)(buf * BN);
     // int32 running sums (two accumulators only): columns 256 + 128 buf
@@ -1136,22 +1253,22 @@ __device__ __forceinline__ void gradx_epilogue(const GemmArgs &g, uint8_t *smem,
       if (!last_chunk || !active) {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acce[buf]);
+        if (lane == 0) acc_release<PAIR>(&acce[buf]);
         continue;
       }
       const bool multi = c > 0;
       if constexpr (NB == 0) {
-        gradx_tile_f<0>(g, t, acc, kp, leads, msum, hc, cwc, U, &acce[buf], q, lane, false);
+        gradx_tile_f<0, PAIR>(g, t, acc, kp, leads, msum, hc, cwc, U, &acce[buf], q, lane, false);
       } else {
         if constexpr (FORM == 2) {
           // a tile outside the fp32 form has unit row terms (kq = (1, 0, 0, 0)):
           // the one-row epilogue stores its exact products P for gradx_raw_fix
-          gradx_tile_f<NB>(g, t, acc, kp, leads, msum, hc, cwc, U, &acce[buf], q, lane,
+          gradx_tile_f<NB, PAIR>(g, t, acc, kp, leads, msum, hc, cwc, U, &acce[buf], q, lane,
                            tform != 1);
         } else if (FORM == 1 && tform == 1) {
-          gradx_tile_f<NB>(g, t, acc, kp, leads, msum, hc, cwc, U, &acce[buf], q, lane, false);
+          gradx_tile_f<NB, PAIR>(g, t, acc, kp, leads, msum, hc, cwc, U, &acce[buf], q, lane, false);
         } else {
-          gradx_tile<NB>(g, t, acc, ints, multi, kp, leads, hc, cwc, U, &acce[buf], q, lane,
+          gradx_tile<NB, PAIR>(g, t, acc, ints, multi, kp, leads, hc, cwc, U, &acce[buf], q, lane,
                          tform == 0);
         }
       }
@@ -1354,14 +1471,263 @@ static __device__ __noinline__ void partial_convert(const GemmArgs &g, uint8_t *
   }
 }
 
+// ---------------------------------------------------------------------------
+// Roles of a CTA pair (PAIR)
+// ---------------------------------------------------------------------------
+// TMA producer: this CTA's 128 rows of A and its 128 of the super tile's 256
+// columns of B; the leader's full barrier counts the bytes of both CTAs.
+template <int MODE>
+__device__ __forceinline__ void produce_pair(const GemmArgs &g, const CUtensorMap &tmA,
+                                             const CUtensorMap &tmB, uint8_t *ops,
+                                             uint64_t *full, uint64_t *empty,
+                                             volatile int *abort_flag, int &s, uint32_t &ph) {
+  const int rank = (int)(blockIdx.x & 1);
+  Item t;
+  for (int64_t local = 0; cta_item<true>(g, local, t) && !*abort_flag; local += 2) {
+    const int32_t m0 = (int32_t)t.m0, n0 = (int32_t)t.n0 + rank * BN;
+    // implicit im2col (see the single-CTA producer)
+    int cimg = 0, cyb = 0, ccg[2] = {0, 0}, ckx[2] = {0, 0}, cky[2] = {0, 0};
+    bool cval[2] = {false, false};
+    if (MODE == MODE_PARTIAL && g.conv) {
+      cimg = (int)(t.kb0 / g.cybi);
+      cyb = (int)(t.kb0 - (int64_t)cimg * g.cybi);
+      for (int h = 0; h < 2; ++h) {
+        const int d = n0 + 64 * h;
+        const int tap = d / g.cin;
+        ccg[h] = d - tap * g.cin;
+        cky[h] = tap / g.ckw;
+        ckx[h] = tap - cky[h] * g.ckw;
+        cval[h] = d < g.N;
+      }
+    }
+    for (int64_t kb = t.kb0; kb < t.kb1; ++kb) {
+      if (!mbar_wait(&empty[s], ph ^ 1u, g.status)) { *abort_flag = 1; return; }
+      if (rank == 0) mbar_expect_tx(&full[s], (uint32_t)(4 * kTileBytes));
+      const uint32_t bar = leader_addr(&full[s]);
+      uint8_t *sa = ops + (size_t)(2 * s) * kTileBytes;
+      uint8_t *sb = sa + kTileBytes;
+      const int32_t kc = (int32_t)(kb * BK);
+      if (MODE == MODE_PARTIAL && g.conv) {
+        const int oy0 = cyb * g.crpb;
+        tma_load_4d_pair(sa, &tmA, m0, 0, oy0, cimg, bar);
+        tma_load_4d_pair(sa + kTileBytes / 2, &tmA, m0 + 64, 0, oy0, cimg, bar);
+        for (int h = 0; h < 2; ++h) {
+          if (cval[h])
+            tma_load_4d_pair(sb + h * (kTileBytes / 2), &tmB, ccg[h], ckx[h] - g.cpad,
+                             oy0 + cky[h] - g.cpad, cimg, bar);
+          else  // past the last tap: a box outside the tensor (zeros)
+            tma_load_4d_pair(sb + h * (kTileBytes / 2), &tmB, 0, 0, g.cih + g.coh + 8, cimg, bar);
+        }
+        if (++cyb == g.cybi) { cyb = 0; ++cimg; }
+      } else {
+        // K-major: one 64 x 128 box; MN-major: two 64 (MN) x 64 (K) boxes
+        if (g.a_kmajor) {
+          tma_load_2d_pair(sa, &tmA, kc, m0, bar);
+        } else {
+          tma_load_2d_pair(sa, &tmA, m0, kc, bar);
+          tma_load_2d_pair(sa + kTileBytes / 2, &tmA, m0 + 64, kc, bar);
+        }
+        if (g.b_kmajor) {
+          tma_load_2d_pair(sb, &tmB, kc, n0, bar);
+        } else {
+          tma_load_2d_pair(sb, &tmB, n0, kc, bar);
+          tma_load_2d_pair(sb + kTileBytes / 2, &tmB, n0 + 64, kc, bar);
+        }
+      }
+      if (++s == g.stages) { s = 0; ph ^= 1u; }
+    }
+  }
+}
+
+// MMA issuer (one lane of the leader): the exact chunks of the super tiles
+// alternate between the two 256-column accumulators.
+__device__ __forceinline__ void issue_pair(const GemmArgs &g, uint8_t *ops, uint64_t *full,
+                                           uint64_t *empty, uint64_t *accf, uint64_t *acce,
+                                           uint64_t *drain, uint32_t tmem,
+                                           volatile int *abort_flag) {
+  int s = 0, b = 0;
+  uint32_t ph = 0, aph = 0u;  // bit b of aph: phase parity of accumulator b
+  const uint32_t idesc = make_idesc(!g.a_kmajor, !g.b_kmajor, 2 * BM, 2 * BN);
+  const uint64_t a_step = g.a_kmajor ? 2u : (2048u >> 4);
+  const uint64_t b_step = g.b_kmajor ? 2u : (2048u >> 4);
+  Item t;
+  bool ok = true;
+  for (int64_t local = 0; ok && cta_item<true>(g, local, t) && !*abort_flag; local += 2) {
+    for (int64_t c0 = t.kb0; ok && c0 < t.kb1; c0 += g.kc_blocks) {
+      const int64_t c1 = min(t.kb1, c0 + g.kc_blocks);
+      const uint32_t par = ((aph >> b) & 1u) ^ 1u;
+      ok = mbar_wait(&acce[2 * b], par, g.status) && mbar_wait(&acce[2 * b + 1], par, g.status);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t dt = tmem + (uint32_t)(b * 2 * BN);
+      for (int64_t kb = c0; kb < c1; ++kb) {
+        if (!mbar_wait(&full[s], ph, g.status)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t a_addr = smem_u32(ops + (size_t)(2 * s) * kTileBytes);
+        const uint32_t b_addr = a_addr + (uint32_t)kTileBytes;
+        const uint64_t da =
+            g.a_kmajor ? sw128_desc(a_addr) : sw128_desc_mn(a_addr, g.mn_lbo, g.mn_sbo);
+        const uint64_t db =
+            g.b_kmajor ? sw128_desc(b_addr) : sw128_desc_mn(b_addr, g.mn_lbo, g.mn_sbo);
+#pragma unroll
+        for (int k = 0; k < BK / 16; ++k)
+          umma_f16_pair(dt, da + a_step * k, db + b_step * k, idesc, (kb > c0 || k > 0) ? 1u : 0u);
+        umma_commit_pair(&empty[s]);
+        if (++s == g.stages) { s = 0; ph ^= 1u; }
+      }
+      umma_commit_pair(&accf[2 * b]);
+      umma_commit_pair(&accf[2 * b + 1]);
+      aph ^= 1u << b;
+      b ^= 1;
+    }
+  }
+  if (!ok) *abort_flag = 1;
+  // every MMA has completed before tensor memory is released
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+          smem_u32(drain))
+      : "memory");
+  mbar_wait(drain, 0, g.status);
+}
+
+// Split-K partials of a pair: set h (warps 4 h ..) owns the 128 columns of
+// half h; a thread keeps its row's 128 int32 running sums in registers, adds
+// each exact chunk to them and at the end stores four 32 x 32 boxes, the
+// partials or, with one split (g.fuse), grad_W dequantized as k_reduce would.
+// Column terms of a super tile in shared memory: ka cb (int64) and cb - Kn mb
+// (fp32) per column, written by the 256 threads together.
+__device__ __forceinline__ void partial_epilogue_pair(const GemmArgs &g, uint8_t *smem,
+                                                      uint8_t *ring, uint64_t *accf,
+                                                      uint64_t *acce, uint32_t tmem,
+                                                      const CUtensorMap *tmOut,
+                                                      volatile int *abort_flag, int warp,
+                                                      int lane) {
+  const int ew = warp - kGemmWarpEpi0, q = warp & 3, h = ew >> 2;
+  uint8_t *box = ring + (size_t)ew * kBoxBytes;
+  const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * BN);
+  long long *col_i = reinterpret_cast<long long *>(smem + kOffPar);          // [256]
+  float *col_f = reinterpret_cast<float *>(smem + kOffPar + 256 * 8);        // [256]
+  const ReduceArgs &r = g.red;
+  float sab = 0.0f, kdd = 0.0f, da = 0.0f, db = 0.0f;
+  int64_t ka = 0, kb = 0, k0 = 0, ma = 0, mb = 0;
+  if (g.fuse) {
+    const float za = *r.zero_a, zb = *r.zero_b;
+    sab = (*r.inv_a) * (*r.inv_b);
+    ma = __float2int_rn(-za);
+    mb = __float2int_rn(-zb);
+    da = za + (float)ma;
+    db = zb + (float)mb;
+    kdd = ll_to_float(r.Kn) * da * db;
+    ka = r.oa - ma;
+    kb = r.ob - mb;
+    k0 = r.Kn * ka * kb - ka * r.Kn * r.ob - kb * r.Kn * r.oa;
+  }
+  uint32_t cc = 0;  // exact chunks so far
+  bool dead = false;
+  bool stored = false;
+  Item t;
+  // the same trip count in all eight warps (they meet at named barriers)
+  for (int64_t local = 0; cta_item<true>(g, local + h, t); local += 2) {
+    dead = dead || *abort_flag;
+    float rt = 0.0f;
+    int64_t Ia = 0;
+    if (g.fuse) {
+      const int64_t d = t.n0 - h * BN + ew * 32 + lane;  // one column each
+      const int64_t cb = d < g.N ? r.cs_b[d] : 0;
+      asm volatile("bar.sync 1, 256;" ::: "memory");  // the last item's terms are read
+      col_i[ew * 32 + lane] = ka * cb;
+      col_f[ew * 32 + lane] = ll_to_float(cb - r.Kn * mb);
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const int64_t c = t.m0 + q * 32 + lane;
+      const int64_t ca = c < g.M ? r.cs_a[c] : 0;
+      rt = db * ll_to_float(ca - r.Kn * ma);
+      Ia = kb * ca + k0;
+    }
+    int sum[BN];
+#pragma unroll
+    for (int j = 0; j < BN; ++j) sum[j] = 0;
+    const int64_t nchunks = (t.kb1 - t.kb0 + g.kc_blocks - 1) / g.kc_blocks;
+    for (int64_t c = 0; c < nchunks; ++c, ++cc) {
+      const int b = (int)(cc & 1u), buf = 2 * b + h;
+      bool got = !dead && !*abort_flag && mbar_wait(&accf[buf], (cc >> 1) & 1u, g.status);
+      got = __all_sync(0xffffffffu, got);
+      if (!got) {
+        dead = true;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t acc = lane_base + (uint32_t)(b * 2 * BN);
+#pragma unroll
+      for (int grp = 0; grp < BN / 32; ++grp) {
+        uint32_t v[32];
+        tmem_ld32_nw(acc + (uint32_t)(grp * 32), v);
+        tmem_wait_ld(v);
+        if (grp == BN / 32 - 1) {  // the accumulator has been read in full
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) acc_release<true>(&acce[buf]);
+        }
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+          sum[grp * 32 + j] += __float2int_rn(__uint_as_float(v[j]));
+      }
+    }
+    if (dead) {
+      *abort_flag = 1;
+      continue;
+    }
+#pragma unroll
+    for (int grp = 0; grp < BN / 32; ++grp) {
+      uint32_t o[32];
+      if (g.fuse) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int col = h * BN + grp * 32 + j;
+          const int64_t I = (int64_t)sum[grp * 32 + j] + col_i[col] + Ia;
+          o[j] = __float_as_uint(sab * (ll_to_float(I) + rt + da * col_f[col] + kdd));
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) o[j] = (uint32_t)sum[grp * 32 + j];
+      }
+      if (stored) {
+        if (lane == 0) bulk_wait_read(0);
+        __syncwarp();
+      }
+#pragma unroll
+      for (int j4 = 0; j4 < 8; ++j4)
+        *reinterpret_cast<uint4 *>(box + sw128_off(lane, j4)) =
+            make_uint4(o[4 * j4], o[4 * j4 + 1], o[4 * j4 + 2], o[4 * j4 + 3]);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0 && t.m0 < g.M && t.n0 < g.N) {
+        tma_store_3d(tmOut, (int32_t)(t.n0 + grp * 32), (int32_t)(t.m0 + q * 32), t.split, box);
+        bulk_commit();
+      }
+      stored = true;
+    }
+  }
+  if (lane == 0) bulk_wait_all();
+  __syncwarp();
+}
+
 // The tiles of this CTA left raw by the fp32-form epilogue (defined with the
 // group fix-up, whose arithmetic it shares).
-template <int NB>
+template <int NB, bool PAIR>
 __device__ __noinline__ void gradx_raw_fix(const GemmArgs &g, const uint32_t *raw_mask, int ew,
                                            int nwarps, int lane, bool p_bits);
 
-template <int MODE, int NB, int FORM>
-__global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
+// PAIR: the CTAs of a cluster of two work as one tensor-core pair
+// (cta_group::2): super tiles of 256 x 256, each CTA staging its 128 rows of
+// A and its 128 columns of B per K block, so that a staged byte and a ring
+// hand-over feed twice the MMA work of a CTA on its own and the instruction
+// is 256 columns wide (1843 against 1487 TFLOP/s at 128).  The leader (rank
+// 0) issues the MMAs for both and counts both CTAs' copies; its commits
+// release the stages and hand over the accumulators in both.  Each CTA's
+// tensor memory holds two accumulators of 256 columns for its 128 rows,
+// drained as four of 128 by the same epilogue sets.
+template <int MODE, int NB, int FORM, bool PAIR = false>
+__global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB, PAIR>::threads, 1)
     k_gemm(const __grid_constant__ CUtensorMap tmA,
            const __grid_constant__ CUtensorMap tmB,
            const __grid_constant__ CUtensorMap tmOut, const GemmArgs g) {
@@ -1392,7 +1758,7 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
   // (FORM 2 runs one exact chunk per tile: never pairs)
   const bool pairs = FORM != 2 && kPerItem && g.nacc == 2;
   const int64_t gstep = (pairs ? 2 : 1) * (int64_t)gridDim.x;
-  constexpr uint32_t kEpiArrivals = kPerItem ? 4u : (uint32_t)kPartialEpiWarps;
+  constexpr uint32_t kEpiArrivals = PAIR ? 8u : kPerItem ? 4u : (uint32_t)kPartialEpiWarps;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -1418,7 +1784,14 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
   if (MODE == MODE_GRADX && NB != 0)
     for (int i = threadIdx.x; i < (int)(kRawMaskBytes / 4); i += blockDim.x)
       reinterpret_cast<uint32_t *>(smem + kOffRaw)[i] = 0u;
-  if (warp == kWarpMma) {
+  if (PAIR && warp == kWarpMma) {
+    asm volatile(
+        "tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+            smem_u32(tmem_slot)),
+        "r"(kTmemCols)
+        : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  } else if (warp == kWarpMma) {
     asm volatile(
         "tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
             smem_u32(tmem_slot)),
@@ -1428,9 +1801,10 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // the peer's barriers exist
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  using LY = GemmLayout<MODE, FORM, NB>;
+  using LY = GemmLayout<MODE, FORM, NB, PAIR>;
 
   auto fail = [&]() { *abort_flag = 1; };
 
@@ -1440,7 +1814,7 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
     if constexpr (LY::regs_epi > 0)
       asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(LY::regs_epi));
     if (MODE == MODE_GRADX) {
-      gradx_epilogue<NB, FORM>(g, smem, ring, accf, acce, pfull, pempty, tmem, &tmOut,
+      gradx_epilogue<NB, FORM, PAIR>(g, smem, ring, accf, acce, pfull, pempty, tmem, &tmOut,
                                abort_flag, warp, lane);
       if constexpr (NB != 0) {
         // every epilogue warp arrives here once; then the tiles left raw
@@ -1448,10 +1822,12 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
         // bit patterns otherwise) are finished
         asm volatile("bar.sync 1, %0;" ::"r"(32 * 4 * LY::sets) : "memory");
         if (!*abort_flag)
-          gradx_raw_fix<NB>(g, reinterpret_cast<const uint32_t *>(smem + kOffRaw),
+          gradx_raw_fix<NB, PAIR>(g, reinterpret_cast<const uint32_t *>(smem + kOffRaw),
                             warp - kGemmWarpEpi0, 4 * LY::sets, lane, FORM != 2);
       }
     }
+    else if constexpr (PAIR)
+      partial_epilogue_pair(g, smem, ring, accf, acce, tmem, &tmOut, abort_flag, warp, lane);
     else if (warp < kGemmWarpEpi0 + kPartialEpiWarps)
       partial_epilogue(g, ring, accf, acce, tmem, &tmOut, abort_flag, warp, lane);
     else if (u8ops)  // the four warps after the partial epilogue
@@ -1465,7 +1841,9 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
     if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
-      if (pairs) {
+      if constexpr (PAIR) {
+        produce_pair<MODE>(g, tmA, tmB, ops, full, empty, abort_flag, s, ph);
+      } else if (pairs) {
         bool ok = true;
         for (int64_t it = blockIdx.x; ok && it < g.n_items && !*abort_flag; it += gstep) {
           Item tt[2];
@@ -1587,7 +1965,10 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
     }
   } else if (warp == kWarpMma) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (PAIR) {
+      if (lane == 0 && (blockIdx.x & 1) == 0)
+        issue_pair(g, ops, full, empty, accf, acce, drain, tmem, abort_flag);
+    } else if (lane == 0) {
       int s = 0;
       uint32_t ph = 0;
       int buf = 0;
@@ -1679,7 +2060,7 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
       mbar_wait(drain, 0, g.status);
     }
   } else if (warp == kGemmWarpPar) {
-    if (MODE == MODE_GRADX) gradx_params<NB, FORM>(g, smem, pfull, pempty, abort_flag, lane);
+    if (MODE == MODE_GRADX) gradx_params<NB, FORM, PAIR>(g, smem, pfull, pempty, abort_flag, lane);
     else if (u8ops) partial_convert(g, ops, uops, full, empty, cvt, fempty, abort_flag, 0, lane);
   } else if (MODE == MODE_PARTIAL && u8ops && warp == kGemmWarpPar + 1) {
     partial_convert(g, ops, uops, full, empty, cvt, fempty, abort_flag, 1, lane);
@@ -1688,12 +2069,19 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB>::threads, 1)
 
   tc_fence_before();
   __syncthreads();
+  // neither CTA of a pair leaves while the other may still reach its memory
+  if constexpr (PAIR) cluster_sync();
   if (warp == kWarpMma) {
     __syncwarp();
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(kTmemCols)
-                 : "memory");
+    if constexpr (PAIR)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(kTmemCols)
+                   : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(kTmemCols)
+                   : "memory");
   }
 }
 
@@ -1865,12 +2253,15 @@ static __device__ __noinline__ void fix_group_general(const FixArgs &f, int64_t 
 // unit of the CTA's raw tiles -- each lane 4 of the tile's 128 columns --
 // with the arithmetic of fix_group_general (int64 integer parts and
 // float-float where the fp32 form is not exact).  NB = 1: one row per unit.
-template <int NB>
+template <int NB, bool PAIR>
 __device__ __noinline__ void gradx_raw_fix(const GemmArgs &g, const uint32_t *raw_mask, int ew,
                                            int nwarps, int lane, bool p_bits) {
   constexpr int NBD = NB > 1 ? NB : 1;
   constexpr int BPT = BN / NBD;  // units per tile
-  int64_t n_local = (g.n_items - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x;
+  int64_t n_local =
+      PAIR ? 2 * ((g.n_items - (int64_t)(blockIdx.x >> 1) + (gridDim.x >> 1) - 1) /
+                  (int64_t)(gridDim.x >> 1))
+           : (g.n_items - (int64_t)blockIdx.x + gridDim.x - 1) / (int64_t)gridDim.x;
   if (n_local > kMaxLocalTiles) n_local = kMaxLocalTiles;
   const int nwords = (int)((n_local + 31) / 32);
   bool any = false;
@@ -1909,7 +2300,8 @@ __device__ __noinline__ void gradx_raw_fix(const GemmArgs &g, const uint32_t *ra
     while (bits) {
       const int l = w * 32 + __ffs(bits) - 1;
       bits &= bits - 1u;
-      const Item t = decode_item(g, (int64_t)blockIdx.x + (int64_t)l * gridDim.x);
+      Item t;
+      if (!cta_item<PAIR>(g, l, t)) continue;
       for (int b = 0; b < BPT; ++b, ++u) {
         if ((int)(u % nwarps) != ew) continue;
         const int64_t k0 = t.n0 + (int64_t)b * NBD;
@@ -1933,5 +2325,11 @@ __device__ __noinline__ void gradx_raw_fix(const GemmArgs &g, const uint32_t *ra
     }
   }
 }
+
+
+typedef void (*GemmKernel)(CUtensorMap, CUtensorMap, CUtensorMap, GemmArgs);
+
+// The pair instance of a mode, block size and epilogue form (fqt_gemm_pair.cu).
+GemmKernel gemm_pair_kernel(int mode, int nb, int form);
 
 }  // namespace fqt
