@@ -1471,16 +1471,19 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
         crpb = 64 / cpw;
         cybi = (oh + crpb - 1) / crpb;
         Kt = (int64_t)g[0] * cybi * 64;
-        // the workspace holds the partials of at most 2.5 N slots (tiny
-        // images would pad far beyond)
-        if (2 * Kt > 5 * Nr) {
-          cpw = crpb = cybi = 0;
-          Kt = Nr;
-        }
       }
     }
     const bool conv_tile = cpw > 0;
     SplitPlan p = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true);
+    // the workspace holds the partials of at most 2.5 N slots: tiny images,
+    // which pad far beyond, take the splits that fit
+    if (conv_tile && 2 * Kt > 5 * Nr) {
+      const int64_t fit = plan_splits(C, D, (Nr * 5 + 1) / 2, a_bits, x_bits, nsm, true).splits;
+      if (p.splits > fit) {
+        p.ks_blocks = (p.kb_total + fit - 1) / fit;
+        p.splits = (int)((p.kb_total + p.ks_blocks - 1) / p.ks_blocks);
+      }
+    }
     const WPlan wp = Nr > 0 ? gradw_plan(Nr, C, D, a_bits, x_bits, nsm) : WPlan{};
     // k_gradw serves the implicit im2col operand with wider output rows (4-D
     // boxes of 32 pixels of one row, ow % 32 == 0); plain matrices take the
