@@ -136,10 +136,16 @@ static fqt_status quantize_conv(const void *X, fqt_dtype dtype, int64_t n, int64
   if (e != cudaSuccess) return cuda_fail(e, "range pass");
   // code(0.0), the padding's code, follows the column sums (device memory)
   int32_t *zc = out->col_sum + (int64_t)kh * kw * c;
+  // 3 x 3, pad 1: the code pass sums the totals (the centre tap's column sums)
+  // and a pass over the border lines makes the other taps of them
+  const bool lines = conv_lines_supported((int)h, (int)wd, (int)c, kh, kw, pad);
   s = launch_fwd_codes(X, dtype == FQT_BF16, pixels, (int)c, bits, out->codes_f16, out->codes,
-                       nullptr, part, npart, out->inv_s, out->zero, reinterpret_cast<int *>(w),
+                       lines ? out->col_sum + 4 * c : nullptr, part, npart, out->inv_s, out->zero, reinterpret_cast<int *>(w),
                        nsm, st, pad > 0 ? 1 : 0, zc);
   if (s != FQT_OK) return s;
+  if (lines)
+    return launch_conv_lines(out->codes_f16, n, (int)h, (int)wd, (int)c, nullptr, out->col_sum,
+                             1 << (bits - 1), st);
   return launch_conv_colsum(out->codes_f16, n, (int)h, (int)wd, (int)c, kh, kw, pad, bits,
                             out->col_sum, st);
 }

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const ReduceArgs r) {
       const int64_t d = d0 + i;
       const int64_t cb = r.cs_b[d];
       long long Pi = P[i];
-      if (r.pad_a) Pi += code_pad * r.pad_a[c * r.taps + d / r.cin];
+      if (r.pad_a) Pi += code_pad * r.pad_a[d / r.cin * r.M + c];
       const int64_t I = Pi + ka * cb + Ia;
       o[i] = sab * (ll_to_float(I) + rt + da * ll_to_float(cb - r.Kn * mb) + kdd);
     }
@@ -249,6 +249,8 @@ static bool pair_faster(const SplitPlan &p, const SplitPlan &q, int num_sms) {
   const int64_t one = ((int64_t)p.m_tiles * p.n_tiles * p.splits + num_sms - 1) / num_sms;
   const int64_t two =
       ((int64_t)q.m_tiles * q.n_tiles * q.splits + num_sms / 2 - 1) / (num_sms / 2);
+  // short splits: the partials and their reduction outweigh the contraction
+  if (q.splits > 1 && q.ks_blocks < 16) return false;
   return q.kb_total >= 4 && 10 * two * (q.ks_blocks + 3) < 9 * one * (p.ks_blocks + 3);
 }
 
@@ -995,7 +997,7 @@ __global__ void __launch_bounds__(256) k_conv_padsum(const uint16_t *__restrict_
         if (row_out || col_out) v += cls_s[(ry * cc + rx) * ch_group + ch];
       }
     }
-    if (v) atomicAdd(&pad_a[(int64_t)(ch0 + ch) * taps + tap], v);
+    if (v) atomicAdd(&pad_a[(int64_t)tap * C + ch0 + ch], v);
   }
 }
 
@@ -1516,7 +1518,11 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
       cudaError_t e = cudaMemsetAsync(pad_a, 0, (size_t)C * taps * 4, st);
       if (e != cudaSuccess) return cuda_fail(e, "padding sums clear");
       const int grp = padsum_group((int)C, g[6]);
-      if (g[6] > 0) {  // without padding no tap reads any
+      if (conv_lines_supported(oh, ow, (int)C, g[4], g[5], g[6])) {
+        const fqt_status ls = launch_conv_lines(static_cast<const uint16_t *>(A16), g[0], oh, ow,
+                                                (int)C, pad_a, nullptr, 0, st);
+        if (ls != FQT_OK) return ls;
+      } else if (g[6] > 0) {  // without padding no tap reads any
         // about 16 loads per thread: runs of images whose border pixels
         // (bounded by the pad rows and columns) fill a CTA
         const int pd = g[6];

@@ -105,8 +105,8 @@ struct ReduceArgs {
   int64_t Kn;        // rows N of dH / X
   int oa, ob;
   // an implicit im2col X~: its padding entered the product as code 2^(bx-1);
-  // P += (code(0) - ob) pad_a[c][tap(d)], pad_a = the A carriers summed over
-  // the rows whose tap reads padding (C x taps), tap(d) = d / cin
+  // P += (code(0) - ob) pad_a[tap(d)][c], pad_a = the A carriers summed over
+  // the rows whose tap reads padding (taps x C), tap(d) = d / cin
   const int32_t *pad_a, *code_zero;
   int taps, cin;
   const int32_t *cs_a, *cs_b;  // column sums of Q_b1 codes (M) and X~ codes (N)

@@ -69,6 +69,10 @@ fqt_status launch_fwd_codes(const void *X, bool bf16, int64_t rows, int cols, in
                             int32_t *code_zero_out = nullptr);
 fqt_status launch_conv_colsum(const uint16_t *f16, int64_t n, int h, int w, int c, int kh,
                               int kw, int pad, int bits, int32_t *col_sum, cudaStream_t st);
+// border sums of 3 x 3, pad 1 conv operands (fqt_conv.cu)
+bool conv_lines_supported(int h, int w, int C, int kh, int kw, int pad);
+fqt_status launch_conv_lines(const uint16_t *f16, int64_t n, int h, int w, int C, int32_t *pad_a,
+                             int32_t *col_sum, int centre, cudaStream_t st);
 bool bhq_pass_supported(int C, int block, bool bf16);
 size_t bhq_pass_bytes(int64_t N, int64_t C);
 fqt_status launch_bhq_passes(QuantArgs &a, bool bf16, int num_sms, void *scratch,
