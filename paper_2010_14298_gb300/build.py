@@ -18,7 +18,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libfqt.so")
-SOURCES = ["fqt_quant.cu", "fqt_group.cu", "fqt_gemm.cu", "fqt_gemm_pair.cu", "fqt_conv.cu",
+SOURCES = ["fqt_quant.cu", "fqt_codes.cu", "fqt_group.cu", "fqt_gemm.cu", "fqt_gemm_pair.cu", "fqt_conv.cu",
            "fqt_api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",

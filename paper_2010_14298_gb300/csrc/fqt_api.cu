@@ -318,11 +318,21 @@ fqt_status fqt_quantize_grad(const void *dH, fqt_dtype dtype, int64_t N,
   if (adapt && N > ((int64_t)1 << 20)) return FQT_EUNSUPPORTED;
   // fixed BHQ blocks of supported shapes: the two-pass quantizer, whose
   // statistics pass also takes the range (no separate range pass)
-  const bool two_pass = kind == FQT_BHQ && !adapt &&
-                        bhq_pass_supported((int)C, block, dtype == FQT_BF16);
+  // (PSQ: the row statistics).  Their scratch is part of fqt_workspace_size; a
+  // smaller workspace takes the one-pass quantizers.
+  const size_t pass_bytes = kind == FQT_BHQ   ? bhq_pass_bytes(N, C)
+                            : kind == FQT_PSQ ? sample_pass_bytes(N, C, 1)
+                                              : 0;
+  const bool two_pass = ws_bytes >= kGemmOffset + pass_bytes &&
+                        ((kind == FQT_BHQ && !adapt && bhq_pass_supported((int)C, block)) ||
+                         (kind == FQT_PSQ && psq_pass_supported((int)C)));
+  // (the BHQ widths and blocks that have always needed it refuse it instead)
+  const bool bhq_need = kind == FQT_BHQ && !adapt && C >= 64 && C <= 4096 && !(C & (C - 1)) &&
+                        (block == 16 || (dtype == FQT_F32 && (block == 4 || block == 8)));
   fqt_status s = check_ws(workspace, ws_bytes,
-                          kGemmOffset + (adapt ? group_workspace_bytes(N)
-                                         : two_pass ? bhq_pass_bytes(N, C) : 0));
+                          kGemmOffset + (adapt      ? group_workspace_bytes(N)
+                                         : bhq_need ? bhq_pass_bytes(N, C)
+                                                    : 0));
   if (s != FQT_OK) return s;
   q_b2->rows = N;
   q_b2->cols = C;
@@ -348,9 +358,27 @@ fqt_status fqt_quantize_grad(const void *dH, fqt_dtype dtype, int64_t N,
   // the column sums the quantizer accumulates into are cleared by the range pass
   int32_t *csum2 = kind == FQT_SHIFT ? q_b2->shift_col_sum : nullptr;
   cudaError_t e = cudaSuccess;
+  // PTQ: the code pass adds the row sums of rows split over warps
+  const bool ptq = kind == FQT_PTQ && ptq_pass_supported((int)C);
+  QuantArgs plan;
+  memset(&plan, 0, sizeof(plan));
+  plan.N = N;
+  plan.C = (int)C;
+  int64_t nz2 = csum2 ? C : 0;
+  if (ptq) {
+    ptq_pass_plan(plan, nsm);
+    if (plan.code_split > 1) {
+      csum2 = q_b2->row_sum;
+      nz2 = csum2 ? N : 0;
+      if (q_b1 && q_b1->row_sum) {
+        e = cudaMemsetAsync(q_b1->row_sum, 0, (size_t)N * 4, st);
+        if (e != cudaSuccess) return cuda_fail(e, "row sums clear");
+      }
+    }
+  }
   if (!two_pass) {
     e = launch_range(dH, dtype == FQT_BF16, N * C, part, &npart, csum, csum ? C : 0, csum2,
-                     csum2 ? C : 0, nsm, st);
+                     nz2, nsm, st);
     if (e != cudaSuccess) return cuda_fail(e, "range pass");
   }
   QuantArgs a;
@@ -412,6 +440,9 @@ fqt_status fqt_quantize_grad(const void *dH, fqt_dtype dtype, int64_t N,
     }
     return launch_bhq_groups(ag, bf16, nsm, st);
   }
+  if (ptq) return launch_ptq_codes(a, bf16, nsm, st);
+  if (two_pass && kind == FQT_PSQ)
+    return launch_sample_passes(a, bf16, 1, nsm, w + kGemmOffset, part, st);
   if (two_pass) {
     QuantArgs aw = a;
     if (want_off) {

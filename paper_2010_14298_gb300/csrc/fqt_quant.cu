@@ -879,28 +879,6 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// BHQ gradient quantizer for fixed blocks (Sec. 4.2, App. D.4) fused with
-// Q_b1 (App. E), in two passes over dH.  The statistics pass holds each
-// block in registers: a team of TEAM warps per block of nb rows, each warp
-// owning a slab of 8 LPR columns (TEAM > 1 only with LPR = 32, slabs of 256
-// columns), lane l owning oct l % LPR of the slab in row l / LPR of each of
-// the STEPS row groups (nb = (32 / LPR) STEPS); row reductions are shuffles
-// inside a warp and one shared-memory exchange at a named barrier of the
-// team.  Its per-entry work is light (statistics, column sums, row minima),
-// so the unrolled block fits the instruction cache.  The code pass streams
-// the rows with rolled loops (rounding, packing, sums need no block-wide
-// exchange once z'_k and w_j are known); k_bhq_offsets then reflects the
-// grad_X offsets hz, hr of each block.
-//
-// Stochastic rounding runs on the fp32 pipe: with U = 128 + u 2^-16 (u the
-// 16-bit uniform, exact in fp32), floor(v + u 2^-16) = floor(rd(v + U)) - 128
-// because rounding down never crosses an integer, and a second round-down
-// addition of 2^23 + 0x6400 - 128 leaves 0x4B006400 + code in the bits:
-// code = floor(v + u 2^-16) = (floor(v 2^16) + u) >> 16, the rule of sr_code16
-// (R1) for v in [0, B].  Byte 0 of those bits is the code and byte 1 is 0x64,
-// so one byte permutation packs two fp16 carriers 1024 + code.
-// ---------------------------------------------------------------------------
 template <int FROM, class V, class Op>
 __device__ __forceinline__ V xor_reduce(V v, Op op) {
 #pragma unroll
@@ -914,899 +892,6 @@ __device__ __forceinline__ V row_reduce(V v, Op op) {
 #pragma unroll
   for (int off = LPR >> 1; off > 0; off >>= 1) v = op(v, shfl_x(v, off));
   return v;
-}
-
-constexpr float kSrMagic = 8414080.0f;     // 2^23 + 0x6400 - 128
-constexpr uint32_t kSrBits = 0x4B006400u;  // bits of 2^23 + 0x6400
-
-// 128 + u 2^-16 for the low and the high 16-bit uniform of a Philox word
-__device__ __forceinline__ float sr_u_lo(uint32_t w) {
-  return __uint_as_float(0x43000000u | (w & 0xFFFFu));
-}
-__device__ __forceinline__ float sr_u_hi(uint32_t w) {
-  return __uint_as_float(__byte_perm(w, 0x43000000u, 0x7632));
-}
-// uniform j (0..7) of an oct: half (j mod 2) of word j / 2
-__device__ __forceinline__ float sr_u(const uint4 &w, int j) {
-  const uint32_t word = (j >> 1) == 0 ? w.x : (j >> 1) == 1 ? w.y : (j >> 1) == 2 ? w.z : w.w;
-  return (j & 1) ? sr_u_hi(word) : sr_u_lo(word);
-}
-
-// kSrBits + code, code = SR(v) for v in [0, B] (v already clamped)
-__device__ __forceinline__ uint32_t sr_bits(float v, float U) {
-  return __float_as_uint(__fadd_rd(__fadd_rd(v, U), kSrMagic));
-}
-
-// Eight codes (kSrBits + code) as centred fp16 carriers code - off.
-__device__ __forceinline__ void store_carriers_bits(uint16_t *dst, const uint32_t (&b)[8],
-                                                    __half2 bias) {
-  uint32_t w[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t h = __byte_perm(b[2 * i], b[2 * i + 1], 0x5410);
-    __half2 v = __hsub2(*reinterpret_cast<const __half2 *>(&h), bias);
-    w[i] = *reinterpret_cast<uint32_t *>(&v);
-  }
-  *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-// Eight codes (kSrBits + code) as bytes.
-__device__ __forceinline__ void store_codes_bits(uint8_t *dst, const uint32_t (&b)[8]) {
-  uint2 v;
-  v.x = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
-  v.y = __byte_perm(__byte_perm(b[4], b[5], 0x0040), __byte_perm(b[6], b[7], 0x0040), 0x5410);
-  *reinterpret_cast<uint2 *>(dst) = v;
-}
-
-// Named barrier of one team of TEAM warps (ids 1..8; 0 is __syncthreads).
-template <int TEAM>
-__device__ __forceinline__ void team_sync(int team) {
-  if constexpr (TEAM > 1)
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(32 * TEAM) : "memory");
-}
-
-constexpr int kTeamRows = 16;  // rows of a block when TEAM > 1 (LPR = 32, STEPS <= 16)
-
-// Per-block results of the statistics pass, read by the code pass: lead row
-// p (as an integer bit pattern), s1, s2 and rho = 1/sqrt(nb) (0 for a block
-// of one row or of zeros), followed in the workspace by w_j for every block.
-struct BhqBlock {
-  float p, s1, s2, rho;
-};
-
-// Workspace bytes of the two-pass BHQ quantizer for blocks of at least 4
-// rows: the per-block record and the C column sums w of every block.
-size_t bhq_pass_bytes(int64_t N, int64_t C) {
-  const int64_t nblk = (N + 3) / 4;
-  return (size_t)nblk * sizeof(BhqBlock) + (size_t)nblk * (size_t)C * sizeof(float) + 512;
-}
-
-// ---------------------------------------------------------------------------
-// Statistics pass of BHQ (the first of the two passes over dH): for every
-// block its row statistics, lead row, lambda1, lambda2, s1, s2 (App. D.4),
-// the reflection's column sums w_j = sum_k e_k s_k h_kj and the row minima
-// z'_k of T = Q diag(s) H (Sec. 4.2), plus the per-CTA (min, max) and
-// non-finite flag of the whole tensor (the range of Q_b1) and the clearing of
-// the column sums the code pass accumulates into.
-// ---------------------------------------------------------------------------
-template <typename T, int LPR, int STEPS, int TEAM, int H>
-__global__ void __launch_bounds__(256, (STEPS >= 8 ? 1 : 2))
-    k_bhq_stats(const QuantArgs a, BhqBlock *__restrict__ bst, float *__restrict__ wsum,
-                float2 *__restrict__ part) {
-  static_assert(TEAM == 1 || (LPR == 32 && STEPS <= kTeamRows), "team layout");
-  static_assert(H == 1 || TEAM == 8, "column halves only for a full team");
-  // H column parts of SLAB * TEAM columns each: a part is read, reduced and
-  // read again (from L2) after the block's scalars are known
-  constexpr int RS = 32 / LPR, SLAB = 8 * LPR, C = SLAB * TEAM * H;
-  constexpr int TPC = 8 / TEAM;  // teams per CTA
-  constexpr int XW = TEAM > 1 ? 8 : 1;
-  __shared__ float2 xs_mm[XW][kTeamRows];
-  __shared__ float xs_tm[XW][kTeamRows];
-  __shared__ float2 red[8];
-  __shared__ int redi[8];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int team = warp / TEAM, wi = warp - team * TEAM;
-  const int nb = a.block;
-  const int sub = lane / LPR, o = lane - sub * LPR;
-  auto col_of = [&](int h) { return ((h * TEAM + wi) * LPR + o) * 8; };
-  const float fB2 = (float)((1u << a.bits) - 1u);
-  // the code pass accumulates column sums (and, split, row sums) into these
-  {
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + tid;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = g; i < C; i += stride) {
-      if (a.csum1) a.csum1[i] = 0;
-      if (a.csum2) a.csum2[i] = 0;
-    }
-    if (a.code_split > 1)
-      for (int64_t i = g; i < a.N; i += stride) {
-        if (a.rsum1) a.rsum1[i] = 0;
-        if (a.rsum2) a.rsum2[i] = 0;
-      }
-  }
-  float gmn = INFINITY, gmx = -INFINITY, nanacc = 0.0f;
-  const int64_t nblocks = (a.N + nb - 1) / nb;
-  const int64_t tstride = (int64_t)gridDim.x * TPC;
-  for (int64_t blk = (int64_t)blockIdx.x * TPC + team; blk < nblocks; blk += tstride) {
-    const int64_t r0 = blk * nb;
-    const int nrows = (int)min((int64_t)nb, a.N - r0);
-    float x[STEPS][8];
-    bool rv[STEPS];
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s) rv[s] = sub + RS * s < nrows;
-    auto load_part = [&](int h) {
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        const int k = sub + RS * s;
-        if (rv[s]) {
-          load_oct(reinterpret_cast<const T *>(a.h) + (r0 + k) * C + col_of(h), x[s]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) x[s][j] = 0.0f;
-        }
-      }
-    };
-    // ---- row statistics (and a NaN that any non-finite entry leaves) ----
-    float rmin[STEPS], rmax[STEPS];
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s) {
-      rmin[s] = INFINITY;
-      rmax[s] = -INFINITY;
-    }
-#pragma unroll 1
-    for (int h = 0; h < H; ++h) {
-      load_part(h);
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        float2 mm = make_float2(INFINITY, -INFINITY);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          mm.x = fminf(mm.x, x[s][j]);
-          mm.y = fmaxf(mm.y, x[s][j]);
-          nanacc = fmaf(x[s][j], 0.0f, nanacc);
-        }
-        mm = row_reduce<LPR>(mm, OpMinMax());
-        rmin[s] = fminf(rmin[s], mm.x);
-        rmax[s] = fmaxf(rmax[s], mm.y);
-      }
-    }
-    if constexpr (TEAM > 1) {
-      if (lane == 0) {
-#pragma unroll
-        for (int s = 0; s < STEPS; ++s) xs_mm[warp][s] = make_float2(rmin[s], rmax[s]);
-      }
-      team_sync<TEAM>(team);
-      float2 mine = make_float2(INFINITY, -INFINITY);
-      if (lane < STEPS) {
-#pragma unroll
-        for (int w2 = 0; w2 < TEAM; ++w2) mine = OpMinMax()(mine, xs_mm[team * TEAM + w2][lane]);
-      }
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        rmin[s] = __shfl_sync(0xffffffffu, mine.x, s);
-        rmax[s] = __shfl_sync(0xffffffffu, mine.y, s);
-      }
-    }
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s)
-      if (rv[s]) {
-        gmn = fminf(gmn, rmin[s]);
-        gmx = fmaxf(gmx, rmax[s]);
-      }
-    // ---- lead row (largest ||h_k||_inf, lowest index on ties), lambda2 ----
-    float bestv = -1.0f;
-    int bestk = 0x7fffffff;
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s) {
-      const int k = sub + RS * s;
-      const float nk = fmaxf(fabsf(rmin[s]), fabsf(rmax[s]));
-      if (rv[s] && (nk > bestv || (nk == bestv && k < bestk))) {
-        bestv = nk;
-        bestk = k;
-      }
-    }
-#pragma unroll
-    for (int off = LPR; off < 32; off <<= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bestv, off);
-      const int ok = __shfl_xor_sync(0xffffffffu, bestk, off);
-      if (ov > bestv || (ov == bestv && ok < bestk)) {
-        bestv = ov;
-        bestk = ok;
-      }
-    }
-    const int p = bestk < nrows ? bestk : 0;
-    const float np = bestv;
-    float l2 = 0.0f;
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s) {
-      const int k = sub + RS * s;
-      if (rv[s] && k != p) l2 = fmaxf(l2, fmaxf(fabsf(rmin[s]), fabsf(rmax[s])));
-    }
-    l2 = xor_reduce<LPR>(l2, OpMaxF());
-    const float lam2 = 2.0f * l2;
-    // range of the lead row, from the lanes that own it
-    float pmin = 0.0f, pmax = 0.0f;
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s)
-      if (s == p / RS) {
-        pmin = rmin[s];
-        pmax = rmax[s];
-      }
-    pmin = __shfl_sync(0xffffffffu, pmin, (p % RS) * LPR);
-    pmax = __shfl_sync(0xffffffffu, pmax, (p % RS) * LPR);
-    // ---- block scalars s1, s2 (App. D.4) and the reflection ----
-    float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
-    if (np > 0.0f) {
-      float lam1 = __fsub_rn(pmax, pmin);
-      if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
-      const float Nf = (float)nrows;
-      if (lam2 > 0.0f) {
-        const float c1 = cbrtf(lam1), c2 = cbrtf(lam2);
-        const float n3 = cbrtf(Nf), n6 = sqrtf(n3);
-        const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
-        s1f = fB2 * n6 / (c1 * den);
-        s2f = fB2 * n6 / (c2 * den);
-      } else {
-        s1f = fB2 * sqrtf(Nf) / lam1;
-      }
-      if (nrows > 1) {
-        rho = 1.0f / sqrtf(Nf);
-        kap = 1.0f / (1.0f - rho);
-      }
-    }
-    float tmin[STEPS];
-#pragma unroll
-    for (int s = 0; s < STEPS; ++s) tmin[s] = INFINITY;
-    // the last part read is still in registers; the others are read again
-#pragma unroll 1
-    for (int h = H - 1; h >= 0; --h) {
-      if (h != H - 1) load_part(h);
-      // w_j = sum_k e_k s_k h_kj over the block (lane: its 8 columns)
-      float w[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) w[j] = 0.0f;
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        const bool lead = (sub + RS * s) == p;
-        const float esk = __fmul_rn(kap * (lead ? rho - 1.0f : rho), lead ? s1f : s2f);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) w[j] = fmaf(esk, x[s][j], w[j]);
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) w[j] = xor_reduce<LPR>(w[j], OpAddF());
-      // ---- row minima of T; the code pass recomputes each t_kj with this
-      // same sequence of roundings, so z'_k is exactly its row minimum ----
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        const bool lead = (sub + RS * s) == p;
-        const float sk = lead ? s1f : s2f;
-        const float ck = lead ? rho - 1.0f : rho;
-        float tm = INFINITY;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) tm = fminf(tm, fmaf(-ck, w[j], __fmul_rn(sk, x[s][j])));
-        tmin[s] = fminf(tmin[s], row_reduce<LPR>(tm, OpMin()));
-      }
-      if (sub == 0) {
-        float *wd = wsum + blk * (int64_t)C + col_of(h);
-        *reinterpret_cast<float4 *>(wd) = make_float4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<float4 *>(wd + 4) = make_float4(w[4], w[5], w[6], w[7]);
-      }
-    }
-    if constexpr (TEAM > 1) {
-      if (lane == 0) {
-#pragma unroll
-        for (int s = 0; s < STEPS; ++s) xs_tm[warp][s] = tmin[s];
-      }
-      team_sync<TEAM>(team);
-      float mine = INFINITY;
-      if (lane < STEPS) {
-#pragma unroll
-        for (int w2 = 0; w2 < TEAM; ++w2) mine = fminf(mine, xs_tm[team * TEAM + w2][lane]);
-      }
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) tmin[s] = __shfl_sync(0xffffffffu, mine, s);
-    }
-    // ---- outputs ----
-    if (wi == 0 && o == 0) {
-#pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        const int k = sub + RS * s;
-        if (!rv[s]) continue;
-        const float sk = k == p ? s1f : s2f;
-        a.inv2[r0 + k] = sk > 0.0f ? __fdiv_rn(1.0f, sk) : 0.0f;
-        a.zero2[r0 + k] = tmin[s];
-      }
-      if (sub == 0) {
-        bst[blk] = BhqBlock{__int_as_float(p), s1f, s2f, rho};
-        a.lead2[blk] = p;
-      }
-    }
-  }
-  // ---- range partials of the CTA (NaN marks a non-finite input) ----
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    gmn = fminf(gmn, __shfl_xor_sync(0xffffffffu, gmn, off));
-    gmx = fmaxf(gmx, __shfl_xor_sync(0xffffffffu, gmx, off));
-    nanacc += __shfl_xor_sync(0xffffffffu, nanacc, off);
-  }
-  if (lane == 0) {
-    red[warp] = make_float2(gmn, gmx);
-    redi[warp] = isnan(nanacc) ? 1 : 0;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    int bad = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-      gmn = fminf(gmn, red[i].x);
-      gmx = fmaxf(gmx, red[i].y);
-      bad |= redi[i];
-    }
-    part[blockIdx.x] = bad ? make_float2(NAN, NAN) : make_float2(gmn, gmx);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Code pass of BHQ (the second pass over dH), fused with Q_b1 (App. E): per
-// entry t = s_k h_kj - c_k w_j (c_k = rho - 1 on the lead row, rho
-// elsewhere) as the statistics pass computed it, v = t - z'_k, stochastic
-// rounding of v (Q_b2) and of s (h - min H) (Q_b1), fp16 carriers (and
-// optional bytes), row sums of Q_b2 and column sums of the grad_W code set.
-// A lane owns two octs of a row, o and o + LPR of a slab of 16 LPR columns
-// (one coalesced 16 LPR x 4-byte access per oct); a warp takes units of
-// kCodeRows rows and 1 / code_split of the row's slabs, walks those slabs one
-// after another and, inside a slab, the unit's rows 32 / LPR at a time,
-// issuing the loads of its next row before it rounds the current one.  A
-// block's w_j and scalars stay in registers while the lane's rows belong to
-// it.  Loops stay rolled; a row's parts meet only in its row sums (atomic
-// when code_split > 1, so that wide rows of few chunks still fill the GPU).
-// ---------------------------------------------------------------------------
-constexpr int kCodeRows = 32;
-
-template <typename T>
-__device__ __forceinline__ void load_two_octs(const T *row, int c_a, int c_b, float (&x)[16]) {
-  float lo[8], hi[8];
-  load_oct(row + c_a, lo);
-  load_oct(row + c_b, hi);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    x[j] = lo[j];
-    x[8 + j] = hi[j];
-  }
-}
-
-// SAMPLES: the per-sample PSQ of fqt_quantize_grad_samples instead of BHQ:
-// v = s_i (h - z_i) with the scalars of sample i = row / rows_per_sample
-// (srec: s, z, inv_s, zero per sample), written per row as well.
-template <typename T, int LPR, bool SAMPLES = false>
-__global__ void __launch_bounds__(256, 2) k_bhq_codes(const QuantArgs a,
-                                                   const BhqBlock *__restrict__ bst,
-                                                   const float *__restrict__ wsum, int lg_nb,
-                                                   const float4 *__restrict__ srec = nullptr,
-                                                   int rows_per_sample = 1) {
-  constexpr int RS = 32 / LPR, SLAB = 16 * LPR;
-  __shared__ float2 red[8];
-  __shared__ int redi[8];
-  __shared__ int rs_s[8][2][kCodeRows];
-  extern __shared__ int csum_s[];  // C column sums of the grad_W code set
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int C = a.C, CO = C / 8;
-  const int sub = lane / LPR, o = lane - sub * LPR;
-
-  // ---- global range (Q_b1 scale) from the statistics-pass partials ----
-  float gmin = INFINITY, gmax = -INFINITY;
-  int bad = 0;
-  for (int i = tid; i < a.npart; i += blockDim.x) {
-    const float2 p = a.part[i];
-    bad |= isnan(p.x);
-    gmin = fminf(gmin, p.x);
-    gmax = fmaxf(gmax, p.y);
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    gmin = fminf(gmin, __shfl_xor_sync(0xffffffffu, gmin, off));
-    gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, off));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, off);
-  }
-  if (lane == 0) {
-    red[warp] = make_float2(gmin, gmax);
-    redi[warp] = bad;
-  }
-  for (int i = tid; i < C; i += blockDim.x) csum_s[i] = 0;
-  __syncthreads();
-  gmin = red[0].x;
-  gmax = red[0].y;
-  bad = redi[0];
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-    gmin = fminf(gmin, red[w].x);
-    gmax = fmaxf(gmax, red[w].y);
-    bad |= redi[w];
-  }
-  if (bad) {
-    if (blockIdx.x == 0 && tid == 0) record_status(a.status, FQT_ENONFINITE);
-    return;
-  }
-  const uint32_t B2 = (1u << a.bits) - 1u;
-  const float fB2 = (float)B2;
-  const float s_g1 = affine_scale(gmin, gmax, 255u);
-  const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
-  if (blockIdx.x == 0 && tid == 0 && has_b1) {
-    a.inv1[0] = __fdiv_rn(1.0f, s_g1);
-    a.zero1[0] = __fmul_rn(s_g1, gmin);
-  }
-  int32_t *const csum_g = has_b1 ? a.csum1 : a.csum2;
-  PhiloxKeys key;
-#pragma unroll
-  for (int i = 0; i < 20; ++i) key.k[i] = a.round_keys[i];
-  const __half2 bias2 = __half2half2(__int2half_rn(1024 + (int)((B2 + 1u) >> 1)));
-  const __half2 bias1 = __half2half2(__int2half_rn(1024 + 128));
-  const bool want_rs1 = has_b1 && a.rsum1 != nullptr;
-  const T *const h = reinterpret_cast<const T *>(a.h);
-  const int nbm = (1 << lg_nb) - 1;
-
-  const int64_t nchunks = (a.N + kCodeRows - 1) / kCodeRows;
-  // code_split: a power of two dividing C / SLAB
-  const int lg_split = a.code_split > 1 ? __ffs(a.code_split) - 1 : 0;
-  const int split = 1 << lg_split;
-  const int part_cols = C >> lg_split;
-  const int64_t nunits = nchunks << lg_split;
-  const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t u = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; u < nunits;
-       u += wstride) {
-    const int64_t ch = u >> lg_split;
-    const int cpart = (int)u & (split - 1);
-    const int64_t row0 = ch * kCodeRows;
-    const int rows = (int)min((int64_t)kCodeRows, a.N - row0);
-    rs_s[warp][0][lane] = 0;
-    rs_s[warp][1][lane] = 0;
-    __syncwarp();
-#pragma unroll 1
-    for (int c0 = cpart * part_cols; c0 < (cpart + 1) * part_cols; c0 += SLAB) {
-      const int ca = c0 + o * 8, cb = ca + 8 * LPR;  // this lane's two octs
-      uint32_t cs[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) cs[j] = 0u;
-      uint32_t cs_rows = 0;
-      int64_t cur_blk = -1;
-      float w[16];
-      float sk_l = 0.0f, sk_o = 0.0f, ck_l = 0.0f, ck_o = 0.0f;
-      int p_lead = -1;
-      // the first row's loads; every later row's are issued one row ahead
-      float xn[16];
-      float zn = 0.0f;
-      {
-        const int rr = sub;
-        if (rr < rows) {
-          load_two_octs(h + (row0 + rr) * C, ca, cb, xn);
-          if (!SAMPLES) zn = a.zero2[row0 + rr];
-        }
-      }
-#pragma unroll 1
-      for (int rb = 0; rb < rows; rb += RS) {  // the same trip count in every lane
-        const int rr = rb + sub;
-        const bool valid = rr < rows;  // the LPR lanes of a row agree
-        float x[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) x[j] = xn[j];
-        const float zr = zn;
-        if (rr + RS < rows) {
-          load_two_octs(h + (row0 + rr + RS) * C, ca, cb, xn);
-          if (!SAMPLES) zn = a.zero2[row0 + rr + RS];
-        }
-        uint32_t acc1 = 0u, acc2 = 0u;
-        if (valid) {
-          const int64_t row = row0 + rr;
-          const int64_t blk = SAMPLES ? row / rows_per_sample : row >> lg_nb;
-          if (blk != cur_blk) {  // a new block (sample): its w_j and scalars
-            if constexpr (SAMPLES) {
-              const float4 sr = srec[blk];  // s, z, inv_s, zero of the sample
-              sk_l = sr.x;
-              ck_l = sr.y;
-              sk_o = sr.z;
-              ck_o = sr.w;
-            } else {
-              const BhqBlock bs = bst[blk];
-              p_lead = __float_as_int(bs.p);
-              sk_l = bs.s1;
-              sk_o = bs.s2;
-              ck_l = bs.rho - 1.0f;
-              ck_o = bs.rho;
-              load_two_octs(wsum + blk * (int64_t)C, ca, cb, w);
-            }
-            cur_blk = blk;
-          }
-          if (SAMPLES && o == 0 && c0 == 0) {
-            a.inv2[row] = sk_o;
-            a.zero2[row] = ck_o;
-          }
-          const bool lead = (int)(row & nbm) == p_lead;
-          const float sk = lead ? sk_l : sk_o;
-          const float ck = lead ? ck_l : ck_o;
-          const uint64_t qa = (uint64_t)row * (uint64_t)CO + (uint64_t)(ca >> 3);
-          const uint64_t qb = qa + (uint64_t)LPR;
-          if (has_b1) {
-            const uint4 ua = philox_oct(qa, 1u, key), ub = philox_oct(qb, 1u, key);
-            uint32_t b[16];
-            acc1 = 0u - 16u * kSrBits;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float v = fminf(__fmul_rn(__fsub_rn(x[j], gmin), s_g1), 255.0f);
-              b[j] = sr_bits(v, sr_u(j < 8 ? ua : ub, j & 7));
-              cs[j] += b[j];
-              acc1 += b[j];
-            }
-            ++cs_rows;
-            uint32_t (&b0)[8] = *reinterpret_cast<uint32_t(*)[8]>(&b[0]);
-            uint32_t (&b1)[8] = *reinterpret_cast<uint32_t(*)[8]>(&b[8]);
-            if (a.c1) {
-              store_codes_bits(a.c1 + row * (int64_t)C + ca, b0);
-              store_codes_bits(a.c1 + row * (int64_t)C + cb, b1);
-            }
-            if (a.f1) {
-              store_carriers_bits(a.f1 + row * (int64_t)C + ca, b0, bias1);
-              store_carriers_bits(a.f1 + row * (int64_t)C + cb, b1, bias1);
-            }
-          }
-          const uint4 ua = philox_oct(qa, 0u, key), ub = philox_oct(qb, 0u, key);
-          uint32_t b[16];
-          acc2 = 0u - 16u * kSrBits;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            // BHQ: t - z'; per-sample PSQ: s (h - z) with the sample's s, z (Sec. 4.1)
-            const float v = SAMPLES ? __fmul_rn(__fsub_rn(x[j], ck_l), sk_l)
-                                    : __fsub_rn(fmaf(-ck, w[j], __fmul_rn(sk, x[j])), zr);
-            b[j] = sr_bits(fminf(v, fB2), sr_u(j < 8 ? ua : ub, j & 7));
-            acc2 += b[j];
-            if (!has_b1) cs[j] += b[j];
-          }
-          if (!has_b1) ++cs_rows;
-          uint32_t (&b0)[8] = *reinterpret_cast<uint32_t(*)[8]>(&b[0]);
-          uint32_t (&b1)[8] = *reinterpret_cast<uint32_t(*)[8]>(&b[8]);
-          if (a.c2) {
-            store_codes_bits(a.c2 + row * (int64_t)C + ca, b0);
-            store_codes_bits(a.c2 + row * (int64_t)C + cb, b1);
-          }
-          if (a.f2) {
-            store_carriers_bits(a.f2 + row * (int64_t)C + ca, b0, bias2);
-            store_carriers_bits(a.f2 + row * (int64_t)C + cb, b1, bias2);
-          }
-        }
-        if (want_rs1) {
-          const int r1 = row_reduce<LPR>((int)acc1, OpAdd());
-          if (o == 0 && valid) rs_s[warp][1][rr] += r1;
-        }
-        const int r2 = row_reduce<LPR>((int)acc2, OpAdd());
-        if (o == 0 && valid) rs_s[warp][0][rr] += r2;
-      }
-      // this slab's column sums: the lanes of one column add theirs
-      if (csum_g) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int v = xor_reduce<LPR>((int)(cs[j] - cs_rows * kSrBits), OpAdd());
-          if (sub == 0 && v) atomicAdd(&csum_s[(j < 8 ? ca : cb) + (j & 7)], v);
-        }
-      }
-    }
-    __syncwarp();
-    if (lane < rows) {
-      if (split > 1) {
-        if (a.rsum2) atomicAdd(&a.rsum2[row0 + lane], rs_s[warp][0][lane]);
-        if (want_rs1) atomicAdd(&a.rsum1[row0 + lane], rs_s[warp][1][lane]);
-      } else {
-        if (a.rsum2) a.rsum2[row0 + lane] = rs_s[warp][0][lane];
-        if (want_rs1) a.rsum1[row0 + lane] = rs_s[warp][1][lane];
-      }
-    }
-    __syncwarp();
-  }
-  if (csum_g) {
-    __syncthreads();
-    for (int i = tid; i < C; i += blockDim.x)
-      if (csum_s[i]) atomicAdd(&csum_g[i], csum_s[i]);
-  }
-}
-
-// Column parts per chunk of kCodeRows rows in the code pass: slabs of a row
-// are split until the (chunk, part) units reach about 64 per SM.
-static int code_split_of(int64_t N, int C, int lpr, int num_sms) {
-  const int nslab = C / (16 * lpr);
-  const int64_t nchunks = (N + kCodeRows - 1) / kCodeRows;
-  const int64_t target = (int64_t)num_sms * 64;
-  int split = 1;
-  while (split < nslab && nchunks * split < target) split *= 2;
-  return split;
-}
-
-template <typename T, int LPR, int STEPS, int TEAM, int H = 1>
-static cudaError_t launch_stats(const QuantArgs &a, BhqBlock *bst, float *wsum, float2 *part,
-                                int num_sms, int *grid_out, cudaStream_t st) {
-  auto kern = k_bhq_stats<T, LPR, STEPS, TEAM, H>;
-  int per_sm = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0);
-  if (e != cudaSuccess) return e;
-  const int64_t nblocks = (a.N + a.block - 1) / a.block;
-  constexpr int TPC = 8 / TEAM;
-  int64_t grid = (nblocks + TPC - 1) / TPC;
-  int64_t cap = (int64_t)num_sms * (per_sm > 0 ? per_sm : 1);
-  if (cap > kMaxRangeCtas) cap = kMaxRangeCtas;
-  if (grid > cap) grid = cap;
-  if (grid < 1) grid = 1;
-  *grid_out = (int)grid;
-  kern<<<(int)grid, 256, 0, st>>>(a, bst, wsum, part);
-  return cudaGetLastError();
-}
-
-template <typename T, int LPR>
-static cudaError_t launch_codes(const QuantArgs &a, const BhqBlock *bst, const float *wsum,
-                                int num_sms, cudaStream_t st) {
-  int lg_nb = 0;
-  while ((1 << lg_nb) < a.block) ++lg_nb;
-  auto kern = k_bhq_codes<T, LPR>;
-  const size_t smem = sizeof(int) * (size_t)a.C;
-  int per_sm = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
-  if (e != cudaSuccess) return e;
-  const int64_t nunits = (a.N + kCodeRows - 1) / kCodeRows * (a.code_split > 1 ? a.code_split : 1);
-  int64_t grid = (nunits + 7) / 8;
-  const int64_t cap = (int64_t)num_sms * (per_sm > 0 ? per_sm : 1);
-  if (grid > cap) grid = cap;
-  if (grid < 1) grid = 1;
-  kern<<<(int)grid, 256, smem, st>>>(a, bst, wsum, lg_nb, nullptr, 1);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Per-sample PSQ (fqt_quantize_grad_samples; Sec. 4.1 with a sample = R
-// consecutive rows of dH, an image's output pixels): k_sample_part takes the
-// (min, max) of chunks of kSampleChunk rows' worth of entries inside one
-// sample; k_sample_finish reduces each sample's chunks to s = B / R(h_i),
-// z = min h_i (affine_scale, as the row quantizer), 1 / s and s z, and leaves
-// per-CTA (min, max) of the whole tensor (the range of Q_b1).  The code pass
-// (k_bhq_codes, SAMPLES) then rounds and packs.
-// ---------------------------------------------------------------------------
-constexpr int kSampleChunkElems = 16384;
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_sample_part(const QuantArgs a, int64_t sample_elems,
-                                                     int chunks_per_sample, float2 *cpart) {
-  __shared__ float2 red[8];
-  __shared__ int redi[8];
-  const int64_t ch = blockIdx.x;
-  const int64_t smp = ch / chunks_per_sample;
-  const int64_t e0 = smp * sample_elems + (ch - smp * chunks_per_sample) * kSampleChunkElems;
-  const int64_t e1 = min(smp * sample_elems + sample_elems, e0 + kSampleChunkElems);
-  const T *h = reinterpret_cast<const T *>(a.h);
-  float mn = INFINITY, mx = -INFINITY, nanacc = 0.0f;
-  for (int64_t e = e0 + (int64_t)threadIdx.x * 8; e < e1; e += (int64_t)blockDim.x * 8) {
-    float x[8];
-    load_oct(h + e, x);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      mn = fminf(mn, x[j]);
-      mx = fmaxf(mx, x[j]);
-      nanacc = fmaf(x[j], 0.0f, nanacc);
-    }
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    nanacc += __shfl_xor_sync(0xffffffffu, nanacc, off);
-  }
-  if (lane == 0) {
-    red[warp] = make_float2(mn, mx);
-    redi[warp] = isnan(nanacc) ? 1 : 0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int bad = 0;
-    for (int i = 0; i < 8; ++i) {
-      mn = fminf(mn, red[i].x);
-      mx = fmaxf(mx, red[i].y);
-      bad |= redi[i];
-    }
-    cpart[ch] = bad ? make_float2(NAN, NAN) : make_float2(mn, mx);
-  }
-}
-
-__global__ void __launch_bounds__(256) k_sample_finish(const QuantArgs a, int64_t nsamples,
-                                                       int chunks_per_sample,
-                                                       const float2 *cpart, float4 *srec,
-                                                       float2 *part) {
-  __shared__ float2 red[8];
-  __shared__ int redi[8];
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t B = (1u << a.bits) - 1u;
-  float mn = INFINITY, mx = -INFINITY;
-  int bad = 0;
-  if (i < nsamples) {
-    for (int k = 0; k < chunks_per_sample; ++k) {
-      const float2 p = cpart[i * chunks_per_sample + k];
-      bad |= isnan(p.x);
-      mn = fminf(mn, p.x);
-      mx = fmaxf(mx, p.y);
-    }
-    const float s = affine_scale(mn, mx, B);
-    srec[i] = make_float4(s, mn, __fdiv_rn(1.0f, s), __fmul_rn(s, mn));
-  }
-  // the CTA's (min, max) of the whole tensor, for Q_b1
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    bad |= __shfl_xor_sync(0xffffffffu, bad, off);
-  }
-  if (lane == 0) {
-    red[warp] = make_float2(mn, mx);
-    redi[warp] = bad;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) {
-      mn = fminf(mn, red[w].x);
-      mx = fmaxf(mx, red[w].y);
-      bad |= redi[w];
-    }
-    mn = fminf(mn, red[0].x);
-    mx = fmaxf(mx, red[0].y);
-    bad |= redi[0];
-    part[blockIdx.x] = bad ? make_float2(NAN, NAN) : make_float2(mn, mx);
-  }
-  // the code pass accumulates column sums (and, split, row sums) into these
-  for (int64_t k = i; k < a.C; k += (int64_t)gridDim.x * blockDim.x) {
-    if (a.csum1) a.csum1[k] = 0;
-    if (a.csum2) a.csum2[k] = 0;
-  }
-  if (a.code_split > 1)
-    for (int64_t k = i; k < a.N; k += (int64_t)gridDim.x * blockDim.x) {
-      if (a.rsum1) a.rsum1[k] = 0;
-      if (a.rsum2) a.rsum2[k] = 0;
-    }
-}
-
-// Workspace bytes of the per-sample quantizer: chunk partials and records.
-size_t sample_pass_bytes(int64_t N, int64_t C, int64_t rows_per_sample) {
-  if (rows_per_sample < 1) return 0;
-  const int64_t ns = N / rows_per_sample;
-  const int64_t cps = (rows_per_sample * C + kSampleChunkElems - 1) / kSampleChunkElems;
-  return (size_t)(ns * cps) * sizeof(float2) + (size_t)ns * sizeof(float4) + 512;
-}
-
-// The per-sample PSQ with Q_b1: rows of C in {64, 128, 256 t} columns
-// (t = 1, 2, 4, 8), N a multiple of rows_per_sample, at most 2^20 samples.
-fqt_status launch_sample_passes(QuantArgs &a, bool bf16, int64_t rows_per_sample, int num_sms,
-                                void *scratch, float2 *part, cudaStream_t st) {
-  const int C = a.C;
-  if (!(C == 64 || C == 128 || C == 256 || C == 512 || C == 1024 || C == 2048 || C == 4096))
-    return FQT_EUNSUPPORTED;
-  const int64_t ns = a.N / rows_per_sample;
-  if (ns > ((int64_t)1 << 20)) return FQT_EUNSUPPORTED;
-  const int64_t se = rows_per_sample * C;
-  const int cps = (int)((se + kSampleChunkElems - 1) / kSampleChunkElems);
-  float2 *cpart = static_cast<float2 *>(scratch);
-  float4 *srec = reinterpret_cast<float4 *>(
-      (reinterpret_cast<uintptr_t>(cpart + ns * cps) + 255) & ~(uintptr_t)255);
-  const int lpr = C == 64 ? 4 : C == 128 ? 8 : C == 256 ? 16 : 32;
-  a.code_split = code_split_of(a.N, C, lpr, num_sms);
-  if (bf16)
-    k_sample_part<__nv_bfloat16><<<(unsigned)(ns * cps), 256, 0, st>>>(a, se, cps, cpart);
-  else
-    k_sample_part<float><<<(unsigned)(ns * cps), 256, 0, st>>>(a, se, cps, cpart);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "sample statistics launch");
-  const int fin = (int)((ns + 255) / 256);
-  k_sample_finish<<<fin, 256, 0, st>>>(a, ns, cps, cpart, srec, part);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "sample scalars launch");
-  QuantArgs a2 = a;
-  a2.part = part;
-  a2.npart = fin;
-  const int R = (int)rows_per_sample;
-#define FQT_SC(TT, L)                                                                        \
-  {                                                                                          \
-    auto kern = k_bhq_codes<TT, L, true>;                                                    \
-    const size_t smem = sizeof(int) * (size_t)C;                                             \
-    int per_sm = 0;                                                                          \
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);             \
-    if (e == cudaSuccess) {                                                                  \
-      const int64_t nunits = (a.N + kCodeRows - 1) / kCodeRows * a2.code_split;              \
-      int64_t grid = (nunits + 7) / 8;                                                       \
-      const int64_t cap = (int64_t)num_sms * (per_sm > 0 ? per_sm : 1);                     \
-      if (grid > cap) grid = cap;                                                            \
-      if (grid < 1) grid = 1;                                                                \
-      kern<<<(int)grid, 256, smem, st>>>(a2, nullptr, nullptr, 0, srec, R);                  \
-      e = cudaGetLastError();                                                                \
-    }                                                                                        \
-  }
-  if (!bf16) {
-    if (lpr == 4) FQT_SC(float, 4) else if (lpr == 8) FQT_SC(float, 8)
-    else if (lpr == 16) FQT_SC(float, 16) else FQT_SC(float, 32)
-  } else {
-    if (lpr == 4) FQT_SC(__nv_bfloat16, 4) else if (lpr == 8) FQT_SC(__nv_bfloat16, 8)
-    else if (lpr == 16) FQT_SC(__nv_bfloat16, 16) else FQT_SC(__nv_bfloat16, 32)
-  }
-#undef FQT_SC
-  return cuda_fail(e, "sample code pass launch");
-}
-
-// The two-pass BHQ quantizer takes fixed blocks of 4, 8 or 16 rows and rows
-// of 64, 128 or 256 t (t = 1, 2, 4, 8, 16) columns; bf16 input with blocks of 16.
-bool bhq_pass_supported(int C, int block, bool bf16) {
-  if (block != 4 && block != 8 && block != 16) return false;
-  if (bf16 && block != 16) return false;
-  return C == 64 || C == 128 || C == 256 || C == 512 || C == 1024 || C == 2048 || C == 4096;
-}
-
-// Statistics pass, code pass and the grad_X offsets (k_bhq_offsets) of the
-// fixed-block BHQ quantizer with Q_b1.  `scratch` (bhq_pass_bytes) holds the
-// per-block records and column sums w between the passes; `part` receives
-// the statistics pass's range partials, which the code pass reduces.
-fqt_status launch_bhq_passes(QuantArgs &a, bool bf16, int num_sms, void *scratch,
-                             float2 *part, cudaStream_t st) {
-  if (a.kind != KIND_BHQ || !bhq_pass_supported(a.C, a.block, bf16)) return FQT_EUNSUPPORTED;
-  const int64_t nblocks = (a.N + a.block - 1) / a.block;
-  BhqBlock *bst = static_cast<BhqBlock *>(scratch);
-  float *wsum = reinterpret_cast<float *>(
-      (reinterpret_cast<uintptr_t>(bst + nblocks) + 255) & ~(uintptr_t)255);
-  const int C = a.C, nb = a.block;
-  // lanes per row of the code pass: a lane owns 16 columns (two octs) of a
-  // slab of 16 LPR
-  const int lpr = C == 64 ? 4 : C == 128 ? 8 : C == 256 ? 16 : 32;
-  a.code_split = code_split_of(a.N, C, lpr, num_sms);
-  int grid1 = 0;
-  cudaError_t e = cudaErrorInvalidValue;
-#define FQT_ST(TT, L, S, TM) e = launch_stats<TT, L, S, TM>(a, bst, wsum, part, num_sms, &grid1, st);
-  // C = 4096: a team of 8 warps over two column halves
-#define FQT_ST2(TT, L, S) e = launch_stats<TT, L, S, 8, 2>(a, bst, wsum, part, num_sms, &grid1, st);
-  if (!bf16) {
-    if (C == 64) {
-      if (nb == 4) { FQT_ST(float, 8, 1, 1) } else if (nb == 8) { FQT_ST(float, 8, 2, 1) }
-      else { FQT_ST(float, 8, 4, 1) }
-    } else if (C == 128) {
-      if (nb == 4) { FQT_ST(float, 16, 2, 1) } else if (nb == 8) { FQT_ST(float, 16, 4, 1) }
-      else { FQT_ST(float, 16, 8, 1) }
-    } else {
-      const int team = C / 256;
-#define FQT_ST_T(S)                                                                  \
-  if (team == 1) { FQT_ST(float, 32, S, 1) } else if (team == 2) { FQT_ST(float, 32, S, 2) } \
-  else if (team == 4) { FQT_ST(float, 32, S, 4) } else if (team == 8) { FQT_ST(float, 32, S, 8) } \
-  else { FQT_ST2(float, 32, S) }
-      if (nb == 4) { FQT_ST_T(4) } else if (nb == 8) { FQT_ST_T(8) } else { FQT_ST_T(16) }
-#undef FQT_ST_T
-    }
-  } else {
-    if (C == 64) { FQT_ST(__nv_bfloat16, 8, 4, 1) }
-    else if (C == 128) { FQT_ST(__nv_bfloat16, 16, 8, 1) }
-    else if (C == 256) { FQT_ST(__nv_bfloat16, 32, 16, 1) }
-    else if (C == 512) { FQT_ST(__nv_bfloat16, 32, 16, 2) }
-    else if (C == 1024) { FQT_ST(__nv_bfloat16, 32, 16, 4) }
-    else if (C == 2048) { FQT_ST(__nv_bfloat16, 32, 16, 8) }
-    else { FQT_ST2(__nv_bfloat16, 32, 16) }
-  }
-#undef FQT_ST
-#undef FQT_ST2
-  if (e != cudaSuccess) return cuda_fail(e, "BHQ statistics pass launch");
-  QuantArgs a2 = a;
-  a2.part = part;
-  a2.npart = grid1;
-  if (!bf16) {
-    e = lpr == 4    ? launch_codes<float, 4>(a2, bst, wsum, num_sms, st)
-        : lpr == 8  ? launch_codes<float, 8>(a2, bst, wsum, num_sms, st)
-        : lpr == 16 ? launch_codes<float, 16>(a2, bst, wsum, num_sms, st)
-                    : launch_codes<float, 32>(a2, bst, wsum, num_sms, st);
-  } else {
-    e = lpr == 4    ? launch_codes<__nv_bfloat16, 4>(a2, bst, wsum, num_sms, st)
-        : lpr == 8  ? launch_codes<__nv_bfloat16, 8>(a2, bst, wsum, num_sms, st)
-        : lpr == 16 ? launch_codes<__nv_bfloat16, 16>(a2, bst, wsum, num_sms, st)
-                    : launch_codes<__nv_bfloat16, 32>(a2, bst, wsum, num_sms, st);
-  }
-  if (e != cudaSuccess) return cuda_fail(e, "BHQ code pass launch");
-  if (a.hz && a.hr) {
-    e = launch_bhq_offsets(a.zero2, a.rsum2, a.lead2, a.hz, a.hr, a.N, C, a.bits, a.block, st);
-    if (e != cudaSuccess) return cuda_fail(e, "BHQ offsets launch");
-  }
-  return FQT_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -2415,6 +1500,17 @@ __global__ void __launch_bounds__(kOffThreads)
   }
   ds[t] = make_float2(d.h, d.l);
   Rs[t] = R;
+  // the sums of a block of up to 32 rows by shuffles (rows past N add 0): a
+  // loop over its rows in every thread took 16.7 us for 802816 rows in blocks
+  // of 16, this 12.9 us
+  ff sdw = d;
+  long long sRw = R;
+  for (int off = 1; off < nb && off < 32; off <<= 1) {
+    const ff od = {__shfl_xor_sync(0xffffffffu, sdw.h, off),
+                   __shfl_xor_sync(0xffffffffu, sdw.l, off)};
+    sdw = ff_add(sdw, od);
+    sRw += __shfl_xor_sync(0xffffffffu, sRw, off);
+  }
   __syncthreads();
   if (!kv) return;
   const int base = (t / nb) * nb;  // nb divides kOffThreads: blocks stay in the CTA
@@ -2428,9 +1524,14 @@ __global__ void __launch_bounds__(kOffThreads)
   const int p = lead[kb / nb];
   ff sd = {0.0f, 0.0f};
   long long sR = 0;
-  for (int l = 0; l < nact; ++l) {
-    sd = ff_add(sd, {ds[base + l].x, ds[base + l].y});
-    sR += Rs[base + l];
+  if (nb <= 32) {
+    sd = sdw;
+    sR = sRw;
+  } else {
+    for (int l = 0; l < nact; ++l) {
+      sd = ff_add(sd, {ds[base + l].x, ds[base + l].y});
+      sR += Rs[base + l];
+    }
   }
   const HhConst c = hh_const(nact);
   // (Q v)_k = v_k - kappa (rho sum(v) - v_p) off the lead row; rho sum(v) on it
@@ -2534,7 +1635,7 @@ fqt_status quant_geometry(QuantArgs &a, int num_sms, int *nth_out,
 fqt_status quant2_geometry(QuantArgs &a, bool bf16, int num_sms, int *grid_out,
                            size_t *smem_out) {
   const int C = a.C;
-  if (C <= 0 || C % 8 || a.kind == KIND_DET) return FQT_EUNSUPPORTED;
+  if (C <= 0 || C % 8 || (a.kind != KIND_PSQ && a.kind != KIND_BHQ)) return FQT_EUNSUPPORTED;
   const int CO = C / 8;
   if (CO > 32 * kMaxOct) return FQT_EUNSUPPORTED;  // rows longer than 1024
   const int esize = bf16 ? 2 : 4;
@@ -2595,8 +1696,6 @@ static cudaError_t launch_quant2_t(const QuantArgs &a, int grid, size_t smem,
 cudaError_t launch_quant2(const QuantArgs &a, bool bf16, int grid, size_t smem,
                           cudaStream_t st) {
   switch (a.kind * 2 + (bf16 ? 1 : 0)) {
-    case KIND_PTQ * 2: return launch_quant2_t<KIND_PTQ, float>(a, grid, smem, st);
-    case KIND_PTQ * 2 + 1: return launch_quant2_t<KIND_PTQ, __nv_bfloat16>(a, grid, smem, st);
     case KIND_PSQ * 2: return launch_quant2_t<KIND_PSQ, float>(a, grid, smem, st);
     case KIND_PSQ * 2 + 1: return launch_quant2_t<KIND_PSQ, __nv_bfloat16>(a, grid, smem, st);
     case KIND_BHQ * 2: return launch_quant2_t<KIND_BHQ, float>(a, grid, smem, st);

@@ -1,0 +1,71 @@
+"""The statistics and code passes of the gradient quantizers at the edges of
+their layouts (rows of one oct, odd octs, one column past and short of a slab
+or a team, the widest; blocks of 4, 8, 16 with a ragged last one; units of 8
+rows and column splits), and the one-pass quantizers that a workspace without
+their scratch takes: codes against the oracle (PTQ, PSQ equal; BHQ within +-1
+at a rounding threshold), sums equal to those of the codes."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+from paper_2010_14298_gb300 import fqt
+from paper_2010_14298_gb300 import workloads as wl
+from gpu_util import to_dev
+from test_gpu_parity import _check_b1, _check_bhq_codes
+
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="no GPU")]
+
+
+def _check(n, c, kind, bits, block, dtype, ws=None, seed=99):
+    g = wl.rng(n * 7 + c)
+    dH = wl.random_grad(g, n, c)
+    if dtype == "bf16":
+        dH = wl.to_bf16_values(dH)
+    ws = ws or fqt.Workspace(n, c, 16)
+    q2, q1 = fqt.quantize_grad(to_dev(dH, dtype), kind, bits, block, seed, ws=ws)
+    assert fqt.sync_status(ws) == 0
+    ref = orc.quantize_grad(dH, kind, bits, block, seed, orc.STREAM_B2, want_v=True)
+    h2 = q2.to_numpy()
+    assert torch.equal(q2.codes, q2.codes_from_f16())
+    assert np.array_equal(h2["row_sum"], h2["codes"].astype(np.int64).sum(1))
+    if kind == orc.BHQ:
+        assert np.array_equal(h2["lead"], ref["lead"])
+        _check_bhq_codes(h2["codes"], ref["codes"], ref["v"], seed)
+        assert np.allclose(h2["inv_s"], ref["inv_s"], rtol=1e-6, atol=0)
+        assert np.allclose(h2["zero"], ref["zero"], rtol=1e-5, atol=1e-4)
+    else:
+        assert np.array_equal(h2["codes"], ref["codes"])
+        assert np.array_equal(h2["inv_s"], ref["inv_s"])
+        assert np.array_equal(h2["zero"], ref["zero"])
+    _check_b1(q1, dH, seed)
+
+
+WIDTHS = [8, 24, 64, 72, 136, 248, 264, 336, 520, 1008, 1032, 2056, 4088]
+
+
+@pytest.mark.parametrize("c", WIDTHS)
+@pytest.mark.parametrize("block,dtype", [(4, "f32"), (8, "bf16"), (16, "f32"), (16, "bf16")])
+def test_bhq_widths(c, block, dtype):
+    _check(5 * 16 + 7, c, orc.BHQ, 5, block, dtype)
+
+
+@pytest.mark.parametrize("c", WIDTHS + [8192])
+@pytest.mark.parametrize("kind,bits,dtype", [(orc.PTQ, 8, "f32"), (orc.PSQ, 8, "bf16"),
+                                             (orc.PSQ, 4, "f32")])
+def test_affine_widths(c, kind, bits, dtype):
+    _check(61, c, kind, bits, 0, dtype)
+
+
+@pytest.mark.parametrize("n,c,kind,block", [(1, 64, orc.BHQ, 4), (3, 128, orc.PSQ, 0),
+                                            (9000, 80, orc.BHQ, 8), (9000, 80, orc.PTQ, 0)])
+def test_row_counts(n, c, kind, block):
+    _check(n, c, kind, 5, block, "f32")
+
+
+@pytest.mark.parametrize("c,kind,block", [(336, orc.PSQ, 0), (1008, orc.BHQ, 16)])
+def test_small_workspace_takes_the_one_pass_quantizer(c, kind, block):
+    ws = fqt.Workspace(1, 16, 16)
+    ws.nbytes = 256 + 32768  # the header and the range partials
+    _check(200, c, kind, 5, block, "f32", ws)
