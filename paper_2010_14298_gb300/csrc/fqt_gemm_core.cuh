@@ -60,7 +60,7 @@ constexpr size_t kBoxBytes = 4096;   // one 32 x 32 fp32 / int32 output box
 //   [kFixedBytes, +S * 32 KiB) S operand stages (A, B)
 //   [..., + 8 * R * 4 KiB)     R output boxes per epilogue warp (TMA store ring)
 // grad_X parameter stages (one per tile in flight), each:
-//   float4 kp[BN]  per row k: inv_sw inv_s_k, .. hz_k, .. y hr_k, m_k
+//   RowPar kp      per row k: inv_sw inv_s_k, .. hz_k, .. y hr_k, m_k
 //   int leads[BN]  lead row of each block;  int msum[BN]  sum of m per block
 //   int cs[BM]     W~ column sums of the tile's columns;  int flag
 constexpr int kParStages = 4;
@@ -445,6 +445,12 @@ struct BoxOut {
   __device__ __forceinline__ void st(int row, float v) const {
     if (jv && row < rows) __stcs(p + row * ld, v);
   }
+  __device__ __forceinline__ void st2(int row, f32x2 v) const {
+    float a, b;
+    unpack2(v, a, b);
+    st(row, a);
+    st(row + 1, b);
+  }
   // all 32 values of the box (then the lead-row overwrites, same thread)
   __device__ __forceinline__ void st32(const float (&o)[32]) const {
     if (!jv) return;
@@ -607,13 +613,55 @@ __device__ __forceinline__ float dequant(const float4 &kq, float t, float U) {
   return __fmaf_rn(kq.x, t, __fmaf_rn(kq.y, U, kq.z));
 }
 
+// The per-row terms (sc, A = sc hz, B = sc y hr, m) of a tile in shared
+// memory, two rows interleaved ({sc, sc', A, A'}, {B, B', m, m'}) so that the
+// epilogue dequantizes rows in packed pairs.
+struct RowPair {
+  f32x2 sc, A, B, m;
+};
+
+struct RowPar {
+  float *p;
+  __device__ __forceinline__ RowPair pair(int k) const {  // rows k, k + 1 (k even)
+    const float4 x = *reinterpret_cast<const float4 *>(p + 4 * k);
+    const float4 y = *reinterpret_cast<const float4 *>(p + 4 * k + 4);
+    return {pack2(x.x, x.y), pack2(x.z, x.w), pack2(y.x, y.y), pack2(y.z, y.w)};
+  }
+  __device__ __forceinline__ float4 row(int k) const {
+    const float *q = p + 8 * (k >> 1) + (k & 1);
+    return make_float4(q[0], q[2], q[4], q[6]);
+  }
+  __device__ __forceinline__ float m(int k) const { return p[8 * (k >> 1) + (k & 1) + 6]; }
+  __device__ __forceinline__ void set(int k, float sc, float A, float B, float m) const {
+    float *q = p + 8 * (k >> 1) + (k & 1);
+    q[0] = sc;
+    q[2] = A;
+    q[4] = B;
+    q[6] = m;
+  }
+};
+
+// dequant() of two rows
+__device__ __forceinline__ f32x2 dequant2(const RowPair &q, f32x2 t, f32x2 U) {
+  return fma2(q.sc, t, fma2(q.A, U, q.B));
+}
+
+// Row i of a column whose row 0 is at p (ld = the row stride in entries; one
+// widening multiply-add per address).
+__device__ __forceinline__ float *row_ptr(float *p, uint32_t ld, int i) {
+  return reinterpret_cast<float *>(reinterpret_cast<char *>(p) + (uint64_t)ld * (uint32_t)(4 * i));
+}
+
 // The integer parts I = P + m CWc of 32 rows (one box) of this thread's
 // column in the int32 form.
 struct Ints {
   int v[32];
   __device__ __forceinline__ float f(int i) const { return __int2float_rn(v[i]); }
-  __device__ __forceinline__ float minus(int i, const BlockFix &b) const {
-    return __fsub_rn(__int2float_rn((int)((uint32_t)v[i] - (uint32_t)b.bi)), b.bf);
+  __device__ __forceinline__ f32x2 f2(int i) const { return pack2(f(i), f(i + 1)); }
+  __device__ __forceinline__ f32x2 minus2(int i, const BlockFix &b) const {
+    return add2(pack2(__int2float_rn((int)((uint32_t)v[i] - (uint32_t)b.bi)),
+                      __int2float_rn((int)((uint32_t)v[i + 1] - (uint32_t)b.bi))),
+                pack2(-b.bf, -b.bf));
   }
 };
 
@@ -634,12 +682,12 @@ __device__ __forceinline__ void load_products(uint32_t acc, uint32_t ints, bool 
 // Loads the products of the 32 rows at TMEM column c0 and forms I
 // (|m| <= i32_mmax and |CWc| <= C 2^(bw-1) are below 2^22).
 __device__ __forceinline__ void load_ints(uint32_t acc, uint32_t ints, bool multi, int c0,
-                                          const float4 *kp, float cwc, Ints &I) {
+                                          const RowPar &kp, float cwc, Ints &I) {
   load_products(acc, ints, multi, c0, I.v);
   const uint32_t cw = (uint32_t)magic_int(cwc);
 #pragma unroll
   for (int i = 0; i < 32; ++i)
-    I.v[i] = (int)((uint32_t)I.v[i] + (uint32_t)magic_int(kp[c0 + i].w) * cw);
+    I.v[i] = (int)((uint32_t)I.v[i] + (uint32_t)magic_int(kp.m(c0 + i)) * cw);
 }
 
 // I of one row (TMEM column col) of this thread's column.
@@ -660,12 +708,13 @@ __host__ __device__ constexpr int leads_per_box(int nb) { return nb > 1 && nb <=
 
 template <int NB>
 __device__ __forceinline__ void box_small(const Ints &I, const int (&Ip)[leads_per_box(NB)],
-                                          const HhConst &hc, const float4 *kp,
+                                          const HhConst &hc, const RowPar &kp,
                                           const int *leads, int r0, int64_t row0,
                                           int64_t N, float U, const BoxOut &w) {
+  const f32x2 U2 = pack2(U, U);
   if (NB == 1) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) w.st(i, dequant(kp[r0 + i], I.f(i), U));
+    for (int i = 0; i < 32; i += 2) w.st2(i, dequant2(kp.pair(r0 + i), I.f2(i), U2));
     return;
   }
   constexpr int NBB = NB > 1 ? NB : 2;
@@ -676,7 +725,8 @@ __device__ __forceinline__ void box_small(const Ints &I, const int (&Ip)[leads_p
     const int nact = left >= NBB ? NBB : (int)(left > 0 ? left : 0);
     if (nact < 2) {  // a one-row block is not transformed
 #pragma unroll
-      for (int l = 0; l < NBB; ++l) w.st(b * NBB + l, dequant(kp[kb0 + l], I.f(b * NBB + l), U));
+      for (int l = 0; l < NBB; l += 2)
+        w.st2(b * NBB + l, dequant2(kp.pair(kb0 + l), I.f2(b * NBB + l), U2));
       continue;
     }
     long long S = 0;
@@ -684,9 +734,10 @@ __device__ __forceinline__ void box_small(const Ints &I, const int (&Ip)[leads_p
     for (int l = 0; l < NBB; ++l) S += I.v[b * NBB + l];
     const BlockFix f = block_fix(nact == NBB ? hc : hh_const(nact), S, Ip[b]);
 #pragma unroll
-    for (int l = 0; l < NBB; ++l) w.st(b * NBB + l, dequant(kp[kb0 + l], I.minus(b * NBB + l, f), U));
+    for (int l = 0; l < NBB; l += 2)
+      w.st2(b * NBB + l, dequant2(kp.pair(kb0 + l), I.minus2(b * NBB + l, f), U2));
     const int p = leads[kb0 / NBB];  // the lead row: a later store of the same thread
-    w.st(b * NBB + p, dequant(kp[kb0 + p], f.lead, U));
+    w.st(b * NBB + p, dequant(kp.row(kb0 + p), f.lead, U));
   }
 }
 
@@ -696,7 +747,7 @@ __device__ __forceinline__ void box_small(const Ints &I, const int (&Ip)[leads_p
 // exact products P are stored as int32 bit patterns for gradx_raw_fix.
 template <int NB, bool PAIR>
 __device__ __forceinline__ void gradx_tile(const GemmArgs &g, const Item &t, uint32_t acc,
-                                           uint32_t ints, bool multi, const float4 *kp,
+                                           uint32_t ints, bool multi, const RowPar &kp,
                                            const int *leads, const HhConst &hc, float cwc,
                                            float U, uint64_t *acce_set, int q, int lane,
                                            bool raw) {
@@ -716,7 +767,7 @@ __device__ __forceinline__ void gradx_tile(const GemmArgs &g, const Item &t, uin
         for (int i = 0; i < 32; ++i) S_big += I.v[i];
       }
       p_big = leads[g0 / (NB > 32 ? NB : 1)];
-      Ip_big = load_int1(acc, ints, multi, g0 + p_big, kp[g0 + p_big].w, cwc);
+      Ip_big = load_int1(acc, ints, multi, g0 + p_big, kp.m(g0 + p_big), cwc);
     }
 #pragma unroll 1
     for (int bx = 0; bx < GW / 32; ++bx) {
@@ -730,7 +781,7 @@ __device__ __forceinline__ void gradx_tile(const GemmArgs &g, const Item &t, uin
         Ip[b] = 0;
         if (NB > 1 && NB <= 32) {
           const int col = r0 + b * (32 / NPP) + leads[(r0 + b * (32 / NPP)) / (32 / NPP)];
-          Ip[b] = load_int1(acc, ints, multi, col, kp[col].w, cwc);
+          Ip[b] = load_int1(acc, ints, multi, col, kp.m(col), cwc);
         }
       }
       if (r0 + 32 == BN) {  // the accumulator has been read in full
@@ -749,13 +800,15 @@ __device__ __forceinline__ void gradx_tile(const GemmArgs &g, const Item &t, uin
         const int nact = left >= NB ? NB : (int)(left > 0 ? left : 0);
         if (nact < 2) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) w.st(i, dequant(kp[r0 + i], I.f(i), U));
+          for (int i = 0; i < 32; i += 2)
+            w.st2(i, dequant2(kp.pair(r0 + i), I.f2(i), pack2(U, U)));
         } else {
           const BlockFix f = block_fix(nact == NB ? hc : hh_const(nact), S_big, Ip_big);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) w.st(i, dequant(kp[r0 + i], I.minus(i, f), U));
+          for (int i = 0; i < 32; i += 2)
+            w.st2(i, dequant2(kp.pair(r0 + i), I.minus2(i, f), pack2(U, U)));
           if (p_big >= bx * 32 && p_big < bx * 32 + 32)
-            w.st(p_big - bx * 32, dequant(kp[g0 + p_big], f.lead, U));
+            w.st(p_big - bx * 32, dequant(kp.row(g0 + p_big), f.lead, U));
         }
       }
     }
@@ -777,8 +830,32 @@ __device__ __forceinline__ BlockFixF block_fix_f(const HhConst &c, int S, int Ip
   return f;
 }
 
-// (Q I)_k of a non-lead row in the fp32 form: (P - bi) + m CWc is exact
-// (every magnitude below 2^24), then the remainder bf.
+// Two non-lead rows of Q I in the fp32 form: (P - bi) + m CWc is exact (every
+// magnitude below 2^24), then the remainder bf.
+__device__ __forceinline__ f32x2 reflect2(f32x2 P, const RowPair &q, f32x2 cwc,
+                                          const BlockFixF &f) {
+  return add2(fma2(q.m, cwc, add2(P, pack2(-f.bi, -f.bi))), pack2(-f.bf, -f.bf));
+}
+
+// The sum of the integers that fp32 values below 2^22 in magnitude hold, off
+// the bits of v + 1.5 2^23 (n such words carry n kMagicBits).
+__device__ __forceinline__ uint32_t magic_sum2(f32x2 v) {
+  float a, b;
+  unpack2(add2(v, pack2(kMagic, kMagic)), a, b);
+  return __float_as_uint(a) + __float_as_uint(b);
+}
+
+__device__ __forceinline__ f32x2 pair_of(const uint32_t *r) {
+  return pack2(__uint_as_float(r[0]), __uint_as_float(r[1]));
+}
+__device__ __forceinline__ void set_pair(uint32_t *r, f32x2 v) {
+  float a, b;
+  unpack2(v, a, b);
+  r[0] = __float_as_uint(a);
+  r[1] = __float_as_uint(b);
+}
+
+// (Q I)_k of a non-lead row, one at a time (the passes over raw rows).
 __device__ __forceinline__ float reflect_f(float P, const float4 &kq, float cwc,
                                            const BlockFixF &f) {
   return __fsub_rn(__fmaf_rn(kq.w, cwc, __fsub_rn(P, f.bi)), f.bf);
@@ -790,21 +867,21 @@ __device__ __forceinline__ float reflect_f(float P, const float4 &kq, float cwc,
 // no block is transformed, so the stores are its exact products P.
 template <int NB, bool PAIR>
 __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, uint32_t acc,
-                                             const float4 *kp, const int *leads,
+                                             const RowPar &kp, const int *leads,
                                              const int *msum, const HhConst &hc, float cwc,
                                              float U, uint64_t *acce_set, int q, int lane,
                                              bool raw) {
-  constexpr int GW = NB > 32 ? NB : 32;
-  constexpr int NPP = leads_per_box(NB);
   constexpr int NBD = NB > 1 ? NB : 1;
   const int cwi = (int)cwc;
+  const f32x2 cw2 = pack2(cwc, cwc), U2 = pack2(U, U);
+  const int64_t j = t.m0 + q * 32 + lane;
+  const bool jv = j < g.M;
+  const uint32_t ld = (uint32_t)g.M;
   if constexpr (NB <= 32) {
     // one block (NB >= 8) or 16 rows (no reflection) per step, loaded from
     // TMEM on its own, so few values are live at a time
     constexpr int CH = NB >= 8 ? NB : (NB <= 1 ? 16 : 8);
     constexpr int BPC = NB > 1 ? CH / NB : 0;  // blocks per chunk
-    const int64_t j = t.m0 + q * 32 + lane;
-    const bool jv = j < g.M;
 #pragma unroll 1
     for (int r0 = 0; r0 < BN; r0 += CH) {
       uint32_t r[CH];
@@ -826,9 +903,9 @@ __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, u
       float *po = g.out + (jv && rows > 0 ? row0 * g.M + j : 0);
       if constexpr (NB <= 1) {
 #pragma unroll
-        for (int i = 0; i < CH; ++i) {
-          const float4 kq = kp[r0 + i];
-          r[i] = __float_as_uint(dequant(kq, __fmaf_rn(kq.w, cwc, __uint_as_float(r[i])), U));
+        for (int i = 0; i < CH; i += 2) {
+          const RowPair kq = kp.pair(r0 + i);
+          set_pair(r + i, dequant2(kq, fma2(kq.m, cw2, pair_of(r + i)), U2));
         }
       }
       int lrow[BPC > 0 ? BPC : 1];
@@ -846,26 +923,26 @@ __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, u
           const int nact = lb >= NBD ? NBD : (int)(lb > 0 ? lb : 0);
           if (nact < 2 || raw) {  // a one-row block is not transformed
 #pragma unroll
-            for (int l = 0; l < NBD; ++l) {
-              const float4 kq = kp[kb0 + l];
-              r[b * NBD + l] = __float_as_uint(
-                  dequant(kq, __fmaf_rn(kq.w, cwc, __uint_as_float(r[b * NBD + l])), U));
+            for (int l = 0; l < NBD; l += 2) {
+              const RowPair kq = kp.pair(kb0 + l);
+              uint32_t *v = r + b * NBD + l;
+              set_pair(v, dequant2(kq, fma2(kq.m, cw2, pair_of(v)), U2));
             }
             continue;
           }
           uint32_t sb = 0u;
 #pragma unroll
-          for (int l = 0; l < NBD; ++l) sb += magic_bits(__uint_as_float(r[b * NBD + l]));
+          for (int l = 0; l < NBD; l += 2) sb += magic_sum2(pair_of(r + b * NBD + l));
           const int S = (int)(sb - (uint32_t)NBD * kMagicBits) + cwi * msum[kb0 / NBD];
           const int p = leads[kb0 / NBD];
-          const float4 kl = kp[kb0 + p];
+          const float4 kl = kp.row(kb0 + p);
           const int Ip = magic_int(__uint_as_float(pp[b])) + (int)kl.w * cwi;
           const BlockFixF f = block_fix_f(nact == NBD ? hc : hh_const(nact), S, Ip);
 #pragma unroll
-          for (int l = 0; l < NBD; ++l) {
-            const float4 kq = kp[kb0 + l];
-            r[b * NBD + l] = __float_as_uint(
-                dequant(kq, reflect_f(__uint_as_float(r[b * NBD + l]), kq, cwc, f), U));
+          for (int l = 0; l < NBD; l += 2) {
+            const RowPair kq = kp.pair(kb0 + l);
+            uint32_t *v = r + b * NBD + l;
+            set_pair(v, dequant2(kq, reflect2(pair_of(v), kq, cw2, f), U2));
           }
           lrow[b] = b * NBD + p;
           lval[b] = dequant(kl, f.lead, U);
@@ -881,11 +958,11 @@ __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, u
       } else if (jv) {
         if (rows == CH) {
 #pragma unroll
-          for (int i = 0; i < CH; ++i) __stcs(po + (int64_t)i * g.M, __uint_as_float(r[i]));
+          for (int i = 0; i < CH; ++i) __stcs(row_ptr(po, ld, i), __uint_as_float(r[i]));
         } else {
 #pragma unroll
           for (int i = 0; i < CH; ++i)
-            if (i < rows) __stcs(po + (int64_t)i * g.M, __uint_as_float(r[i]));
+            if (i < rows) __stcs(row_ptr(po, ld, i), __uint_as_float(r[i]));
         }
         // the lead rows: later stores of the same thread to the same address
 #pragma unroll
@@ -894,123 +971,60 @@ __device__ __forceinline__ void gradx_tile_f(const GemmArgs &g, const Item &t, u
       }
     }
   } else {
+    // blocks of more than 32 rows: their sums over all boxes of 32 first
 #pragma unroll 1
-  for (int g0 = 0; g0 < BN; g0 += GW) {
-    int S_big = 0, Ip_big = 0, p_big = 0;
-    if constexpr (NB > 32) {
+    for (int g0 = 0; g0 < BN; g0 += NBD) {
       uint32_t sb = 0u;
 #pragma unroll 1
-      for (int bx = 0; bx < GW / 32; ++bx) {
+      for (int bx = 0; bx < NBD / 32; ++bx) {
         uint32_t r[32];
         tmem_ld32_nw(acc + (uint32_t)(g0 + bx * 32), r);
         tmem_wait_ld(r);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) sb += magic_bits(__uint_as_float(r[i]));
+        for (int i = 0; i < 32; i += 2) sb += magic_sum2(pair_of(r + i));
       }
-      S_big = (int)(sb - (uint32_t)NB * kMagicBits) + cwi * msum[g0 / NBD];
-      p_big = leads[g0 / NBD];
-      uint32_t v[1];
-      v[0] = tmem_ld1_nw(acc + (uint32_t)(g0 + p_big));
-      tmem_wait_ld(v);
-      Ip_big = magic_int(__uint_as_float(v[0])) + (int)kp[g0 + p_big].w * cwi;
-    }
+      const int S = (int)(sb - (uint32_t)NB * kMagicBits) + cwi * msum[g0 / NBD];
+      const int p = leads[g0 / NBD];
+      uint32_t pv[1];
+      pv[0] = tmem_ld1_nw(acc + (uint32_t)(g0 + p));
+      tmem_wait_ld(pv);
+      const float4 kl = kp.row(g0 + p);
+      const int Ip = magic_int(__uint_as_float(pv[0])) + (int)kl.w * cwi;
+      const int64_t left = g.N - (t.n0 + g0);
+      const int nact = left >= NB ? NB : (int)(left > 0 ? left : 0);
+      const bool refl = nact >= 2 && !raw;
+      const BlockFixF f = block_fix_f(nact == NB || !refl ? hc : hh_const(nact), S, Ip);
 #pragma unroll 1
-    for (int bx = 0; bx < GW / 32; ++bx) {
-      const int r0 = g0 + bx * 32;
-      const BoxOut w = box_out(g, t, q, lane, r0);
-      uint32_t r[32];
-      tmem_ld32_nw(acc + (uint32_t)r0, r);
-      uint32_t pp[NPP];
-#pragma unroll
-      for (int b = 0; b < NPP; ++b)
-        pp[b] = (NB > 1 && NB <= 32)
-                    ? tmem_ld1_nw(acc + (uint32_t)(r0 + b * NBD + leads[(r0 + b * NBD) / NBD]))
-                    : 0u;
-      tmem_wait_ld(r);
-      tmem_wait_ld(pp);
-      if (r0 + 32 == BN) {  // the accumulator has been read in full
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) acc_release<PAIR>(acce_set);
-      }
-      // every output of the box is formed in registers before the first
-      // store, so the per-row loads from shared memory need not wait for
-      // the stores into the (possibly aliasing) box
-      // outputs overwrite the products in place (r holds fp32 bit patterns)
-      int lead_row = -1;
-      float lead_val = 0.0f;
-      if constexpr (NB == 1) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float4 kq = kp[r0 + i];
-          r[i] = __float_as_uint(dequant(kq, __fmaf_rn(kq.w, cwc, __uint_as_float(r[i])), U));
+      for (int bx = 0; bx < NBD / 32; ++bx) {
+        const int r0 = g0 + bx * 32;
+        const BoxOut w = box_out(g, t, q, lane, r0);
+        uint32_t r[32];
+        tmem_ld32_nw(acc + (uint32_t)r0, r);
+        tmem_wait_ld(r);
+        if (r0 + 32 == BN) {  // the accumulator has been read in full
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) acc_release<PAIR>(acce_set);
         }
-      } else if constexpr (NB <= 32) {
-        float lv[32 / NBD];
-        int lp[32 / NBD];
+        if (refl) {
 #pragma unroll
-        for (int b = 0; b < 32 / NBD; ++b) {
-          const int kb0 = r0 + b * NBD;
-          const int64_t left = g.N - (t.n0 + kb0);
-          const int nact = left >= NBD ? NBD : (int)(left > 0 ? left : 0);
-          lp[b] = -1;
-          lv[b] = 0.0f;
-          if (nact < 2 || raw) {  // a one-row block is not transformed
-#pragma unroll
-            for (int l = 0; l < NBD; ++l) {
-              const float4 kq = kp[kb0 + l];
-              r[b * NBD + l] = __float_as_uint(dequant(kq, __fmaf_rn(kq.w, cwc, __uint_as_float(r[b * NBD + l])), U));
-            }
-            continue;
-          }
-          uint32_t sb = 0u;
-#pragma unroll
-          for (int l = 0; l < NBD; ++l) sb += magic_bits(__uint_as_float(r[b * NBD + l]));
-          const int S = (int)(sb - (uint32_t)NBD * kMagicBits) + cwi * msum[kb0 / NBD];
-          const int p = leads[kb0 / NBD];
-          const int Ip = magic_int(__uint_as_float(pp[b])) + (int)kp[kb0 + p].w * cwi;
-          const BlockFixF f = block_fix_f(nact == NBD ? hc : hh_const(nact), S, Ip);
-#pragma unroll
-          for (int l = 0; l < NBD; ++l) {
-            const float4 kq = kp[kb0 + l];
-            r[b * NBD + l] = __float_as_uint(dequant(kq, reflect_f(__uint_as_float(r[b * NBD + l]), kq, cwc, f), U));
-          }
-          lp[b] = b * NBD + p;
-          lv[b] = dequant(kp[kb0 + p], f.lead, U);
-        }
-        w.st32(reinterpret_cast<const float (&)[32]>(r));
-        // the lead rows: later stores of the same thread
-#pragma unroll
-        for (int b = 0; b < 32 / NBD; ++b)
-          if (lp[b] >= 0) w.st(lp[b], lv[b]);
-      } else {
-        const int64_t left = g.N - (t.n0 + g0);
-        const int nact = left >= NB ? NB : (int)(left > 0 ? left : 0);
-        if (nact < 2 || raw) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float4 kq = kp[r0 + i];
-            r[i] = __float_as_uint(dequant(kq, __fmaf_rn(kq.w, cwc, __uint_as_float(r[i])), U));
+          for (int i = 0; i < 32; i += 2) {
+            const RowPair kq = kp.pair(r0 + i);
+            set_pair(r + i, dequant2(kq, reflect2(pair_of(r + i), kq, cw2, f), U2));
           }
         } else {
-          const BlockFixF f = block_fix_f(nact == NB ? hc : hh_const(nact), S_big, Ip_big);
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float4 kq = kp[r0 + i];
-            r[i] = __float_as_uint(dequant(kq, reflect_f(__uint_as_float(r[i]), kq, cwc, f), U));
-          }
-          if (p_big >= bx * 32 && p_big < bx * 32 + 32) {
-            lead_row = p_big - bx * 32;
-            lead_val = dequant(kp[g0 + p_big], f.lead, U);
+          for (int i = 0; i < 32; i += 2) {
+            const RowPair kq = kp.pair(r0 + i);
+            set_pair(r + i, dequant2(kq, fma2(kq.m, cw2, pair_of(r + i)), U2));
           }
         }
-      }
-      if constexpr (NB == 1 || NB > 32) {
         w.st32(reinterpret_cast<const float (&)[32]>(r));
-        if (lead_row >= 0) w.st(lead_row, lead_val);
+        // the lead row: a later store of the same thread
+        if (refl && p >= bx * 32 && p < bx * 32 + 32)
+          w.st(p - bx * 32, dequant(kl, f.lead, U));
       }
     }
-  }
   }
 }
 
@@ -1077,17 +1091,18 @@ __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, u
   const ff y = two_sum((float)g.ow, zw);
   const int Cn = (int)g.K;
   TileLoads cur, nxt;
-  Item t;
-  if (cta_item<PAIR>(g, 0, t)) tile_loads<NB>(g, t, lane, cur);
-  for (int64_t local = 0; cta_item<PAIR>(g, local, t) && !*abort_flag; ++local) {
-    Item tn;
-    if (cta_item<PAIR>(g, local + 1, tn)) tile_loads<NB>(g, tn, lane, nxt);
+  Item t, tn;
+  bool have = cta_item<PAIR>(g, 0, t);
+  if (have) tile_loads<NB>(g, t, lane, cur);
+  for (int64_t local = 0; have && !*abort_flag; ++local) {
+    const bool more = cta_item<PAIR>(g, local + 1, tn);
+    if (more) tile_loads<NB>(g, tn, lane, nxt);
     const int s = (int)(local % kParStages);
     const uint32_t wrap = (uint32_t)(local / kParStages);
     const bool got = mbar_wait(&pempty[s], (wrap & 1u) ^ 1u, g.status);
     if (!__all_sync(0xffffffffu, got)) { *abort_flag = 1; break; }
     uint8_t *P = smem + kOffPar + (size_t)s * kParBytes;
-    float4 *kp = reinterpret_cast<float4 *>(P);
+    const RowPar kp{reinterpret_cast<float *>(P)};
     int *leads = reinterpret_cast<int *>(P + kParLeads);
     int *msum = reinterpret_cast<int *>(P + kParMsum);
     int *cs = reinterpret_cast<int *>(P + kParCs);
@@ -1119,7 +1134,7 @@ __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, u
           A = B = m = 0.0f;
         }
       }
-      kp[lane + 32 * i] = make_float4(sc, A, B, m);
+      kp.set(lane + 32 * i, sc, A, B, m);
       mabs = fmaxf(mabs, fabsf(m));
       mrow[i] = m;
     }
@@ -1167,7 +1182,7 @@ __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, u
     const bool raw = NB != 0 && !(mabs <= (FORM == 2 ? g.flt_mmax : g.i32_mmax));
     if (raw) {
 #pragma unroll
-      for (int i = 0; i < BN / 32; ++i) kp[lane + 32 * i] = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+      for (int i = 0; i < BN / 32; ++i) kp.set(lane + 32 * i, 1.0f, 0.0f, 0.0f, 0.0f);
       if (lane == 0 && local < kMaxLocalTiles) raw_mask[local >> 5] |= 1u << (local & 31);
     }
     // 1: the fp32 form, 2: the int32 form, 0: raw
@@ -1179,6 +1194,8 @@ __device__ __forceinline__ void gradx_params(const GemmArgs &g, uint8_t *smem, u
     __syncwarp();
     if (lane == 0) mbar_arrive(&pfull[s]);
     cur = nxt;
+    t = tn;
+    have = more;
   }
 }
 
@@ -1213,7 +1230,7 @@ __device__ __forceinline__ void gradx_epilogue(const GemmArgs &g, uint8_t *smem,
     const bool gotp = mbar_wait(&pfull[s], (uint32_t)(local / kParStages) & 1u, g.status);
     if (!__all_sync(0xffffffffu, gotp)) { ok = false; break; }
     const uint8_t *P = smem + kOffPar + (size_t)s * kParBytes;
-    const float4 *kp = reinterpret_cast<const float4 *>(P);
+    const RowPar kp{reinterpret_cast<float *>(const_cast<uint8_t *>(P))};
     const int *leads = reinterpret_cast<const int *>(P + kParLeads);
     const int *msum = reinterpret_cast<const int *>(P + kParMsum);
     const int cs = reinterpret_cast<const int *>(P + kParCs)[q * 32 + lane];
