@@ -237,21 +237,35 @@ size_t gemm_workspace_bytes(int64_t N, int64_t C, int64_t D) {
 }
 
 // Whether a contraction takes CTA pairs: p the plan of single CTAs, q that of
-// pairs.  A K block takes about the same time in either (0.41 us for a CTA's
-// 128 x 128, 0.42-0.49 us for a pair's 256 x 256, measured on reductions of
-// 1024 to 8192), so the one with clearly fewer K blocks in its longest chain
-// of waves is taken (three more per item for its start and end).  Measured,
-// 8192 tokens 1024 <-> 4096: grad_X 92 -> 57 us and 86 -> 54 us, forward 86
-// -> 55 us, grad_W 119 -> 63 us with its reduction fused.  Fewer than four K
-// blocks are bound by the output's stores, where the pair has nothing to
-// give.
-static bool pair_faster(const SplitPlan &p, const SplitPlan &q, int num_sms) {
+// pairs.  A K block takes about 0.4 us in either (128 x 128 for a CTA, 256 x
+// 256 for a pair), so the one with clearly fewer K blocks in its longest
+// chain of waves is taken.  Measured, 8192 tokens 1024 <-> 4096: grad_X 92 ->
+// 57 us and 86 -> 54 us, forward 86 -> 55 us, grad_W 119 -> 63 us with its
+// reduction fused.
+// grad_X and the forward: below `min_kb` K blocks per tile the epilogue and
+// its stores bound both, which a pair does not speed up: four with the fp32
+// form (50176 x 256 x 2304: 130 -> 122 us), eight with the int32 one (53910 x
+// 352 x 400, six K blocks: 86.6 -> 90.1 us).
+static bool pair_faster(const SplitPlan &p, const SplitPlan &q, int num_sms, int min_kb) {
+  const int64_t one = ((int64_t)p.m_tiles * p.n_tiles + num_sms - 1) / num_sms;
+  const int64_t two = ((int64_t)q.m_tiles * q.n_tiles + num_sms / 2 - 1) / (num_sms / 2);
+  return q.kb_total >= min_kb && 10 * two * (q.ks_blocks + 3) < 9 * one * (p.ks_blocks + 3);
+}
+
+// grad_W: a pair's item costs about 12 us beside its K blocks (a CTA's 5: the
+// pair drains 128 x 256 sums per CTA), and every split writes and reads back
+// its partials; the pair has to be ahead by 15% (53910 x 352 x 400, 19 splits
+// of 45 K blocks against 12 of 71: 37.3 us against 41.1 with its reduction).
+static bool pair_faster_w(const SplitPlan &p, const SplitPlan &q, int64_t C, int64_t D,
+                          int num_sms) {
   const int64_t one = ((int64_t)p.m_tiles * p.n_tiles * p.splits + num_sms - 1) / num_sms;
   const int64_t two =
       ((int64_t)q.m_tiles * q.n_tiles * q.splits + num_sms / 2 - 1) / (num_sms / 2);
-  // short splits: the partials and their reduction outweigh the contraction
-  if (q.splits > 1 && q.ks_blocks < 16) return false;
-  return q.kb_total >= 4 && 10 * two * (q.ks_blocks + 3) < 9 * one * (p.ks_blocks + 3);
+  const double red = (double)C * (double)D * 8.0 / 5000.0;  // ns per split
+  const double t1 = (double)one * (410.0 * (double)p.ks_blocks + 5000.0) + red * p.splits;
+  const double t2 =
+      (double)two * (400.0 * (double)q.ks_blocks + 12000.0) + (q.splits > 1 ? red * q.splits : 0.0);
+  return t2 < 0.85 * t1;
 }
 
 // The kernel instance of a mode, BHQ block size (1 = no reflection) and
@@ -900,7 +914,7 @@ fqt_status linear_forward(const fqt_qtensor *qx, const fqt_qtensor *qw, float *H
   g.flt_mmax = flt ? (float)mmax : -1.0f;
   g.i32_mmax = int32_form_mmax(D, qw->bits, qx->bits, 1);
   const SplitPlan pp = plan_splits(C, Nr, D, qw->bits, qx->bits, nsm, false, true);
-  const bool pair = flt && pair_faster(p, pp, nsm);
+  const bool pair = flt && pair_faster(p, pp, nsm, 4);
   return run_gemm(qw->codes_f16, 1, qw->bits, qx->codes_f16, 1, qx->bits, C, Nr, D,
                   pair ? pp : p, g, H, MODE_GRADX, 1, epilogue_form(flt, mmax, qx->bits), st,
                   pair);
@@ -1373,7 +1387,7 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
       const SplitPlan pp = plan_splits(D, Nr, C, qw->bits, q_b2->bits, nsm, false, true);
       const int form = adapt ? 2 : epilogue_form(flt, mmax, q_b2->bits);
       const bool pair = C <= kc_terms && gemm_pair_kernel(MODE_GRADX, nb, form) &&
-                        pair_faster(p, pp, nsm);
+                        pair_faster(p, pp, nsm, form == 2 ? 4 : 8);
       fqt_status s = run_gemm(qw->codes_f16, 0, qw->bits, q_b2->codes_f16, 1, q_b2->bits,
                               D, Nr, C, pair ? pp : p, g, grad_X, MODE_GRADX, nb, form, st, pair);
       if (s != FQT_OK) return s;
@@ -1499,7 +1513,7 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
     bool pair = false;
     if (Nr > 0 && !w_ok && !bytes && C > BM) {
       const SplitPlan pp = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true, true);
-      pair = pair_faster(p, pp, nsm) &&
+      pair = pair_faster_w(p, pp, C, D, nsm) &&
              (int64_t)kGemmOffset + pp.splits * C * D * 4 + pad_bytes <= (int64_t)ws_bytes;
       if (pair) p = pp;
     }
