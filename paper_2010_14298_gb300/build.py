@@ -1,7 +1,8 @@
 """Builds the CUDA library paper_2010_14298_gb300/_lib/libfqt.so for sm_103a.
 
 Each translation unit is compiled by nvcc in parallel, then linked into one
-shared object with a plain C ABI (include/fqt.h).  Run as a script or call
+shared object with a plain C ABI (include/fqt.h); the Python binding's native
+marshalling (csrc/fqt_py.c) is a small extension module linked against it.  Run as a script or call
 ``build()``; an up-to-date library is not rebuilt.
 """
 from __future__ import annotations
@@ -11,6 +12,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -18,6 +20,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libfqt.so")
+PYEXT = os.path.join(LIBDIR, "_fqt_py.so")
 SOURCES = ["fqt_quant.cu", "fqt_codes.cu", "fqt_group.cu", "fqt_gemm.cu", "fqt_gemm_pair.cu", "fqt_conv.cu",
            "fqt_api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -35,16 +38,16 @@ def _nvcc() -> str:
 def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
     files += [os.path.join(CSRC, f) for f in os.listdir(CSRC)
-              if f.endswith((".cuh", ".h"))]
+              if f.endswith((".cuh", ".h", ".c"))]
     files.append(os.path.join(INCLUDE, "fqt.h"))
     files.append(os.path.abspath(__file__))
     return files
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYEXT):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYEXT))
     return all(os.path.getmtime(f) <= t for f in _inputs())
 
 
@@ -75,6 +78,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+    tmp = PYEXT + f".tmp{os.getpid()}"
+    cmd = [shutil.which("gcc") or "gcc", "-O2", "-std=c11", "-shared", "-fPIC",
+           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+           os.path.join(CSRC, "fqt_py.c"), "-o", tmp, "-L", LIBDIR, "-l:libfqt.so",
+           "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"building the Python extension failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, PYEXT)
     return LIB
 
 
