@@ -66,13 +66,13 @@ static fqt_status quantize_forward(const void *X, fqt_dtype dtype, int64_t rows,
   float2 *part = reinterpret_cast<float2 *>(w + kRangeOffset);
   int npart = 0;
   cudaError_t e = launch_range(X, dtype == FQT_BF16, rows * cols, part, &npart,
-                               out->col_sum, out->col_sum ? cols : 0, nullptr, 0,
-                               nsm, st);
+                               out->col_sum, out->col_sum ? cols : 0, out->row_sum,
+                               out->row_sum ? rows : 0, nsm, st);
   if (e != cudaSuccess) return cuda_fail(e, "range pass");
-  if (!out->row_sum && cols / 8 <= 1024)
+  if (cols / 8 <= 1024 && (!out->row_sum || fwd_codes_row_sums((int)cols)))
     return launch_fwd_codes(X, dtype == FQT_BF16, rows, (int)cols, bits, out->codes_f16,
                             out->codes, out->col_sum, part, npart, out->inv_s, out->zero,
-                            reinterpret_cast<int *>(w), nsm, st);
+                            reinterpret_cast<int *>(w), nsm, st, 0, nullptr, out->row_sum);
   QuantArgs a;
   memset(&a, 0, sizeof(a));
   a.h = X;

@@ -66,7 +66,8 @@ fqt_status launch_fwd_codes(const void *X, bool bf16, int64_t rows, int cols, in
                             uint16_t *f16, uint8_t *c8, int32_t *col_sum, const float2 *part,
                             int npart, float *inv_out, float *zero_out, int *status,
                             int num_sms, cudaStream_t st, int conv_zero = 0,
-                            int32_t *code_zero_out = nullptr);
+                            int32_t *code_zero_out = nullptr, int32_t *row_sum = nullptr);
+bool fwd_codes_row_sums(int cols);
 fqt_status launch_conv_colsum(const uint16_t *f16, int64_t n, int h, int w, int c, int kh,
                               int kw, int pad, int bits, int32_t *col_sum, cudaStream_t st);
 // border sums of 3 x 3, pad 1 conv operands (fqt_conv.cu)

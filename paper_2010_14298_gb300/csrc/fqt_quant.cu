@@ -1120,13 +1120,13 @@ fqt_status launch_shift(QuantArgs &a, bool bf16, int num_sms, cudaStream_t st) {
 constexpr int kFwdUnroll = 4;
 constexpr int kFwdMaxThreads = 1024;
 
-template <typename T>
+template <typename T, bool ROWS>
 __global__ void __launch_bounds__(kFwdMaxThreads)
     k_fwd_codes(const T *__restrict__ X, int64_t rows, int cols, int rpi,
                 uint16_t *__restrict__ f16, uint8_t *__restrict__ c8,
                 int32_t *__restrict__ col_sum, const float2 *__restrict__ part, int npart,
                 float *inv_out, float *zero_out, int bits, int *status, int conv_zero,
-                int32_t *code_zero_out) {
+                int32_t *code_zero_out, int32_t *__restrict__ row_sum) {
   extern __shared__ int csum_s[];  // cols
   __shared__ float2 red[kFwdMaxThreads / 32];
   __shared__ int redi[kFwdMaxThreads / 32];
@@ -1210,6 +1210,17 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
       const int64_t e = row[u] * cols + o * 8;
       if (f16) store_carriers8(f16 + e, c, off);
       if (c8) store_codes8(c8 + e, c);
+      if constexpr (ROWS) {
+        // the lanes of a row add up first (whole warps of one row, or rows of
+        // a power of two of lanes); the range pass cleared the sums
+        int v = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v += (int)c[j];
+        const unsigned act = __activemask();
+        const int span = min(opr, 32);
+        for (int d = 1; d < span; d <<= 1) v += __shfl_xor_sync(act, v, d);
+        if ((lane & (span - 1)) == 0) atomicAdd(&row_sum[row[u]], v);
+      }
     }
   }
   if (col_sum) {
@@ -1224,30 +1235,42 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
   }
 }
 
+// Row sums in the code pass: rows of whole warps, or of a power of two of lanes.
+bool fwd_codes_row_sums(int cols) {
+  const int opr = cols / 8;
+  return cols % 8 == 0 && opr <= kFwdMaxThreads && (opr % 32 == 0 || !(opr & (opr - 1)));
+}
+
 fqt_status launch_fwd_codes(const void *X, bool bf16, int64_t rows, int cols, int bits,
                             uint16_t *f16, uint8_t *c8, int32_t *col_sum, const float2 *part,
                             int npart, float *inv_out, float *zero_out, int *status,
                             int num_sms, cudaStream_t st, int conv_zero,
-                            int32_t *code_zero_out) {
+                            int32_t *code_zero_out, int32_t *row_sum) {
   const int opr = cols / 8;
   if (cols % 8 || opr > kFwdMaxThreads) return FQT_EUNSUPPORTED;
   int rpi = 512 / opr;  // about 512 threads: two CTAs per SM
   if (rpi < 1) rpi = 1;
   const int nth = ((rpi * opr + 31) / 32) * 32;
   const int64_t groups = (rows + rpi - 1) / rpi;
-  int64_t grid = (int64_t)num_sms * (kFwdMaxThreads * 2 / nth >= 2 ? 2 : 1) * 4;
+  // every CTA adds its column sums once: four waves of CTAs even out the tail
+  // of narrow rows, but at 4096 columns their atomics cost more than the codes
+  // (8192 x 4096 bf16: 37 us with four, 30 with one)
+  int64_t grid = (int64_t)num_sms * (kFwdMaxThreads * 2 / nth >= 2 ? 2 : 1) *
+                 (cols >= 1024 ? 1 : 4);
   const int64_t need = (groups + kFwdUnroll - 1) / kFwdUnroll;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
   const size_t smem = (size_t)cols * sizeof(int);
-  if (bf16)
-    k_fwd_codes<__nv_bfloat16><<<(int)grid, nth, smem, st>>>(
-        reinterpret_cast<const __nv_bfloat16 *>(X), rows, cols, rpi, f16, c8, col_sum, part,
-        npart, inv_out, zero_out, bits, status, conv_zero, code_zero_out);
-  else
-    k_fwd_codes<float><<<(int)grid, nth, smem, st>>>(
-        reinterpret_cast<const float *>(X), rows, cols, rpi, f16, c8, col_sum, part, npart,
-        inv_out, zero_out, bits, status, conv_zero, code_zero_out);
+  auto launch = [&](auto kern, auto *x) {
+    kern<<<(int)grid, nth, smem, st>>>(x, rows, cols, rpi, f16, c8, col_sum, part, npart, inv_out,
+                                       zero_out, bits, status, conv_zero, code_zero_out, row_sum);
+  };
+  const auto *xb = reinterpret_cast<const __nv_bfloat16 *>(X);
+  const auto *xf = reinterpret_cast<const float *>(X);
+  if (bf16 && row_sum) launch(k_fwd_codes<__nv_bfloat16, true>, xb);
+  else if (bf16) launch(k_fwd_codes<__nv_bfloat16, false>, xb);
+  else if (row_sum) launch(k_fwd_codes<float, true>, xf);
+  else launch(k_fwd_codes<float, false>, xf);
   return cuda_fail(cudaGetLastError(), "forward codes launch");
 }
 

@@ -69,3 +69,17 @@ def test_small_workspace_takes_the_one_pass_quantizer(c, kind, block):
     ws = fqt.Workspace(1, 16, 16)
     ws.nbytes = 256 + 32768  # the header and the range partials
     _check(200, c, kind, 5, block, "f32", ws)
+
+
+@pytest.mark.parametrize("rows,cols", [(5, 8), (67, 16), (200, 64), (33, 128), (70, 256),
+                                       (41, 768), (9, 8192), (50, 24), (50, 1104)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_forward_row_sums(rows, cols, dtype):
+    g = wl.rng(rows + cols)
+    X = g.standard_normal((rows, cols)).astype(np.float32)
+    X = wl.to_bf16_values(X) if dtype == "bf16" else X
+    q = fqt.quantize_act(to_dev(X, dtype), 8, row_sum=True)
+    codes = q.to_numpy()["codes"].astype(np.int64)
+    assert np.array_equal(codes, orc.quantize_fwd(X, 8)["codes"])
+    assert np.array_equal(q.row_sum.cpu().numpy(), codes.sum(1))
+    assert np.array_equal(q.col_sum.cpu().numpy(), codes.sum(0))
