@@ -349,6 +349,14 @@ __device__ __forceinline__ float ll_to_float(long long v) {
   return __ll2float_rn(v);
 }
 
+// ll_to_float for |v| < 2^45 without a conversion instruction: v = a 2^23 + b
+// with both parts read off the bits of fp32 numbers of known exponent.
+__device__ __forceinline__ float i45_to_float(long long v) {
+  const float a = __fsub_rn(__int_as_float(0x4B400000 + (int)(v >> 23)), 12582912.0f);
+  const float b = __fsub_rn(__int_as_float(0x4B000000 | (int)(v & 0x7FFFFF)), 8388608.0f);
+  return __fmaf_rn(a, 8388608.0f, b);
+}
+
 // An int32 as float-float, exactly, with 32-bit conversions only.
 __device__ __forceinline__ ff ff_from_i32s(int v) {
   const float h = __int2float_rn(v);

@@ -38,12 +38,19 @@ namespace fqt {
 // ---------------------------------------------------------------------------
 // Split-K reduction (int64) and the grad_W / raw epilogues
 // ---------------------------------------------------------------------------
-// A thread sums four consecutive outputs of one row over all splits (one
-// 16-byte load per split, coalesced across the warp, two splits in flight)
-// and dequantizes them (r.vec; else one output per thread).
-constexpr int kRedThreads = 256;
+// A thread sums four consecutive outputs of one row (r.vec; else one output)
+// over every `groups`-th split, one 16-byte load per split, coalesced across
+// the warp and four in flight; the groups of an output meet in shared memory
+// and the first dequantizes.  Few outputs with many splits were a chain of
+// loads in a handful of CTAs: 256 x 64 over 76 splits 11.2 us with one group,
+// 5.6 with eight; 112 x 80 over 152 splits 16.6 -> 6.2 us; 1008 x 2048 in one
+// split (no 64-bit division or conversion per output) 12.0 -> 9.4 us.  With
+// two groups and few splits the meeting costs more than it hides (1200 x 336
+// over 5: 5.4 us with one group, 7.2 with two).
+constexpr int kRedThreads = 256, kRedGroups = 8;
 
-__global__ void __launch_bounds__(kRedThreads) k_reduce(const ReduceArgs r) {
+__global__ void __launch_bounds__(kRedThreads) k_reduce(const ReduceArgs r, int groups) {
+  __shared__ long long part_s[kRedThreads][4];
   const int64_t total = r.M * r.N;
   const bool vec = r.vec != 0;
   const int W = vec ? 4 : 1;
@@ -61,36 +68,56 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const ReduceArgs r) {
   // centred product P (ca, cb the code column sums)
   const int64_t ka = r.oa - ma, kb = ob - mb;
   const int64_t k0 = r.Kn * ka * kb - ka * r.Kn * ob - kb * r.Kn * r.oa;
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t idx = u * W;
+  const int upc = kRedThreads / groups;  // units per CTA and step
+  const int ul = (int)threadIdx.x & (upc - 1), grp = (int)threadIdx.x / upc;
+  for (int64_t u0 = (int64_t)blockIdx.x * upc; u0 < units; u0 += (int64_t)gridDim.x * upc) {
+    const int64_t u = u0 + ul, idx = u * W;
     long long P[4] = {0, 0, 0, 0};
-    if (vec) {
+    if (u < units && vec) {
       const int4 *src = reinterpret_cast<const int4 *>(r.part + idx);
       const int64_t step = total >> 2;
-      int sp = 0;
-      for (; sp + 1 < r.splits; sp += 2) {
-        const int4 x = __ldcs(src + (int64_t)sp * step), y = __ldcs(src + (int64_t)(sp + 1) * step);
-        P[0] += (long long)x.x + y.x;
-        P[1] += (long long)x.y + y.y;
-        P[2] += (long long)x.z + y.z;
-        P[3] += (long long)x.w + y.w;
+      int sp = grp;
+      for (; sp + 3 * groups < r.splits; sp += 4 * groups) {
+        int4 x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] = __ldcs(src + (int64_t)(sp + i * groups) * step);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          P[0] += x[i].x;
+          P[1] += x[i].y;
+          P[2] += x[i].z;
+          P[3] += x[i].w;
+        }
       }
-      if (sp < r.splits) {
+      for (; sp < r.splits; sp += groups) {
         const int4 x = __ldcs(src + (int64_t)sp * step);
         P[0] += x.x;
         P[1] += x.y;
         P[2] += x.z;
         P[3] += x.w;
       }
-    } else {
-      for (int sp = 0; sp < r.splits; ++sp) P[0] += __ldcs(r.part + (int64_t)sp * total + idx);
+    } else if (u < units) {
+      for (int sp = grp; sp < r.splits; sp += groups)
+        P[0] += __ldcs(r.part + (int64_t)sp * total + idx);
     }
+    if (groups > 1) {
+      __syncthreads();  // the last step's sums are read
+#pragma unroll
+      for (int i = 0; i < 4; ++i) part_s[threadIdx.x][i] = P[i];
+      __syncthreads();
+      if (grp == 0)
+        for (int g = 1; g < groups; ++g)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) P[i] += part_s[g * upc + ul][i];
+    }
+    if (grp != 0 || u >= units) continue;
     if (!deq) {
       for (int i = 0; i < W; ++i) r.out_i64[idx + i] = P[i];
       continue;
     }
-    const int64_t c = idx / r.N, d0 = idx - c * r.N;
+    const int64_t c = total < ((int64_t)1 << 32) ? (int64_t)((uint32_t)idx / (uint32_t)r.N)
+                                                 : idx / r.N;
+    const int64_t d0 = idx - c * r.N;
     const int64_t ca = r.cs_a[c];
     // row term db (ca - Kn ma) of this thread's row
     const float rt = db * ll_to_float(ca - r.Kn * ma);
@@ -100,9 +127,11 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const ReduceArgs r) {
       const int64_t d = d0 + i;
       const int64_t cb = r.cs_b[d];
       long long Pi = P[i];
-      if (r.pad_a) Pi += code_pad * r.pad_a[d / r.cin * r.M + c];
+      if (r.pad_a) Pi += code_pad * r.pad_a[(int64_t)((uint32_t)d / (uint32_t)r.cin) * r.M + c];
       const int64_t I = Pi + ka * cb + Ia;
-      o[i] = sab * (ll_to_float(I) + rt + da * ll_to_float(cb - r.Kn * mb) + kdd);
+      const float f = (uint64_t)(I + ((int64_t)1 << 44)) < ((uint64_t)1 << 45) ? i45_to_float(I)
+                                                                               : ll_to_float(I);
+      o[i] = sab * (f + rt + da * ll_to_float(cb - r.Kn * mb) + kdd);
     }
     if (vec)
       *reinterpret_cast<float4 *>(r.out_f32 + idx) = make_float4(o[0], o[1], o[2], o[3]);
@@ -472,11 +501,16 @@ static void launch_reduce(ReduceArgs r, cudaStream_t st) {
   auto a16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
   r.vec = (r.N & 3) == 0 && a16(r.part) && (r.out_i64 || a16(r.out_f32));
   const int64_t units = r.vec ? total >> 2 : total;
-  int64_t grid = (units + kRedThreads - 1) / kRedThreads;
-  const int64_t cap = (int64_t)device_sm_count() * 8;
+  // groups of splits until the GPU has about 512 threads per SM
+  const int64_t nsm = device_sm_count();
+  int groups = 1;
+  while (groups < kRedGroups && groups * 2 <= r.splits && units * groups < nsm * 512) groups *= 2;
+  const int64_t upc = kRedThreads / groups;
+  int64_t grid = (units + upc - 1) / upc;
+  const int64_t cap = nsm * 8;
   if (grid > cap) grid = cap;
   if (grid < 1) grid = 1;
-  k_reduce<<<(int)grid, kRedThreads, 0, st>>>(r);
+  k_reduce<<<(int)grid, kRedThreads, 0, st>>>(r, groups);
 }
 
 static size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }

@@ -1607,14 +1607,6 @@ __device__ __forceinline__ void issue_pair(const GemmArgs &g, uint8_t *ops, uint
   mbar_wait(drain, 0, g.status);
 }
 
-// ll_to_float for |v| < 2^45 without a conversion instruction: v = a 2^23 + b
-// with both parts read off the bits of fp32 numbers of known exponent.
-__device__ __forceinline__ float i45_to_float(long long v) {
-  const float a = __fsub_rn(__int_as_float(0x4B400000 + (int)(v >> 23)), 12582912.0f);
-  const float b = __fsub_rn(__int_as_float(0x4B000000 | (int)(v & 0x7FFFFF)), 8388608.0f);
-  return __fmaf_rn(a, 8388608.0f, b);
-}
-
 // Split-K partials of a pair: set h (warps 4 h ..) owns the 128 columns of
 // half h; a thread keeps its row's 128 int32 running sums in registers, adds
 // each exact chunk to them and at the end stores four 32 x 32 boxes, the
