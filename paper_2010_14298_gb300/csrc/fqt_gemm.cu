@@ -224,6 +224,45 @@ static SplitPlan plan_splits(int64_t M, int64_t N, int64_t K, int a_bits,
   return p;
 }
 
+// The plan of k_gemm_wide: the tile width (128, 192 or 256 columns) whose waves
+// take least, or `fixed` columns.  A K block takes 0.25 to 0.4 us (0.3 of 192
+// columns where one copy serves the taps of a kernel row), an item 8 us beside
+// them (its 128 x 256 sums).
+static double wide_plan(int64_t M, int64_t N, int64_t K, int a_bits, int b_bits, int num_sms,
+                        int fixed, SplitPlan *best, int *wn) {
+  double least = 1e300;
+  for (int w = fixed ? fixed : 128; w <= (fixed ? fixed : 256); w += 64) {
+    SplitPlan p;
+    p.m_tiles = (int)((M + BM - 1) / BM);
+    p.n_tiles = (int)((N + w - 1) / w);
+    p.kb_total = std::max<int64_t>(1, (K + BK - 1) / BK);
+    const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles;
+    int64_t splits = std::max<int64_t>(1, num_sms / tiles);
+    const int64_t max_terms = ((int64_t)1 << 31) >> (a_bits + b_bits - 2);
+    splits = std::max(splits, (K + max_terms - 1) / max_terms);
+    splits = std::min(splits, p.kb_total);
+    p.ks_blocks = (p.kb_total + splits - 1) / splits;
+    p.splits = (int)((p.kb_total + p.ks_blocks - 1) / p.ks_blocks);
+    const int64_t waves = (tiles * p.splits + num_sms - 1) / num_sms;
+    const double t = (double)waves * ((double)p.ks_blocks * ((fixed ? 60.0 : 100.0) + 1.2 * w) + 8000.0) +
+                     (double)M * (double)N * 8.0 / 5000.0 * p.splits;
+    if (t < least) {
+      least = t;
+      *best = p;
+      *wn = w;
+    }
+  }
+  return least;
+}
+
+// The single-CTA plan's time on the same scale.
+static double single_time(const SplitPlan &p, int64_t M, int64_t N, int num_sms) {
+  const int64_t waves =
+      ((int64_t)p.m_tiles * p.n_tiles * p.splits + num_sms - 1) / num_sms;
+  return (double)waves * (410.0 * (double)p.ks_blocks + 5000.0) +
+         (double)M * (double)N * 8.0 / 5000.0 * p.splits;
+}
+
 // The k_gradw plan for grad_W of C x D over K rows, or splits = 0 when the
 // shape does not fit it.
 struct WPlan {
@@ -258,6 +297,15 @@ size_t gemm_workspace_bytes(int64_t N, int64_t C, int64_t D) {
     // CTA pairs (more than 128 rows of grad_W)
     const int64_t s2 = C > BM ? plan_splits(C, D, Kp, b, 8, nsm, true, true).splits : 0;
     if (s2 > sp) sp = s2;
+    if (C <= BM && D > BN) {
+      SplitPlan wp;
+      int wn;
+      for (const int64_t K : {N, Kp})  // the widest tiles have the most splits
+        for (const int fixed : {0, 2 * BN}) {
+          wide_plan(C, D, K, b, 8, nsm, fixed, &wp, &wn);
+          if (wp.splits > sp) sp = wp.splits;
+        }
+    }
     if (sp > splits) splits = sp;
   }
   // + the padding table of an implicit im2col X~ (C x taps, taps <= D)
@@ -348,7 +396,7 @@ static GemmKernel gemm_kernel(int mode, int nb, int form) {
 static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *Bm,
                            int b_kmajor, int b_bits, int64_t M, int64_t N, int64_t K,
                            const SplitPlan &p, GemmArgs &g, void *out, int mode, int nb,
-                           int form, cudaStream_t st, bool pair = false) {
+                           int form, cudaStream_t st, bool pair = false, int wide = 0) {
   const bool partial = mode == MODE_PARTIAL;
   // byte operands (g.u8): split-K partials of MN-major operands only
   if (g.u8 && (!partial || a_kmajor || b_kmajor)) return FQT_EUNSUPPORTED;
@@ -364,7 +412,8 @@ static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *
     ok = make_map_f16_box4(&ta, A, (uint64_t)g.cnimg, (uint64_t)g.coh, (uint64_t)g.cow,
                            (uint64_t)M, (uint32_t)g.cpw, (uint32_t)g.crpb) &&
          make_map_f16_box4(&tb, Bm, (uint64_t)g.cnimg, (uint64_t)g.cih, (uint64_t)g.ciw,
-                           (uint64_t)g.cin, (uint32_t)g.cpw, (uint32_t)g.crpb);
+                           (uint64_t)g.cin, (uint32_t)(g.cpw + (g.taps ? g.taps - 1 : 0)),
+                           (uint32_t)g.crpb);
   } else {
     ok = a_kmajor ? make_map_f16(&ta, A, (uint64_t)K, (uint64_t)M, BK, BM)
                   : make_map_f16(&ta, A, (uint64_t)M, (uint64_t)K, 64, BK);
@@ -451,6 +500,24 @@ static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *
   g.ks_blocks = p.ks_blocks;
   g.kb_total = p.kb_total;
   g.n_items = (int64_t)p.m_tiles * p.n_tiles * p.splits;
+  if (wide) {  // k_gemm_wide: the threads and registers of a pair's partials
+    g.wn = wide;
+    g.stages = kMaxStages;
+    uint32_t bb = (uint32_t)(g.taps ? g.crpb * (g.cpw + g.taps - 1) : wide) * 128u;
+    bb = (bb + 1023u) & ~1023u;
+    while (g.stages > 2 && gemm_wide_smem(bb, g.stages) > 227 * 1024) --g.stages;
+    const size_t smem = gemm_wide_smem(bb, g.stages);
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, k_gemm_wide);
+    if (e != cudaSuccess) return cuda_fail(e, "wide gemm attributes");
+    if (fa.numRegs * LP::threads < 128 * LP::regs_ctl + 256 * LP::regs_epi)
+      return FQT_EUNSUPPORTED;
+    e = cudaFuncSetAttribute(k_gemm_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(e, "wide gemm shared-memory attribute");
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(g.n_items, device_sm_count()));
+    k_gemm_wide<<<(int)grid, LP::threads, smem, st>>>(ta, tb, to, g);
+    return cuda_fail(cudaGetLastError(), "wide gemm launch");
+  }
   const size_t smem = gemm_smem_bytes(g.stages, g.ring, g.ustages);
   const cudaError_t ea =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1551,8 +1618,31 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
              (int64_t)kGemmOffset + pp.splits * C * D * 4 + pad_bytes <= (int64_t)ws_bytes;
       if (pair) p = pp;
     }
-    // one split: the pair's epilogue dequantizes, no partials and no reduction
-    const bool fuse = pair && p.splits == 1 && !conv && aligned16(grad_W);
+    // At most one tile of rows: wide tiles, where their plan is ahead by 10%
+    // and its partials fit; an implicit im2col operand of kw = 2 to 4 taps a
+    // row then reads its pixels once per kernel row.  An explicit operand is
+    // read from HBM, which both plans wait for (64 x 576 over 131072 rows: 41
+    // and 42 us).
+    int wide = 0, row_taps = 0;
+    if (Nr > 0 && !w_ok && !bytes && C <= BM && D > BN) {
+      SplitPlan wp;
+      int wn;
+      row_taps = conv && qx->conv[5] >= 2 && qx->conv[5] <= 4 ? qx->conv[5] : 0;
+      double t = wide_plan(C, D, Kt, a_bits, x_bits, nsm, 64 * row_taps, &wp, &wn);
+      double ts = single_time(p, C, D, nsm);
+      if (!conv) {
+        const double mem = (double)Kt * (double)(C + D) * 2.0 / 6500.0;
+        t = std::max(t, mem + 8000.0);
+        ts = std::max(ts, mem + 5000.0);
+      }
+      if (t < 0.9 * ts &&
+          (int64_t)kGemmOffset + wp.splits * C * D * 4 + pad_bytes <= (int64_t)ws_bytes) {
+        wide = wn;
+        p = wp;
+      }
+    }
+    // one split: the epilogue dequantizes, no partials and no reduction
+    const bool fuse = (pair || wide) && p.splits == 1 && !conv && aligned16(grad_W);
     const int splits = w_ok ? wp.splits : p.splits;
     const size_t pbytes = (size_t)splits * (size_t)C * (size_t)D * 4;
     const int taps = conv ? qx->conv[4] * qx->conv[5] : 0;
@@ -1623,6 +1713,7 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
       if (conv_tile) {
         const int32_t *cv = qx->conv;
         g.conv = 1;
+        g.taps = wide ? row_taps : 0;
         g.cpw = cpw;
         g.crpb = crpb;
         g.cybi = cybi;
@@ -1638,7 +1729,7 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
       g.fuse = fuse ? 1 : 0;
       g.red = r;
       fqt_status s = run_gemm(A16, 0, a_bits, X16, 0, qx->bits, C, D, Kt, p, g,
-                              fuse ? (void *)grad_W : (void *)part, MODE_PARTIAL, 1, 0, st, pair);
+                              fuse ? (void *)grad_W : (void *)part, MODE_PARTIAL, 1, 0, st, pair, wide);
       if (s != FQT_OK) return s;
       if (fuse) return FQT_OK;
     } else {

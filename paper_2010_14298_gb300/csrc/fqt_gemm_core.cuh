@@ -151,8 +151,10 @@ struct GemmArgs {
   // read as 4-D boxes of (64 channels, pw, rpb, 1)
   int conv, cpw, crpb, cybi, coh, cih, cin, ckw, cpad, cow, ciw;
   int64_t cnimg;
-  // a pair's partials with one split: grad_W itself (red) instead of partials
+  // a pair's (a wide tile's) partials with one split: grad_W itself (red)
   int fuse;
+  int wn;                      // columns of a wide tile (k_gemm_wide)
+  int taps;                    // its column atoms are the taps of a kernel row (0: consecutive)
   ReduceArgs red;
   int *status;
 };
@@ -509,6 +511,16 @@ __device__ __forceinline__ bool cta_item(const GemmArgs &g, int64_t local, Item 
     t = decode_item(g, it);
     return true;
   }
+}
+
+// The tiles of a CTA of k_gemm_wide: items of 128 x g.wn, as two column halves
+// (local = 2 item + half, the second from column 128 on).
+__device__ __forceinline__ bool wide_item(const GemmArgs &g, int64_t local, Item &t) {
+  const int64_t it = (int64_t)blockIdx.x + (local >> 1) * (int64_t)gridDim.x;
+  if (it >= g.n_items) return false;
+  t = decode_item(g, it);
+  t.n0 = t.n0 / BN * g.wn + (local & 1) * BN;
+  return true;
 }
 
 // The accumulator's consumer is done with it: the pair's MMA issuer (the
@@ -1615,6 +1627,8 @@ __device__ __forceinline__ void issue_pair(const GemmArgs &g, uint8_t *ops, uint
 // took 9 of the 60.5 us of 1024 x 4096 over 8192 rows, now 2.)
 // Column terms of a super tile in shared memory: ka cb (int64) and cb - Kn mb
 // (fp32) per column, written by the 256 threads together.
+// WIDE: the same for k_gemm_wide (columns past g.wn are not stored).
+template <bool WIDE>
 __device__ __forceinline__ void partial_epilogue_pair(const GemmArgs &g, uint8_t *smem,
                                                       uint8_t *ring, uint64_t *accf,
                                                       uint64_t *acce, uint32_t tmem,
@@ -1646,7 +1660,8 @@ __device__ __forceinline__ void partial_epilogue_pair(const GemmArgs &g, uint8_t
   bool stored = false;
   Item t;
   // the same trip count in all eight warps (they meet at named barriers)
-  for (int64_t local = 0; cta_item<true>(g, local + h, t); local += 2) {
+  for (int64_t local = 0; WIDE ? wide_item(g, local + h, t) : cta_item<true>(g, local + h, t);
+       local += 2) {
     dead = dead || *abort_flag;
     float rt = 0.0f;
     int64_t Ia = 0;
@@ -1698,7 +1713,7 @@ __device__ __forceinline__ void partial_epilogue_pair(const GemmArgs &g, uint8_t
         if (grp == BN / 32 - 1) {  // the accumulator has been read in full
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) acc_release<true>(&acce[buf]);
+          if (lane == 0) acc_release<!WIDE>(&acce[buf]);
         }
 #pragma unroll
         for (int j = 0; j < 32; ++j)
@@ -1711,6 +1726,7 @@ __device__ __forceinline__ void partial_epilogue_pair(const GemmArgs &g, uint8_t
     }
 #pragma unroll
     for (int grp = 0; grp < BN / 32; ++grp) {
+      if (WIDE && h * BN + grp * 32 >= g.wn) break;
       uint32_t o[32];
       if (g.fuse) {
         const int c0 = h * BN + grp * 32;
@@ -1741,7 +1757,13 @@ __device__ __forceinline__ void partial_epilogue_pair(const GemmArgs &g, uint8_t
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0 && t.m0 < g.M && t.n0 < g.N) {
-        tma_store_3d(tmOut, (int32_t)(t.n0 + grp * 32), (int32_t)(t.m0 + q * 32), t.split, box);
+        int32_t col = (int32_t)(t.n0 + grp * 32);
+        if (WIDE && g.taps) {  // tile = (kernel row, 64 channels), atom = tap of the row
+          const int j = h * BN + grp * 32, tile = (int)(t.n0 - h * BN) / g.wn;
+          const int gpr = g.cin / 64, ky = tile / gpr;
+          col = (ky * g.taps + j / 64) * g.cin + (tile - ky * gpr) * 64 + j % 64;
+        }
+        tma_store_3d(tmOut, col, (int32_t)(t.m0 + q * 32), t.split, box);
         bulk_commit();
       }
       stored = true;
@@ -1867,7 +1889,7 @@ __global__ void __launch_bounds__(GemmLayout<MODE, FORM, NB, PAIR>::threads, 1)
       }
     }
     else if constexpr (PAIR)
-      partial_epilogue_pair(g, smem, ring, accf, acce, tmem, &tmOut, abort_flag, warp, lane);
+      partial_epilogue_pair<false>(g, smem, ring, accf, acce, tmem, &tmOut, abort_flag, warp, lane);
     else if (warp < kGemmWarpEpi0 + kPartialEpiWarps)
       partial_epilogue(g, ring, accf, acce, tmem, &tmOut, abort_flag, warp, lane);
     else if (u8ops)  // the four warps after the partial epilogue
@@ -2420,6 +2442,13 @@ inline bool aligned16(const void *p) {
 }
 
 typedef void (*GemmKernel)(CUtensorMap, CUtensorMap, CUtensorMap, GemmArgs);
+
+// Split-K partials of one or two 64-row atoms of A against up to 256 columns
+// of B (fqt_gemm_pair.cu).
+size_t gemm_wide_smem(uint32_t b_bytes, int stages);
+__global__ void k_gemm_wide(const __grid_constant__ CUtensorMap tmA,
+                            const __grid_constant__ CUtensorMap tmB,
+                            const __grid_constant__ CUtensorMap tmOut, const GemmArgs g);
 
 // The pair instance of a mode, block size and epilogue form (fqt_gemm_pair.cu).
 GemmKernel gemm_pair_kernel(int mode, int nb, int form);
