@@ -685,8 +685,8 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
         if (rv && sl == 0) rowst[r] = mm;
       }
       __syncthreads();
-      if (tid < G) {
-        const int k0 = tid * nb;
+      for (int gb = tid; gb < G; gb += kQ2Threads) {  // G up to 2048 (narrow rows)
+        const int k0 = gb * nb;
         const int nrows = min(nb, rows - k0);
         float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
         int p = 0;
@@ -721,9 +721,9 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
               kap = 1.0f / (1.0f - rho);
             }
           }
-          a.lead2[(r0 / nb) + tid] = p;
+          a.lead2[(r0 / nb) + gb] = p;
         }
-        float *bp = bpar + tid * 8;
+        float *bp = bpar + gb * 8;
         bp[0] = s1f;
         bp[1] = s2f;
         bp[2] = rho;

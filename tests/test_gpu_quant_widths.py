@@ -64,6 +64,14 @@ def test_row_counts(n, c, kind, block):
     _check(n, c, kind, 5, block, "f32")
 
 
+@pytest.mark.parametrize("n,c,block,dtype", [(1523, 16, 2, "bf16"), (1100, 8, 2, "f32"),
+                                             (2500, 8, 2, "bf16")])
+def test_more_blocks_than_threads_per_unit(n, c, block, dtype):
+    """Narrow rows: a staged unit of k_quant2 holds up to 1024 blocks, more than
+    its CTA has threads."""
+    _check(n, c, orc.BHQ, 5, block, dtype)
+
+
 @pytest.mark.parametrize("c,kind,block", [(336, orc.PSQ, 0), (1008, orc.BHQ, 16)])
 def test_small_workspace_takes_the_one_pass_quantizer(c, kind, block):
     ws = fqt.Workspace(1, 16, 16)
