@@ -324,7 +324,8 @@ fqt_status fqt_quantize_grad(const void *dH, fqt_dtype dtype, int64_t N,
                             : kind == FQT_PSQ ? sample_pass_bytes(N, C, 1)
                                               : 0;
   const bool two_pass = ws_bytes >= kGemmOffset + pass_bytes &&
-                        ((kind == FQT_BHQ && !adapt && bhq_pass_supported((int)C, block)) ||
+                        ((kind == FQT_BHQ && !adapt &&
+                          bhq_pass_order((int)C, block, dtype == FQT_BF16) >= 0) ||
                          (kind == FQT_PSQ && psq_pass_supported((int)C)));
   // (the BHQ widths and blocks that have always needed it refuse it instead)
   const bool bhq_need = kind == FQT_BHQ && !adapt && C >= 64 && C <= 4096 && !(C & (C - 1)) &&

@@ -3,8 +3,9 @@
 //   PTQ       k_range (fqt_quant.cu), k_codes
 //   PSQ       k_row_stats (a row per sample), k_codes
 //   PSQ with a sample per image: k_sample_part, k_sample_finish, k_codes
-//   BHQ, fixed blocks of 4, 8 or 16 rows: k_bhq_stats, k_codes
-//             (k_bhq_offsets in fqt_quant.cu follows for grad_X's offsets)
+//   BHQ, fixed blocks of 4, 8 or 16 rows: k_bhq_stats, k_codes; of 32, 64 or
+//             128 rows: k_bhq_stats_big, k_codes (k_bhq_offsets in
+//             fqt_quant.cu follows for grad_X's offsets)
 // Rows may have any multiple of 8 columns up to kCodesMaxCols (BHQ: 4096).
 //
 // Stochastic rounding runs on the fp32 pipe (two entries per instruction up to
@@ -21,6 +22,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <math.h>
+#include <string.h>
 #include <algorithm>
 
 #include "fqt_common.cuh"
@@ -211,6 +213,25 @@ struct BhqBlock {
   float p, s1, s2, rho;
 };
 
+// How the reflection's column sums w_j = sum_k e_k s_k h_kj are rounded, the
+// rows in ascending order but for W_FOLDED: fma of the product e_k s_k;
+// W_FMA: fma of e_k and the rounded s_k h_kj (as k_quant2); W_ADD: rounded
+// products, added, and the block scalars in fp64 (as k_quant).  A shape keeps
+// one order whichever kernels serve it, so its codes do not depend on the
+// workspace.
+enum { W_FOLDED = 0, W_FMA = 1, W_ADD = 2 };
+
+// w2 += e s x for one pair of columns, in the given order.  (W_ADD in scalar
+// operations: a packed sum of a packed product came out as one rounding.)
+__device__ __forceinline__ f32x2 w_add(int order, float e, float s, f32x2 x, f32x2 w2) {
+  const f32x2 t = mul2(pack2(s, s), x);
+  if (order == W_FMA) return fma2(pack2(e, e), t, w2);
+  float ta, tb, wa, wb;
+  unpack2(t, ta, tb);
+  unpack2(w2, wa, wb);
+  return pack2(__fadd_rn(wa, __fmul_rn(e, ta)), __fadd_rn(wb, __fmul_rn(e, tb)));
+}
+
 // Workspace bytes of the two-pass BHQ quantizer for blocks of at least 4
 // rows: the per-block record and the C column sums w of every block.
 size_t bhq_pass_bytes(int64_t N, int64_t C) {
@@ -242,7 +263,7 @@ size_t bhq_pass_bytes(int64_t N, int64_t C) {
 template <typename T, int LPR, int STEPS, int TEAM, int H, int WARPS, int MINB>
 __global__ void __launch_bounds__(32 * WARPS, MINB)
     k_bhq_stats(const QuantArgs a, BhqBlock *__restrict__ bst, float *__restrict__ wsum,
-                float2 *__restrict__ part) {
+                float2 *__restrict__ part, int order) {
   static_assert(TEAM == 1 || (LPR == 32 && STEPS <= kTeamRows), "team layout");
   static_assert(H == 1 || TEAM == 8, "column parts only for a full team");
   static_assert(WARPS % TEAM == 0, "whole teams");
@@ -251,6 +272,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
   constexpr int XW = TEAM > 1 ? WARPS : 1;
   __shared__ float2 xs_mm[XW][kTeamRows];
   __shared__ float xs_tm[XW][kTeamRows];
+  __shared__ BhqScale xs_sc[TPC];
   __shared__ float2 red[WARPS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int team = warp / TEAM, wi = warp - team * TEAM;
@@ -318,25 +340,20 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
     const float pmin = __shfl_sync(0xffffffffu, rmn, plane);
     const float pmax = __shfl_sync(0xffffffffu, rmx, plane);
     // ---- block scalars s1, s2 (App. D.4) and the reflection ----
-    float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
-    if (np > 0.0f) {
-      float lam1 = __fsub_rn(pmax, pmin);
-      if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
-      const float Nf = (float)nrows;
-      if (lam2 > 0.0f) {
-        const float c1 = cbrtf(lam1), c2 = cbrtf(lam2);
-        const float n3 = cbrtf(Nf), n6 = sqrtf(n3);
-        const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
-        s1f = fB2 * n6 / (c1 * den);
-        s2f = fB2 * n6 / (c2 * den);
-      } else {
-        s1f = fB2 * sqrtf(Nf) / lam1;
+    BhqScale sc;
+    if (LPR < 32 || order != W_ADD) {
+      sc = bhq_scale(np, __fsub_rn(pmax, pmin), lam2, nrows, fB2);
+    } else if constexpr (TEAM == 1) {
+      sc = bhq_scale_f64(np, __fsub_rn(pmax, pmin), lam2, nrows, a.bits);
+    } else {  // in one warp: the fp64 pipe takes 16 cycles per instruction
+      if (wi == 0) {
+        sc = bhq_scale_f64(np, __fsub_rn(pmax, pmin), lam2, nrows, a.bits);
+        if (lane == 0) xs_sc[team] = sc;
       }
-      if (nrows > 1) {
-        rho = 1.0f / sqrtf(Nf);
-        kap = 1.0f / (1.0f - rho);
-      }
+      team_sync<TEAM>(team);
+      sc = xs_sc[team];
     }
+    const float s1f = sc.s1, s2f = sc.s2, rho = sc.rho, kap = sc.kap;
     const float el = __fmul_rn(kap * (rho - 1.0f), s1f), eo = __fmul_rn(kap * rho, s2f);
     float tmn = INFINITY;  // z' of row kown
     // the last part read is still in registers; the others are read again
@@ -347,12 +364,21 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
       f32x2 w2[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) w2[i] = pack2(0.0f, 0.0f);
+      if (LPR < 32 || order == W_FOLDED) {
 #pragma unroll
-      for (int s = 0; s < STEPS; ++s) {
-        const float e = sub + RS * s == p ? el : eo;
-        const f32x2 e2 = pack2(e, e);
+        for (int s = 0; s < STEPS; ++s) {
+          const float e = sub + RS * s == p ? el : eo;
+          const f32x2 e2 = pack2(e, e);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) w2[i] = fma2(e2, x[s].pair(i), w2[i]);
+          for (int i = 0; i < 4; ++i) w2[i] = fma2(e2, x[s].pair(i), w2[i]);
+        }
+      } else {
+#pragma unroll
+        for (int s = 0; s < STEPS; ++s) {
+          const float e = kap * (s == p ? rho - 1.0f : rho), sk = s == p ? s1f : s2f;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) w2[i] = w_add(order, e, sk, x[s].pair(i), w2[i]);
+        }
       }
       float w[8];
 #pragma unroll
@@ -406,6 +432,193 @@ __global__ void __launch_bounds__(32 * WARPS, MINB)
         a.lead2[blk] = p;
       }
     }
+  }
+  cta_range(gmn, gmx, red, part + blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// The same statistics pass for blocks of 32, 64 or 128 rows, which registers
+// do not hold: a CTA per block reads it three times, the second and third from
+// L1 or L2: rows over warps for the row ranges (LPR lanes a row, four rows in
+// flight), pairs of columns over threads for w, the rows in order, and rows
+// over warps again for z'.
+// What bounds it: the latency of the three passes at a block per CTA.  53910 x
+// 352 bf16 in blocks of 64 (38 MB), with the code pass: k_range and k_quant2,
+// one staged pass with the range pass before it, 127 -> 80 us; 50176 x 256
+// fp32 in blocks of 32: 108 -> 52, 2471 x 208: 17 -> 14, 8192 x 2048: 152 -> 74
+// (fp64 block scalars, about 10 us of them).
+// ---------------------------------------------------------------------------
+constexpr int kBigRows = 128;
+
+template <typename T>
+__device__ __forceinline__ f32x2 load_pair(const T *p) {
+  if constexpr (sizeof(T) == 4) {
+    const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+    return pack2(v.x, v.y);
+  } else {
+    const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(p));
+    return pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
+  }
+}
+
+template <typename T, int LPR>
+__global__ void __launch_bounds__(256, 3)
+    k_bhq_stats_big(const QuantArgs a, BhqBlock *__restrict__ bst, float *__restrict__ wsum,
+                    float2 *__restrict__ part, int order) {
+  constexpr int RS = 32 / LPR, U = 4, WR = 8 * RS;  // rows of the CTA at a time
+  extern __shared__ __align__(16) float wcol[];     // C column sums
+  __shared__ float2 mm_s[kBigRows];
+  __shared__ BhqScale sc_s;
+  __shared__ float2 red[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int sub = lane / LPR, o = lane - sub * LPR;
+  const int nb = a.block, C = a.C, CO = C / 8;
+  const float fB2 = (float)((1u << a.bits) - 1u);
+  const T *const hp = reinterpret_cast<const T *>(a.h);
+  clear_sums(a);
+  float gmn = INFINITY, gmx = -INFINITY;
+  const int64_t nblocks = (a.N + nb - 1) / nb;
+  for (int64_t blk = blockIdx.x; blk < nblocks; blk += gridDim.x) {
+    const int64_t r0 = blk * nb;
+    const int nrows = (int)min((int64_t)nb, a.N - r0);
+    const T *const hb = hp + r0 * C;
+    // ---- row ranges (rows past the last repeat it) ----
+    for (int q = warp * RS + sub; q - sub < nrows; q += U * WR) {
+      float mn[U], mx[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        mn[u] = INFINITY;
+        mx[u] = -INFINITY;
+      }
+      for (int c = o; c < CO; c += LPR) {
+        Oct<T> x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          x[u].load(hb + (int64_t)min(q + u * WR, nrows - 1) * C + c * 8);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          mn[u] = min_nan(mn[u], x[u].min8());
+          mx[u] = max_nan(mx[u], x[u].max8());
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int off = LPR >> 1; off > 0; off >>= 1) {
+          mn[u] = min_nan(mn[u], __shfl_xor_sync(0xffffffffu, mn[u], off));
+          mx[u] = max_nan(mx[u], __shfl_xor_sync(0xffffffffu, mx[u], off));
+        }
+        gmn = min_nan(gmn, mn[u]);
+        gmx = max_nan(gmx, mx[u]);
+        if (o == 0 && q + u * WR < nrows) mm_s[q + u * WR] = make_float2(mn[u], mx[u]);
+      }
+    }
+    __syncthreads();
+    // ---- lead row and scalars, in every warp ----
+    uint32_t key[kBigRows / 32], best = 0u, second = 0u, at = 0xFFFFFFFFu;
+#pragma unroll
+    for (int i = 0; i < kBigRows / 32; ++i) {
+      const int k = 32 * i + lane;
+      key[i] = 0u;
+      if (k < nrows) key[i] = __float_as_uint(fmaxf(fabsf(mm_s[k].x), fabsf(mm_s[k].y)));
+      best = max(best, key[i]);
+    }
+    best = __reduce_max_sync(0xffffffffu, best);
+#pragma unroll
+    for (int i = kBigRows / 32 - 1; i >= 0; --i)
+      if (32 * i + lane < nrows && key[i] == best) at = 32 * i + lane;
+    const int p = (int)__reduce_min_sync(0xffffffffu, at) & (nb - 1);
+#pragma unroll
+    for (int i = 0; i < kBigRows / 32; ++i)
+      if (32 * i + lane != p) second = max(second, key[i]);
+    second = __reduce_max_sync(0xffffffffu, second);
+    const float np = __uint_as_float(best), lam1 = __fsub_rn(mm_s[p].y, mm_s[p].x);
+    const float lam2 = 2.0f * __uint_as_float(second);
+    BhqScale sc;
+    if (order != W_ADD) {
+      sc = bhq_scale(np, lam1, lam2, nrows, fB2);
+    } else {  // in one warp (fp64)
+      if (warp == 0) {
+        sc = bhq_scale_f64(np, lam1, lam2, nrows, a.bits);
+        if (lane == 0) sc_s = sc;
+      }
+      __syncthreads();
+      sc = sc_s;
+    }
+    // ---- w ----
+    const float el = sc.kap * (sc.rho - 1.0f), eo = sc.kap * sc.rho;
+    for (int c = tid * 2; c < C; c += 512) {
+      f32x2 w2 = pack2(0.0f, 0.0f);
+      for (int k0 = 0; k0 < nrows; k0 += 16) {
+        f32x2 x[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          x[k] = load_pair(hb + (int64_t)min(k0 + k, nrows - 1) * C + c);
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (k0 + k < nrows) {
+            const bool lead = k0 + k == p;
+            w2 = w_add(order, lead ? el : eo, lead ? sc.s1 : sc.s2, x[k], w2);
+          }
+      }
+      float2 w;
+      unpack2(w2, w.x, w.y);
+      *reinterpret_cast<float2 *>(wcol + c) = w;
+      *reinterpret_cast<float2 *>(wsum + blk * (int64_t)C + c) = w;
+    }
+    __syncthreads();
+    // ---- row minima of T (see k_bhq_stats) ----
+    for (int q = warp * RS + sub; q - sub < nrows; q += U * WR) {
+      float mn[U];
+      f32x2 sk2[U], nc2[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        mn[u] = INFINITY;
+        const bool lead = q + u * WR == p;
+        const float sk = lead ? sc.s1 : sc.s2, nck = lead ? 1.0f - sc.rho : -sc.rho;
+        sk2[u] = pack2(sk, sk);
+        nc2[u] = pack2(nck, nck);
+      }
+      for (int c = o; c < CO; c += LPR) {
+        Oct<T> x[U];
+        Oct<float> w;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          x[u].load(hb + (int64_t)min(q + u * WR, nrows - 1) * C + c * 8);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          *reinterpret_cast<float4 *>(&w.v[4 * i]) =
+              *reinterpret_cast<const float4 *>(wcol + c * 8 + 4 * i);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float t[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            unpack2(fma2(nc2[u], w.pair(i), mul2(sk2[u], x[u].pair(i))), t[2 * i], t[2 * i + 1]);
+          mn[u] = min_nan(
+              mn[u],
+              min_nan(min3_nan(min3_nan(min3_nan(t[0], t[1], t[2]), t[3], t[4]), t[5], t[6]),
+                      t[7]));
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int off = LPR >> 1; off > 0; off >>= 1)
+          mn[u] = min_nan(mn[u], __shfl_xor_sync(0xffffffffu, mn[u], off));
+        const int k = q + u * WR;
+        if (o == 0 && k < nrows) {
+          const float sk = k == p ? sc.s1 : sc.s2;
+          a.inv2[r0 + k] = sk > 0.0f ? __fdiv_rn(1.0f, sk) : 0.0f;
+          a.zero2[r0 + k] = mn[u];
+        }
+      }
+    }
+    if (tid == 0) {
+      bst[blk] = BhqBlock{__int_as_float(p), sc.s1, sc.s2, sc.rho};
+      a.lead2[blk] = p;
+    }
+    __syncthreads();  // the tables are reused
   }
   cta_range(gmn, gmx, red, part + blockIdx.x);
 }
@@ -1075,15 +1288,34 @@ fqt_status launch_sample_passes(QuantArgs &a, bool bf16, int64_t rows_per_sample
                    "sample code pass launch");
 }
 
-// The two-pass BHQ quantizer takes fixed blocks of 4, 8 or 16 rows and rows
-// of up to 4096 columns (a multiple of 8).
-bool bhq_pass_supported(int C, int block) {
-  return (block == 4 || block == 8 || block == 16) && C % 8 == 0 && C <= 4096;
+// The two-pass BHQ quantizer: the order of w of a shape, or -1 for the shapes
+// that stay with the one-pass quantizers.  Powers of two from 64 to 4096
+// columns with blocks of 16 (fp32: 4 and 8 too) fold e and s and add a warp's
+// row groups last; the others keep the rounding of the one-pass quantizer that
+// takes them without this scratch, whose rows are added in order, so a warp
+// holds whole columns of them (200000 x 80 fp32 in blocks of 16: 179 us
+// staged, 83 so).  Blocks of one and two rows stay with it, as do blocks of up
+// to 16 of rows of fewer than 32 columns, most of whose lanes would be idle
+// (200000 x 16: 45 against 61 us; x 24: 59 against 61).
+int bhq_pass_order(int C, int block, bool bf16) {
+  if (C % 8 || C > 4096 || block < 4) return -1;
+  if (C >= 64 && !(C & (C - 1)) && (block == 16 || (!bf16 && block < 16))) return W_FOLDED;
+  if (block <= 16 && C < 32) return -1;
+  QuantArgs q;
+  memset(&q, 0, sizeof(q));
+  q.N = 1;
+  q.C = C;
+  q.kind = KIND_BHQ;
+  q.block = block;
+  int nth, grid;
+  size_t smem;
+  if (quant2_geometry(q, bf16, 1, &grid, &smem) == FQT_OK) return W_FMA;
+  return quant_geometry(q, 1, &nth, &grid, &smem) == FQT_OK ? W_ADD : -1;
 }
 
 template <typename T, int LPR, int STEPS, int TEAM, int H>
 static cudaError_t launch_stats(const QuantArgs &a, BhqBlock *bst, float *wsum, float2 *part,
-                                int num_sms, int *grid_out, cudaStream_t st) {
+                                int num_sms, int *grid_out, int order, cudaStream_t st) {
   // registers of the block per thread: 8 (fp32) or 4 per oct
   constexpr int data = STEPS * (sizeof(T) == 4 ? 8 : 4);
   constexpr int WARPS = data >= 64 ? (TEAM == 8 ? 8 : 12) : 8;
@@ -1093,24 +1325,34 @@ static cudaError_t launch_stats(const QuantArgs &a, BhqBlock *bst, float *wsum, 
   int64_t grid = std::min<int64_t>((nblocks + TPC - 1) / TPC, (int64_t)num_sms * MINB);
   if (grid < 1) grid = 1;
   *grid_out = (int)grid;
-  k_bhq_stats<T, LPR, STEPS, TEAM, H, WARPS, MINB><<<(int)grid, 32 * WARPS, 0, st>>>(a, bst, wsum,
-                                                                                     part);
+  k_bhq_stats<T, LPR, STEPS, TEAM, H, WARPS, MINB><<<(int)grid, 32 * WARPS, 0, st>>>(
+      a, bst, wsum, part, order);
   return cudaGetLastError();
 }
 
 template <typename T>
 static cudaError_t launch_stats_any(const QuantArgs &a, BhqBlock *bst, float *wsum, float2 *part,
-                                    int num_sms, int *grid, cudaStream_t st) {
+                                    int num_sms, int *grid, int order, cudaStream_t st) {
   const int C = a.C, nb = a.block;
-#define FQT_ST(L, S, TM, HH) return launch_stats<T, L, S, TM, HH>(a, bst, wsum, part, num_sms, grid, st);
+  if (nb > 16) {
+    // a CTA per block, three per SM; the fewest lanes that hold a row
+    const int64_t nblocks = (a.N + nb - 1) / nb;
+    *grid = (int)std::max<int64_t>(1, std::min<int64_t>(nblocks, (int64_t)num_sms * 3));
+    auto kern = C <= 64 ? k_bhq_stats_big<T, 8> : C <= 128 ? k_bhq_stats_big<T, 16>
+                                                           : k_bhq_stats_big<T, 32>;
+    kern<<<*grid, 256, sizeof(float) * (size_t)C, st>>>(a, bst, wsum, part, order);
+    return cudaGetLastError();
+  }
+#define FQT_ST(L, S, TM, HH) \
+  return launch_stats<T, L, S, TM, HH>(a, bst, wsum, part, num_sms, grid, order, st);
 #define FQT_ST_NB(L, TM, HH)                                                     \
   {                                                                              \
     if (nb == 4) FQT_ST(L, L / 8, TM, HH)                                        \
     if (nb == 8) FQT_ST(L, L / 4, TM, HH)                                        \
     FQT_ST(L, L / 2, TM, HH)                                                     \
   }
-  if (C <= 64) FQT_ST_NB(8, 1, 1)
-  if (C <= 128) FQT_ST_NB(16, 1, 1)
+  if (order == W_FOLDED && C <= 64) FQT_ST_NB(8, 1, 1)
+  if (order == W_FOLDED && C <= 128) FQT_ST_NB(16, 1, 1)
   if (C <= 256) FQT_ST_NB(32, 1, 1)
   if (C <= 512) FQT_ST_NB(32, 2, 1)
   if (C <= 1024) FQT_ST_NB(32, 4, 1)
@@ -1126,7 +1368,8 @@ static cudaError_t launch_stats_any(const QuantArgs &a, BhqBlock *bst, float *ws
 // the statistics pass's range partials, which the code pass reduces.
 fqt_status launch_bhq_passes(QuantArgs &a, bool bf16, int num_sms, void *scratch,
                              float2 *part, cudaStream_t st) {
-  if (a.kind != KIND_BHQ || !bhq_pass_supported(a.C, a.block)) return FQT_EUNSUPPORTED;
+  const int order = a.kind == KIND_BHQ ? bhq_pass_order(a.C, a.block, bf16) : -1;
+  if (order < 0) return FQT_EUNSUPPORTED;
   const int64_t nblocks = (a.N + a.block - 1) / a.block;
   BhqBlock *bst = static_cast<BhqBlock *>(scratch);
   float *wsum = reinterpret_cast<float *>(
@@ -1135,8 +1378,9 @@ fqt_status launch_bhq_passes(QuantArgs &a, bool bf16, int num_sms, void *scratch
   int lg;
   codes_plan(a, lpr, num_sms, &lg);
   int grid1 = 0;
-  cudaError_t e = bf16 ? launch_stats_any<__nv_bfloat16>(a, bst, wsum, part, num_sms, &grid1, st)
-                       : launch_stats_any<float>(a, bst, wsum, part, num_sms, &grid1, st);
+  cudaError_t e = bf16 ? launch_stats_any<__nv_bfloat16>(a, bst, wsum, part, num_sms, &grid1, order,
+                                                          st)
+                       : launch_stats_any<float>(a, bst, wsum, part, num_sms, &grid1, order, st);
   if (e != cudaSuccess) return cuda_fail(e, "BHQ statistics pass launch");
   QuantArgs a2 = a;
   a2.part = part;

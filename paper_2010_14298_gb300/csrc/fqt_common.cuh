@@ -386,4 +386,61 @@ __device__ __forceinline__ HhConst hh_const(int n) {
   return c;
 }
 
+// The block scalars s1, s2 of App. D.4, rho = 1/sqrt(nb) and kappa = 1/(1 -
+// rho) of a block of nrows rows, from the lead row's norm np and range and
+// twice the next norm (all zero for a zero block).
+struct BhqScale {
+  float s1, s2, rho, kap;
+};
+
+__device__ __forceinline__ BhqScale bhq_scale(float np, float lam1, float lam2, int nrows,
+                                              float fB2) {
+  BhqScale r = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (np > 0.0f) {
+    if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
+    const float Nf = (float)nrows;
+    if (lam2 > 0.0f) {
+      const float c1 = cbrtf(lam1), c2 = cbrtf(lam2);
+      const float n3 = cbrtf(Nf), n6 = sqrtf(n3);
+      const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
+      r.s1 = fB2 * n6 / (c1 * den);
+      r.s2 = fB2 * n6 / (c2 * den);
+    } else {
+      r.s1 = fB2 * sqrtf(Nf) / lam1;
+    }
+    if (nrows > 1) {
+      r.rho = 1.0f / sqrtf(Nf);
+      r.kap = 1.0f / (1.0f - r.rho);
+    }
+  }
+  return r;
+}
+
+// The same in fp64, rounded once (k_quant's shapes).
+static __device__ __noinline__ BhqScale bhq_scale_f64(float np, float lam1, float lam2, int nrows,
+                                               int bits) {
+  BhqScale r = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (np > 0.0f) {
+    if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
+    const double Nd = (double)nrows, B = (double)((1u << bits) - 1u);
+    double s1, s2 = 0.0;
+    if (lam2 > 0.0f) {
+      const double c1 = cbrt((double)lam1), c2 = cbrt((double)lam2);
+      const double den = c1 * c1 * pow(Nd, -1.0 / 3.0) + c2 * c2 * pow(Nd, 2.0 / 3.0);
+      s1 = B * pow(Nd, 1.0 / 6.0) / (c1 * den);
+      s2 = B * pow(Nd, 1.0 / 6.0) / (c2 * den);
+    } else {  // limit lambda2 -> 0: the other rows are zero
+      s1 = B * sqrt(Nd) / (double)lam1;
+    }
+    r.s1 = (float)s1;
+    r.s2 = lam2 > 0.0f ? (float)s2 : 0.0f;
+    if (nrows > 1) {
+      const double rho = 1.0 / sqrt(Nd);
+      r.rho = (float)rho;
+      r.kap = (float)(1.0 / (1.0 - rho));
+    }
+  }
+  return r;
+}
+
 }  // namespace fqt

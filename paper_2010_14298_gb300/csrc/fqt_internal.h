@@ -74,7 +74,7 @@ fqt_status launch_conv_colsum(const uint16_t *f16, int64_t n, int h, int w, int 
 bool conv_lines_supported(int h, int w, int C, int kh, int kw, int pad);
 fqt_status launch_conv_lines(const uint16_t *f16, int64_t n, int h, int w, int C, int32_t *pad_a,
                              int32_t *col_sum, int centre, cudaStream_t st);
-bool bhq_pass_supported(int C, int block);
+int bhq_pass_order(int C, int block, bool bf16);
 bool ptq_pass_supported(int C);
 bool psq_pass_supported(int C);
 void ptq_pass_plan(QuantArgs &a, int num_sms);

@@ -301,34 +301,12 @@ __global__ void __launch_bounds__(NTMAX) k_quant(const QuantArgs a) {
         for (int k = 0; k < nrows; ++k)
           if (k != p) lam2 = fmaxf(lam2, fmaxf(fabsf(rs[k].x), fabsf(rs[k].y)));
         lam2 = 2.0f * lam2;
-        float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
-        if (np > 0.0f) {
-          float lam1 = __fsub_rn(rs[p].y, rs[p].x);
-          if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
-          const double Nd = (double)nrows;
-          double s1, s2 = 0.0;
-          if (lam2 > 0.0f) {  // s1, s2 of App. D.4
-            const double c1 = cbrt((double)lam1), c2 = cbrt((double)lam2);
-            const double den = c1 * c1 * pow(Nd, -1.0 / 3.0) +
-                               c2 * c2 * pow(Nd, 2.0 / 3.0);
-            s1 = (double)B2 * pow(Nd, 1.0 / 6.0) / (c1 * den);
-            s2 = (double)B2 * pow(Nd, 1.0 / 6.0) / (c2 * den);
-          } else {  // limit lambda2 -> 0: the other rows are zero
-            s1 = (double)B2 * sqrt(Nd) / (double)lam1;
-          }
-          s1f = (float)s1;
-          s2f = lam2 > 0.0f ? (float)s2 : 0.0f;
-          if (nrows > 1) {
-            const double r = 1.0 / sqrt(Nd);
-            rho = (float)r;
-            kap = (float)(1.0 / (1.0 - r));
-          }
-        }
+        const BhqScale sc = bhq_scale_f64(np, __fsub_rn(rs[p].y, rs[p].x), lam2, nrows, a.bits);
         float *bp = bpar + grp * 8;
-        bp[0] = s1f;
-        bp[1] = s2f;
-        bp[2] = rho;
-        bp[3] = kap;
+        bp[0] = sc.s1;
+        bp[1] = sc.s2;
+        bp[2] = sc.rho;
+        bp[3] = sc.kap;
         bp[4] = __int_as_float(p);
         a.lead2[u] = p;
       }
@@ -688,7 +666,7 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
       for (int gb = tid; gb < G; gb += kQ2Threads) {  // G up to 2048 (narrow rows)
         const int k0 = gb * nb;
         const int nrows = min(nb, rows - k0);
-        float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
+        BhqScale sc = {0.0f, 0.0f, 0.0f, 0.0f};
         int p = 0;
         if (nrows > 0) {
           float np = -1.0f;
@@ -702,32 +680,15 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
             const float2 q = rowst[k0 + k];
             if (k != p) lam2 = fmaxf(lam2, fmaxf(fabsf(q.x), fabsf(q.y)));
           }
-          lam2 = 2.0f * lam2;
-          if (np > 0.0f) {
-            float lam1 = __fsub_rn(rowst[k0 + p].y, rowst[k0 + p].x);
-            if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
-            const float Nf = (float)nrows;
-            if (lam2 > 0.0f) {  // s1, s2 of App. D.4
-              const float c1 = cbrtf(lam1), c2 = cbrtf(lam2);
-              const float n3 = cbrtf(Nf), n6 = sqrtf(n3);
-              const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
-              s1f = (float)B2 * n6 / (c1 * den);
-              s2f = (float)B2 * n6 / (c2 * den);
-            } else {  // lambda2 -> 0: the other rows are zero
-              s1f = (float)B2 * sqrtf(Nf) / lam1;
-            }
-            if (nrows > 1) {
-              rho = 1.0f / sqrtf(Nf);
-              kap = 1.0f / (1.0f - rho);
-            }
-          }
+          sc = bhq_scale(np, __fsub_rn(rowst[k0 + p].y, rowst[k0 + p].x), 2.0f * lam2, nrows,
+                         (float)B2);
           a.lead2[(r0 / nb) + gb] = p;
         }
         float *bp = bpar + gb * 8;
-        bp[0] = s1f;
-        bp[1] = s2f;
-        bp[2] = rho;
-        bp[3] = kap;
+        bp[0] = sc.s1;
+        bp[1] = sc.s2;
+        bp[2] = sc.rho;
+        bp[3] = sc.kap;
         bp[4] = __int_as_float(p);
       }
       __syncthreads();

@@ -51,6 +51,37 @@ def test_bhq_widths(c, block, dtype):
     _check(5 * 16 + 7, c, orc.BHQ, 5, block, dtype)
 
 
+@pytest.mark.parametrize("n,c,block,dtype", [
+    (33, 8, 32, "f32"), (200, 24, 128, "bf16"), (777, 72, 64, "bf16"), (129, 136, 128, "f32"),
+    (300, 264, 32, "f32"), (131, 1008, 64, "bf16"), (64, 1024, 64, "f32"), (95, 2048, 32, "f32"),
+    (1, 64, 32, "f32")])
+def test_bhq_big_blocks(n, c, block, dtype):
+    _check(n, c, orc.BHQ, 5, block, dtype)
+
+
+@pytest.mark.parametrize("n,c", [(1523, 32), (700, 80), (1523, 128), (1523, 200), (301, 1008),
+                                 (301, 1512), (200, 2048), (70, 4096)])
+@pytest.mark.parametrize("block", [4, 8, 16, 32, 64, 128])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_bhq_passes_equal_the_one_pass_quantizer(n, c, block, dtype):
+    """A workspace without the passes' scratch takes the one-pass quantizers:
+    every output equal, whichever kernels serve the shape."""
+    if block * c > 65536:
+        pytest.skip("blocks of this width are refused")
+    always = c >= 64 and not c & (c - 1) and (block == 16 or (dtype == "f32" and block < 16))
+    if always:
+        pytest.skip("these shapes refuse the smaller workspace")
+    x = to_dev(wl.random_grad(wl.rng(n + c + block), n, c), dtype)
+    small = fqt.Workspace(1, 16, 16)
+    small.nbytes = 256 + 32768  # the header and the range partials
+    a2, a1 = fqt.quantize_grad(x, orc.BHQ, 8, block, 5, ws=fqt.Workspace(n, c, 16))
+    b2, b1 = fqt.quantize_grad(x, orc.BHQ, 8, block, 5, ws=small)
+    for f in ("codes", "inv_s", "zero", "row_sum", "lead", "hz", "hr"):
+        assert torch.equal(getattr(a2, f), getattr(b2, f)), f
+    for f in ("codes", "inv_s", "zero", "col_sum"):
+        assert torch.equal(getattr(a1, f), getattr(b1, f)), f
+
+
 @pytest.mark.parametrize("c", WIDTHS + [8192])
 @pytest.mark.parametrize("kind,bits,dtype", [(orc.PTQ, 8, "f32"), (orc.PSQ, 8, "bf16"),
                                              (orc.PSQ, 4, "f32")])
