@@ -1294,13 +1294,14 @@ fqt_status launch_sample_passes(QuantArgs &a, bool bf16, int64_t rows_per_sample
 // row groups last; the others keep the rounding of the one-pass quantizer that
 // takes them without this scratch, whose rows are added in order, so a warp
 // holds whole columns of them (200000 x 80 fp32 in blocks of 16: 179 us
-// staged, 83 so).  Blocks of one and two rows stay with it, as do blocks of up
-// to 16 of rows of fewer than 32 columns, most of whose lanes would be idle
-// (200000 x 16: 45 against 61 us; x 24: 59 against 61).
+// staged, 83 so).  Blocks of one and two rows stay with it, as do rows of
+// fewer than 40 columns, most of whose lanes would be idle (200000 rows of 16
+// in blocks of 16: 45 against 61 us, of 32 in blocks of 4: 60 against 70, of
+// 24 in blocks of 64: 68 against 76; of 40 in blocks of 16: 95 against 63).
 int bhq_pass_order(int C, int block, bool bf16) {
   if (C % 8 || C > 4096 || block < 4) return -1;
   if (C >= 64 && !(C & (C - 1)) && (block == 16 || (!bf16 && block < 16))) return W_FOLDED;
-  if (block <= 16 && C < 32) return -1;
+  if (C < 40) return -1;
   QuantArgs q;
   memset(&q, 0, sizeof(q));
   q.N = 1;

@@ -52,14 +52,14 @@ def test_bhq_widths(c, block, dtype):
 
 
 @pytest.mark.parametrize("n,c,block,dtype", [
-    (33, 8, 32, "f32"), (200, 24, 128, "bf16"), (777, 72, 64, "bf16"), (129, 136, 128, "f32"),
+    (33, 40, 32, "f32"), (200, 56, 128, "bf16"), (777, 72, 64, "bf16"), (129, 136, 128, "f32"),
     (300, 264, 32, "f32"), (131, 1008, 64, "bf16"), (64, 1024, 64, "f32"), (95, 2048, 32, "f32"),
     (1, 64, 32, "f32")])
 def test_bhq_big_blocks(n, c, block, dtype):
     _check(n, c, orc.BHQ, 5, block, dtype)
 
 
-@pytest.mark.parametrize("n,c", [(1523, 32), (700, 80), (1523, 128), (1523, 200), (301, 1008),
+@pytest.mark.parametrize("n,c", [(1523, 40), (700, 80), (1523, 128), (1523, 200), (301, 1008),
                                  (301, 1512), (200, 2048), (70, 4096)])
 @pytest.mark.parametrize("block", [4, 8, 16, 32, 64, 128])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
