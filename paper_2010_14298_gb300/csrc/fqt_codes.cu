@@ -4,8 +4,9 @@
 //   PSQ       k_row_stats (a row per sample), k_codes
 //   PSQ with a sample per image: k_sample_part, k_sample_finish, k_codes
 //   BHQ, fixed blocks of 4, 8 or 16 rows: k_bhq_stats, k_codes; of 32, 64 or
-//             128 rows: k_bhq_stats_big, k_codes (k_bhq_offsets in
-//             fqt_quant.cu follows for grad_X's offsets)
+//             128 rows: k_bhq_stats_big, k_codes (grad_X's offsets: k_codes
+//             where its units hold whole blocks, else k_bhq_offsets in
+//             fqt_quant.cu)
 // Rows may have any multiple of 8 columns up to kCodesMaxCols (BHQ: 4096).
 //
 // Stochastic rounding runs on the fp32 pipe (two entries per instruction up to
@@ -817,7 +818,9 @@ size_t sample_pass_bytes(int64_t N, int64_t C, int64_t rows_per_sample) {
 // 33 -> 25 us, 8192 x 4096 bf16 70 -> 50 us, 8192 x 1024 bf16 PTQ-8 (k_quant2
 // before) 29 -> 16 us.  Staging the rows through shared memory three deep
 // (cp.async) instead of one row ahead in registers was slower (397 us on the
-// first shape).
+// first shape).  grad_X's BHQ offsets of a unit that holds whole blocks are
+// computed from the row sums at its end: 305 -> 312 us on the first shape, and
+// no k_bhq_offsets (13 us).
 // ---------------------------------------------------------------------------
 constexpr int kCodeRows = 32;
 constexpr int kCodesMaxCols = 8192;
@@ -1134,6 +1137,30 @@ __global__ void __launch_bounds__(256, 2)
       if (!one_slab) flush_cs(c0);
     }
     __syncwarp();
+    // grad_X's offsets, where the unit holds whole blocks and whole rows
+    if (MODE == CODES_BHQ && a.hz) {
+      const bool kv = lane < rows;
+      const int base = lane & ~nbm, nact = min(nbm + 1, rows - base);
+      ff d = {0.0f, 0.0f};
+      long long R = 0;
+      int p = 0;
+      if (kv) {
+        bhq_offset_terms(a.zero2[row0 + lane], rs_s[warp][0][lane], C, 1 << (a.bits - 1), &d, &R);
+        p = __float_as_int(bst[(row0 + lane) >> lg_nb].p);
+      }
+      ff sd = d;
+      long long sR = R;
+      bhq_offset_sums(&sd, &sR, nbm + 1);
+      const ff dp = {__shfl_sync(0xffffffffu, d.h, base + p),
+                     __shfl_sync(0xffffffffu, d.l, base + p)};
+      const long long Rp = __shfl_sync(0xffffffffu, R, base + p);
+      if (kv) {
+        const float2 v = nact < 2 ? make_float2(ff_round(d), ff_round(ff_from_int(R)))
+                                  : bhq_offset_reflect(d, R, sd, sR, dp, Rp, lane - base == p, nact);
+        a.hz[row0 + lane] = v.x;
+        a.hr[row0 + lane] = v.y;
+      }
+    }
     if (lane < rows) {
       if (split > 1) {
         if (a.rsum2) atomicAdd(&a.rsum2[row0 + lane], rs_s[warp][0][lane]);
@@ -1170,13 +1197,21 @@ static int codes_lpr(int C) {
 // Rows per unit and column parts of the code pass: about 64 units per SM
 // (four per warp), first by splitting wide rows into slabs, then by units of
 // 16 and 8 rows.
-static void codes_plan(QuantArgs &a, int lpr, int num_sms, int *lg_urows) {
+static void codes_plan(QuantArgs &a, int lpr, int num_sms, int *lg_urows, int lg_nb = 0) {
   const int nslab = (a.C + 16 * lpr - 1) / (16 * lpr);
   const int64_t target = (int64_t)num_sms * 64;
   int lg = 5, split = 1;
   auto units = [&]() { return ((a.N + (1 << lg) - 1) >> lg) * (int64_t)split; };
   while (split < nslab && units() < target) split *= 2;
   while (lg > 3 && units() < target) --lg;
+  // units of whole blocks hold what grad_X's offsets need: three per warp are
+  // still enough (131072 x 64: code pass 21.9 -> 22.9 us without 3.7 + 2.5 for
+  // k_bhq_offsets and its gap)
+  if (split == 1 && lg < lg_nb && lg_nb <= 5) {
+    const int few = lg;
+    lg = lg_nb;
+    if (units() < (int64_t)num_sms * 48) lg = few;
+  }
   a.code_split = split;
   *lg_urows = lg;
 }
@@ -1377,7 +1412,9 @@ fqt_status launch_bhq_passes(QuantArgs &a, bool bf16, int num_sms, void *scratch
       (reinterpret_cast<uintptr_t>(bst + nblocks) + 255) & ~(uintptr_t)255);
   const int lpr = codes_lpr(a.C);
   int lg;
-  codes_plan(a, lpr, num_sms, &lg);
+  int lg_nb = 0;
+  while ((1 << lg_nb) < a.block) ++lg_nb;
+  codes_plan(a, lpr, num_sms, &lg, a.hz && a.hr ? lg_nb : 0);
   int grid1 = 0;
   cudaError_t e = bf16 ? launch_stats_any<__nv_bfloat16>(a, bst, wsum, part, num_sms, &grid1, order,
                                                           st)
@@ -1386,11 +1423,12 @@ fqt_status launch_bhq_passes(QuantArgs &a, bool bf16, int num_sms, void *scratch
   QuantArgs a2 = a;
   a2.part = part;
   a2.npart = grid1;
-  int lg_nb = 0;
-  while ((1 << lg_nb) < a.block) ++lg_nb;
+  // a warp that holds whole rows of whole blocks has what the offsets need
+  const bool fused = a.hz && a.hr && a.rsum2 && a2.code_split == 1 && lg_nb <= lg;
+  if (!fused) a2.hz = a2.hr = nullptr;
   e = launch_codes<CODES_BHQ>(a2, bf16, lpr, bst, wsum, lg_nb, nullptr, 1, lg, num_sms, st);
   if (e != cudaSuccess) return cuda_fail(e, "BHQ code pass launch");
-  if (a.hz && a.hr) {
+  if (a.hz && a.hr && !fused) {
     e = launch_bhq_offsets(a.zero2, a.rsum2, a.lead2, a.hz, a.hr, a.N, a.C, a.bits, a.block, st);
     if (e != cudaSuccess) return cuda_fail(e, "BHQ offsets launch");
   }

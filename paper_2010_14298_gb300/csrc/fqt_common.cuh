@@ -443,4 +443,39 @@ static __device__ __noinline__ BhqScale bhq_scale_f64(float np, float lam1, floa
   return r;
 }
 
+// grad_X offsets of a BHQ row (k_bhq_offsets): the fraction d of its offset oa +
+// zero beside the integer that the epilogue takes, and R = sum_c (a_c + m).
+__device__ __forceinline__ void bhq_offset_terms(float zero, int rsum, int C, int oa, ff *d,
+                                                 long long *R) {
+  const ff x = two_sum((float)oa, zero);
+  const float m = rintf(x.h);  // the epilogue rounds the same fp32 sum
+  *d = fast_two_sum(__fsub_rn(x.h, m), x.l);
+  *R = (long long)rsum - (long long)C * oa + (long long)C * (long long)m;
+}
+
+// Their sums over a block of nb <= 32 rows, one row per lane, blocks side by
+// side in the warp (rows that do not exist add 0).
+__device__ __forceinline__ void bhq_offset_sums(ff *sd, long long *sR, int nb) {
+  for (int off = 1; off < nb; off <<= 1) {
+    const ff od = {__shfl_xor_sync(0xffffffffu, sd->h, off),
+                   __shfl_xor_sync(0xffffffffu, sd->l, off)};
+    *sd = ff_add(*sd, od);
+    *sR += __shfl_xor_sync(0xffffffffu, *sR, off);
+  }
+}
+
+// (hz, hr) of a row of a block of nact >= 2: (Q v)_k = v_k - kappa (rho sum(v) -
+// v_p) off the lead row p, rho sum(v) on it.
+__device__ __forceinline__ float2 bhq_offset_reflect(ff d, long long R, ff sd, long long sR,
+                                                     ff dp, long long Rp, bool lead, int nact) {
+  const HhConst c = hh_const(nact);
+  const ff rsd = ff_mul(c.rho, sd);
+  const ff rsR = ff_mul(c.rho, ff_from_int(sR));
+  if (lead) return make_float2(ff_round(rsd), ff_round(rsR));
+  const ff wd = ff_add(rsd, ff_neg(dp));
+  const ff wR = ff_add(rsR, ff_neg(ff_from_int(Rp)));
+  return make_float2(ff_round(ff_add(d, ff_neg(ff_mul(c.kap, wd)))),
+                     ff_round(ff_add(ff_from_int(R), ff_neg(ff_mul(c.kap, wR)))));
+}
+
 }  // namespace fqt

@@ -1476,12 +1476,7 @@ __global__ void __launch_bounds__(kOffThreads)
   const bool kv = k < N;
   ff d = {0.0f, 0.0f};
   long long R = 0;
-  if (kv) {
-    const ff x = two_sum((float)oa, zero[k]);
-    const float m = rintf(x.h);  // the epilogue rounds the same fp32 sum
-    d = fast_two_sum(__fsub_rn(x.h, m), x.l);
-    R = (long long)rsum[k] - (long long)C * oa + (long long)C * (long long)m;
-  }
+  if (kv) bhq_offset_terms(zero[k], rsum[k], C, oa, &d, &R);
   ds[t] = make_float2(d.h, d.l);
   Rs[t] = R;
   // the sums of a block of up to 32 rows by shuffles (rows past N add 0): a
@@ -1489,12 +1484,7 @@ __global__ void __launch_bounds__(kOffThreads)
   // of 16, this 12.9 us
   ff sdw = d;
   long long sRw = R;
-  for (int off = 1; off < nb && off < 32; off <<= 1) {
-    const ff od = {__shfl_xor_sync(0xffffffffu, sdw.h, off),
-                   __shfl_xor_sync(0xffffffffu, sdw.l, off)};
-    sdw = ff_add(sdw, od);
-    sRw += __shfl_xor_sync(0xffffffffu, sRw, off);
-  }
+  bhq_offset_sums(&sdw, &sRw, min(nb, 32));
   __syncthreads();
   if (!kv) return;
   const int base = (t / nb) * nb;  // nb divides kOffThreads: blocks stay in the CTA
@@ -1517,19 +1507,10 @@ __global__ void __launch_bounds__(kOffThreads)
       sR += Rs[base + l];
     }
   }
-  const HhConst c = hh_const(nact);
-  // (Q v)_k = v_k - kappa (rho sum(v) - v_p) off the lead row; rho sum(v) on it
-  const ff rsd = ff_mul(c.rho, sd);
-  const ff rsR = ff_mul(c.rho, ff_from_int(sR));
-  if (t - base == p) {
-    hz[k] = ff_round(rsd);
-    hr[k] = ff_round(rsR);
-    return;
-  }
-  const ff wd = ff_add(rsd, ff_neg({ds[base + p].x, ds[base + p].y}));
-  const ff wR = ff_add(rsR, ff_neg(ff_from_int(Rs[base + p])));
-  hz[k] = ff_round(ff_add(d, ff_neg(ff_mul(c.kap, wd))));
-  hr[k] = ff_round(ff_add(ff_from_int(R), ff_neg(ff_mul(c.kap, wR))));
+  const float2 o = bhq_offset_reflect(d, R, sd, sR, {ds[base + p].x, ds[base + p].y},
+                                      Rs[base + p], t - base == p, nact);
+  hz[k] = o.x;
+  hr[k] = o.y;
 }
 
 cudaError_t launch_bhq_offsets(const float *zero, const int32_t *rsum,

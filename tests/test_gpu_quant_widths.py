@@ -59,7 +59,7 @@ def test_bhq_big_blocks(n, c, block, dtype):
     _check(n, c, orc.BHQ, 5, block, dtype)
 
 
-@pytest.mark.parametrize("n,c", [(1523, 40), (700, 80), (1523, 128), (1523, 200), (301, 1008),
+@pytest.mark.parametrize("n,c", [(1523, 40), (700, 80), (240003, 40), (1523, 128), (1523, 200), (301, 1008),
                                  (301, 1512), (200, 2048), (70, 4096)])
 @pytest.mark.parametrize("block", [4, 8, 16, 32, 64, 128])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
