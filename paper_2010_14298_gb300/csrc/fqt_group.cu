@@ -53,6 +53,8 @@ constexpr int kKeysThreads = 1024;
 // sizes follow the sorted norms (non-increasing up to the rounding), so
 // every such group has an index below N / kBigGroup + 1.
 constexpr int kBigGroup = 64;
+// Groups of up to kSmallGroup rows: a sub-warp each.
+constexpr int kSmallGroup = 4;
 __host__ __device__ inline int64_t big_grid(int64_t N) { return N / kBigGroup + 1; }
 // the sort's tile offsets are summed per CTA over all tiles: 256 tiles at most
 constexpr int64_t kMaxGroupRows = (int64_t)1 << 20;
@@ -319,7 +321,7 @@ struct BestFF {
 __global__ void __launch_bounds__(256) k_grp_choose(const uint32_t *__restrict__ keys, int64_t N,
                                                     const ff *__restrict__ tsum, ff *cincl,
                                                     BestFF *best, long long *Gout, ff *SGout,
-                                                    unsigned *count) {
+                                                    unsigned *count, unsigned *slots) {
   __shared__ ff red[8];
   __shared__ ff bv_s[8];
   __shared__ long long bg_s[8];
@@ -403,13 +405,14 @@ __global__ void __launch_bounds__(256) k_grp_choose(const uint32_t *__restrict__
     last = atomicAdd(count, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (!last) return;
+  if (!last || warp) return;
   __threadfence();
-  // the best of all CTAs (the order of `better` is total: any grouping); one
-  // thread over 128 of them took 9 of the kernel's 22.4 us at 131072 rows
+  // the best of all CTAs, by one warp (the order of `better` is total: any
+  // grouping); one thread over 128 of them took 9 of the kernel's 22.4 us at
+  // 131072 rows
   ff fv = {INFINITY, 0.0f};
   long long fg = 0x7fffffffffffffffll;
-  for (int bb = tid; bb < (int)gridDim.x; bb += 256) {
+  for (int bb = lane; bb < (int)gridDim.x; bb += 32) {
     const volatile BestFF *x = best + bb;
     const ff xv = {x->h, x->l};
     const long long xg = x->g;
@@ -427,22 +430,13 @@ __global__ void __launch_bounds__(256) k_grp_choose(const uint32_t *__restrict__
       fg = og;
     }
   }
-  if (lane == 0) {
-    bv_s[warp] = fv;
-    bg_s[warp] = fg;
-  }
-  __syncthreads();
-  if (tid != 0) return;
-  for (int w = 1; w < 8; ++w)
-    if (better(bv_s[w], bg_s[w], fv, fg)) {
-      fv = bv_s[w];
-      fg = bg_s[w];
-    }
+  if (lane) return;
   if (fg < 1 || fg >= N) fg = 1;  // N = 1: one group
   *Gout = fg;
   const volatile ff *cg = cincl + fg - 1;
   *SGout = ff{cg->h, cg->l};
   *count = 0u;
+  slots[0] = slots[1] = 0u;  // k_grp_layout and k_bhq_groups
 }
 
 // e_j of the cumulative rounding, in fp64 (two divisions per group) so that
@@ -466,7 +460,6 @@ __global__ void __launch_bounds__(256) k_grp_layout(const int32_t *__restrict__ 
                                                     int32_t *perm, int32_t *gstart,
                                                     int32_t *gsize, unsigned *slots) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) *slots = 0u;
   if (i > N) return;
   const int64_t G = *Gp;
   if (i >= G) {
@@ -478,6 +471,10 @@ __global__ void __launch_bounds__(256) k_grp_layout(const int32_t *__restrict__ 
   int64_t e1 = cum_size(i + 1, N, G, SG, cincl);
   if (e1 < e0) e1 = e0;
   const int64_t k0 = i + e0, ns = e1 - e0;
+  // one past the last group of more than kSmallGroup rows
+  const unsigned act = __activemask();
+  const unsigned lim = __reduce_max_sync(act, ns + 1 > kSmallGroup ? (unsigned)i + 1u : 0u);
+  if (lim && (threadIdx.x & 31) == __ffs(act) - 1) atomicMax(slots + 1, lim);
   gstart[i] = (int32_t)k0;
   perm[k0] = vals[i];
   for (int64_t t = 0; t < ns; ++t) perm[k0 + 1 + t] = vals[N - e1 + t];
@@ -486,10 +483,18 @@ __global__ void __launch_bounds__(256) k_grp_layout(const int32_t *__restrict__ 
 
 // ---------------------------------------------------------------------------
 // Quantizer over the groups: a warp per group, RS = 32 / LPR rows per step
-// (LPR lanes per row, 8 columns per lane).  Pass 1 reads the rows for the
+// (LPR lanes per row, 8 columns per lane); runs of one-row groups a row per
+// sub-warp, and (64 columns) runs of groups of up to four rows a group per
+// sub-warp, read once and held in registers.  Pass 1 reads the rows for the
 // lead row's range, lambda2 and the column sums of the small rows; pass 2
 // re-reads them (L2) for the transform, the row minima, SR and packing; the
 // grad_X offsets hz, hr are reflected at the end (see k_bhq_team).
+// What bounds it: the serial chain of a warp (queue, gstart, perm, rows, the
+// reductions of each row), so groups of more rows than a sub-warp takes are
+// handed out one by one, before the others: 131072 x 64 fp32 with 1% outlier
+// rows 84 -> 70 us, lognormal rows 115 -> 68, equal rows 99 -> 51; 50000 x 128
+// 52 -> 37 and 96 -> 56.  Loading four steps of every group ahead was slower
+// (84 -> 107: the registers of a third resident CTA).
 // ---------------------------------------------------------------------------
 template <int LPR>
 __device__ __forceinline__ float2 row_minmax(float2 v) {
@@ -533,7 +538,7 @@ __device__ __forceinline__ int sub_addi(int v) {
 }
 
 template <typename T, int LPR>
-__global__ void __launch_bounds__(256, 3) k_bhq_groups(const QuantArgs a) {
+__global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const QuantArgs a) {
   __shared__ float2 red[8];
   __shared__ int redi[8];
   extern __shared__ int csum_s[];  // C column sums of Q_b1
@@ -666,23 +671,175 @@ __global__ void __launch_bounds__(256, 3) k_bhq_groups(const QuantArgs a) {
     }
   };
 
-  // A warp takes slots of RS consecutive groups from a queue: all single
-  // rows -> one step; otherwise the groups one after another, a warp each.
+  // One group of up to kSmall rows per sub-warp (n rows from k0; none: n = 0),
+  // its rows in registers: the arithmetic and the order of every sum are those
+  // of a group on a whole warp below.
+  constexpr int kSmall = kSmallGroup;
+  auto do_small = [&](int64_t k0, int n) {
+    const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
+    int64_t src[kSmall];
+    float x[kSmall][8];
+#pragma unroll
+    for (int r = 0; r < kSmall; ++r) {
+      src[r] = r < n ? (int64_t)__ldg(a.perm + k0 + r) : 0;
+      if (src[r] < 0 || src[r] >= N) {
+        badp = true;
+        src[r] = 0;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kSmall; ++r) {
+      if (r < n) {
+        load_oct(h + src[r] * C + o * 8, x[r]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[r][j] = 0.0f;
+      }
+    }
+    float pmin = 0.0f, pmax = 0.0f, l2 = 0.0f;
+#pragma unroll
+    for (int r = 0; r < kSmall; ++r) {
+      if (r >= nmax) break;
+      float2 mm = make_float2(INFINITY, -INFINITY);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        mm.x = fminf(mm.x, x[r][j]);
+        mm.y = fmaxf(mm.y, x[r][j]);
+      }
+      mm = row_minmax<LPR>(mm);
+      if (r == 0) {
+        pmin = mm.x;
+        pmax = mm.y;
+      } else {
+        l2 = fmaxf(l2, fmaxf(fabsf(mm.x), fabsf(mm.y)));  // (absent rows are 0)
+      }
+    }
+    const float np = fmaxf(fabsf(pmin), fabsf(pmax));
+    const BhqScale sc = bhq_scale(np, __fsub_rn(pmax, pmin), 2.0f * l2, n, (float)B2);
+    const float el = sc.kap * (sc.rho - 1.0f), es = sc.kap * sc.rho;
+    float w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      // the rows r of a sub-warp in order, then the sub-warps r % RS
+      const float csm = RS == 4   ? x[1][j] + (x[2][j] + x[3][j])
+                        : RS == 2 ? x[2][j] + (x[1][j] + x[3][j])
+                                  : (x[1][j] + x[2][j]) + x[3][j];
+      w[j] = fmaf(es, __fmul_rn(sc.s2, csm), el * __fmul_rn(sc.s1, x[0][j]));
+    }
+    ff d[kSmall], R[kSmall];
+#pragma unroll
+    for (int r = 0; r < kSmall; ++r) d[r] = R[r] = {0.0f, 0.0f};
+#pragma unroll
+    for (int r = 0; r < kSmall; ++r) {
+      if (r >= nmax) break;
+      const bool v = r < n;
+      const float sk = r == 0 ? sc.s1 : sc.s2;
+      const float ck = r == 0 ? sc.rho - 1.0f : sc.rho;
+      float t[8];
+      float tmin = INFINITY;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        t[j] = fmaf(-ck, w[j], __fmul_rn(sk, x[r][j]));
+        tmin = fminf(tmin, t[j]);
+      }
+      const float z2 = row_min<LPR>(tmin);
+      const int64_t row = k0 + r;
+      uint32_t c[8];
+      int rs2 = 0, rs1 = 0;
+      if (v) {
+        const uint4 w2 = philox_oct((uint64_t)row * (uint64_t)CO + (uint64_t)o, 0u, key);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          c[j] = sr_code16(__fmul_rn(__fsub_rn(t[j], z2), 65536.0f), u16_of(w2, j), B2);
+          rs2 += (int)c[j];
+        }
+        if (a.c2) store_codes8(a.c2 + row * (int64_t)C + o * 8, c);
+        if (a.f2) store_carriers8(a.f2 + row * (int64_t)C + o * 8, c, og2);
+        if (has_b1) {
+          const uint4 w1 = philox_oct((uint64_t)src[r] * (uint64_t)CO + (uint64_t)o, 1u, key);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float vv = __fmul_rn(__fsub_rn(x[r][j], gmin), s_g1_16);
+            c[j] = sr_code16(vv, u16_of(w1, j), 255u);
+            rs1 += (int)c[j];
+            cs[j] += (int)c[j];
+          }
+          if (a.c1) store_codes8(a.c1 + src[r] * (int64_t)C + o * 8, c);
+          if (a.f1) store_carriers8(a.f1 + src[r] * (int64_t)C + o * 8, c, 128u);
+        }
+      }
+      rs2 = row_add<LPR>(rs2);
+      if (has_b1 && a.rsum1) rs1 = row_add<LPR>(rs1);
+      if (v) {
+        const ff xo = two_sum((float)og2, z2);
+        const float m = rintf(xo.h);
+        d[r] = fast_two_sum(__fsub_rn(xo.h, m), xo.l);
+        R[r] = two_sum((float)(rs2 - C * (int)og2), __fmul_rn((float)C, m));
+        if (o == r) {
+          if (a.rsum2) a.rsum2[row] = rs2;
+          if (has_b1 && a.rsum1) a.rsum1[src[r]] = rs1;
+          a.inv2[row] = sk > 0.0f ? __fdiv_rn(1.0f, sk) : 0.0f;
+          a.zero2[row] = z2;
+        }
+      }
+    }
+    if (a.hz && n > 0) {
+      auto total = [&](const ff (&q)[kSmall]) {
+        return RS == 4   ? ff_add(ff_add(q[0], q[1]), ff_add(q[2], q[3]))
+               : RS == 2 ? ff_add(ff_add(q[0], q[2]), ff_add(q[1], q[3]))
+                         : ff_add(ff_add(ff_add(q[0], q[1]), q[2]), q[3]);
+      };
+      const HhConst hc = hh_const(n);
+      const ff rsd = ff_mul(hc.rho, total(d)), rsR = ff_mul(hc.rho, total(R));
+      const ff kd = ff_mul(hc.kap, ff_add(rsd, {-ff_round(d[0]), 0.0f}));
+      const ff kR = ff_mul(hc.kap, ff_add(rsR, ff_neg(R[0])));
+#pragma unroll
+      for (int r = 0; r < kSmall; ++r)
+        if (r < n && o == r) {
+          ff vd = d[r], vR = R[r];
+          if (n >= 2) {
+            vd = r == 0 ? rsd : ff_add({ff_round(d[r]), 0.0f}, ff_neg(kd));
+            vR = r == 0 ? rsR : ff_add({ff_round(R[r]), 0.0f}, ff_neg(kR));
+          }
+          a.hz[k0 + r] = ff_round(vd);
+          a.hr[k0 + r] = ff_round(vR);
+        }
+    }
+  };
+
+  constexpr bool kSub = RS == 4;  // (wider rows: the registers cost more than it gives)
+  // A warp takes slots of groups from a queue (one ahead): single groups
+  // while there are any of more than kSmallGroup rows (a warp each, the
+  // largest first), then RS consecutive groups: all single rows -> one step,
+  // else a sub-warp each.
+  const int64_t lim = RS == 1 ? N : min(N, ((int64_t)a.slots[1] + RS - 1) / RS * RS);
+  unsigned slot = 0u;
+  if (kSub && lane == 0) slot = atomicAdd(a.slots, 1u);
   for (;;) {
-    unsigned slot = 0u;
-    if (lane == 0) slot = atomicAdd(a.slots, 1u);
-    const int64_t g0 = (int64_t)__shfl_sync(0xffffffffu, slot, 0) * RS;
+    if (!kSub && lane == 0) slot = atomicAdd(a.slots, 1u);
+    const int64_t u = __shfl_sync(0xffffffffu, slot, 0);
+    const int ng = u < lim ? 1 : RS;
+    const int64_t g0 = u < lim ? u : lim + (u - lim) * RS;
     if (g0 >= N) break;
-    const int64_t gk = g0 + (lane < RS ? lane : 0);
+    if (kSub && lane == 0) slot = atomicAdd(a.slots, 1u);
+    const int64_t gk = g0 + (lane < ng ? lane : 0);
     const int64_t ka = gk < N ? __ldg(a.gstart + gk) : N;
     const int64_t kb = gk < N ? __ldg(a.gstart + gk + 1) : N;
     const int64_t s0 = __shfl_sync(0xffffffffu, ka, 0);
     if (s0 >= N) break;  // groups past G are empty and gstart does not decrease
-    if (__all_sync(0xffffffffu, lane >= RS || (ka < N && kb == ka + 1))) {
+    if (ng == RS && __all_sync(0xffffffffu, lane >= RS || (ka < N && kb == ka + 1))) {
       do_singles(s0);
       continue;
     }
-  for (int gs = 0; gs < RS; ++gs) {
+    if constexpr (kSub) {
+      const int64_t size = min(kb, N) - min(ka, N);
+      if (ng == RS && __all_sync(0xffffffffu, lane >= RS || size <= kSmall)) {
+        do_small(__shfl_sync(0xffffffffu, ka, sub),
+                 (int)max((int64_t)0, __shfl_sync(0xffffffffu, size, sub)));
+        continue;
+      }
+    }
+  for (int gs = 0; gs < ng; ++gs) {
     const int64_t gi = g0 + gs;
     if (gi >= N) break;
     const int64_t k0 = __ldg(a.gstart + gi);
@@ -1284,7 +1441,8 @@ fqt_status launch_bhq_grouping(const void *dH, bool bf16, int64_t N, int C, int3
   if (e != cudaSuccess) return cuda_fail(e, "radix sort launch");
   // after four passes the sorted keys are back in k0 / v0
   k_grp_tsum<<<ntc, 256, 0, st>>>(kin, N, s.tsum);
-  k_grp_choose<<<ntc, 256, 0, st>>>(kin, N, s.tsum, s.cincl, s.best, s.G, s.SG, s.count);
+  k_grp_choose<<<ntc, 256, 0, st>>>(kin, N, s.tsum, s.cincl, s.best, s.G, s.SG, s.count,
+                                 s.slots);
   k_grp_layout<<<(int)((N + 1 + 255) / 256), 256, 0, st>>>(vin, N, s.cincl, s.G, s.SG, perm,
                                                              gstart, gsize, s.slots);
   if (slot_counter) *slot_counter = s.slots;
@@ -1297,7 +1455,7 @@ fqt_status launch_bhq_groups(QuantArgs &a, bool bf16, int num_sms, cudaStream_t 
   if (a.C % 8) return FQT_EUNSUPPORTED;
   const int CO = a.C / 8;
   if (CO != 8 && CO != 16 && CO != 32) return FQT_EUNSUPPORTED;
-  const int grid = num_sms * 3;
+  const int grid = num_sms * (CO == 8 ? 2 : 3);  // resident (__launch_bounds__)
   const size_t smem = sizeof(int) * (size_t)a.C;
   const int64_t bgrid = big_grid(a.N);
   if (bgrid > 0x7fffffff) return FQT_EUNSUPPORTED;

@@ -122,3 +122,43 @@ def test_forward_row_sums(rows, cols, dtype):
     assert np.array_equal(codes, orc.quantize_fwd(X, 8)["codes"])
     assert np.array_equal(q.row_sum.cpu().numpy(), codes.sum(1))
     assert np.array_equal(q.col_sum.cpu().numpy(), codes.sum(0))
+
+
+@pytest.mark.parametrize("n", [3, 6, 37, 515, 3001])
+@pytest.mark.parametrize("c,rows,dtype", [(64, "equal", "f32"), (64, "outliers", "bf16"),
+                                          (64, "lognormal", "f32"), (128, "outliers", "f32")])
+def test_adaptive_group_sizes(n, c, rows, dtype):
+    """Groups of one to four rows side by side, larger ones alone, in one call."""
+    g = wl.rng(n + c)
+    dH = wl.random_grad(g, n, c, {"equal": 0.0, "outliers": 0.3, "lognormal": 2.0}[rows],
+                        0.05 if rows == "outliers" else 0.0)
+    if dtype == "bf16":
+        dH = wl.to_bf16_values(dH)
+    q2, q1 = fqt.quantize_grad(to_dev(dH, dtype), orc.BHQ, 5, 0, 11)
+    ref = orc.quantize_grad(dH, orc.BHQ, 5, 0, 11, orc.STREAM_B2, want_v=True)
+    h2 = q2.to_numpy()
+    assert np.array_equal(h2["perm"], ref["perm"])
+    _check_bhq_codes(h2["codes"], ref["codes"], ref["v"], 11)
+    assert np.array_equal(h2["row_sum"], h2["codes"].astype(np.int64).sum(1))
+    assert np.allclose(h2["zero"], ref["zero"], rtol=1e-5, atol=1e-4)
+    _check_b1(q1, dH, 11)
+
+
+@pytest.mark.parametrize("n,c,d", [(130, 16, 16), (3000, 24, 40), (777, 136, 200), (9001, 72, 24),
+                                   (40000, 16, 48), (60001, 336, 56)])
+def test_grad_w_reduction_shapes(n, c, d):
+    """Splits that do not divide into their groups, row lengths off a vector."""
+    g = wl.rng(n)
+    c, d = (c + 15) // 16 * 16, (d + 15) // 16 * 16
+    dH = to_dev(wl.random_grad(g, n, c), "f32")
+    X = to_dev(g.uniform(-1, 1, (n, d)).astype(np.float32), "f32")
+    _, q1 = fqt.quantize_grad(dH, orc.PSQ, 5, 0, 2)
+    qx = fqt.quantize_act(X, 8)
+    ws = fqt.Workspace(n, c, d)
+    _, gw = fqt.linear_backward(q1, q1, qx, None, grad_x=False, ws=ws)
+    assert fqt.sync_status(ws) == 0
+    ref = (torch.from_numpy(orc.dequant(q1.to_numpy())).cuda().T.double()
+           @ torch.from_numpy(orc.dequant(qx.to_numpy())).cuda().double()).cpu().numpy()
+    got = gw.double().cpu().numpy()
+    floor = 1e-3 * np.abs(ref).max(axis=1, keepdims=True)
+    assert (np.abs(got - ref) / np.maximum(np.abs(ref), floor)).max() <= 1e-3
