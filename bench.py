@@ -45,7 +45,7 @@ KIND, BITS, BLOCK = 2, 5, 16  # Q_b2 = BHQ-5, block 16
 SWEEP_BATCH = 256
 CALLS = ["quantize_act", "quantize_weight", "quantize_grad", "grad_x", "grad_w"]
 KERNELS = {"quantize_act": "k_range + k_fwd_codes", "quantize_weight": "k_range + k_fwd_codes",
-           "quantize_grad": "k_bhq_stats + k_bhq_codes + k_bhq_offsets", "grad_x": "k_gemm",
+           "quantize_grad": "k_bhq_stats + k_codes (+ k_bhq_offsets)", "grad_x": "k_gemm",
            "grad_w": "split-K k_gemm + k_reduce"}
 
 
@@ -211,16 +211,14 @@ def alg_bytes(N: int, C: int, D: int, eb: int = 4, block: int = BLOCK) -> dict:
 
 
 def launches(C: int, kind: int = KIND, block: int = BLOCK, implicit: bool = False) -> dict:
-    """Kernels each call launches (fixed by the library's dispatch): Q_f and
-    Q_theta are a range pass and a code pass; the fixed-block BHQ quantizer on
-    the widths of its two-pass form is a statistics pass, a code pass and the
-    grad_X offsets, on other widths a range pass, one fused pass and the
-    offsets (PTQ and PSQ: a range pass and one fused pass); grad_X is one
-    contraction, grad_W the split-K contraction and its reduction; an
-    implicit im2col X~ adds the column sums to Q_f and the padding sums to
-    grad_W."""
+    """Kernels each call launches at least (by the library's dispatch): Q_f and
+    Q_theta are a range pass and a code pass; the gradient quantizer is a
+    statistics pass (PTQ: a range pass) and a code pass (BHQ: and the grad_X
+    offsets where the code pass does not hold whole blocks); grad_X is one
+    contraction, grad_W the split-K contraction and its reduction; an implicit
+    im2col X~ adds the column sums to Q_f and the padding sums to grad_W."""
     return {"quantize_act": 3 if implicit else 2, "quantize_weight": 2,
-            "quantize_grad": 3 if kind == KIND else 2,
+            "quantize_grad": 2,
             "grad_x": 1, "grad_w": 3 if implicit else 2}
 
 

@@ -9,17 +9,10 @@
 // terms; between chunks the epilogue warps fold the accumulator into an
 // int32 running sum kept in tensor memory (tcgen05.st).
 //
-// Warp roles of the persistent kernel (320 threads, one CTA per SM):
-//   warp 0        TMA producer: fp16 operand tiles (128 x 64 per operand,
-//                 128-byte swizzle) into a ring of shared-memory stages
-//                 (cp.async.bulk.tensor, mbarrier transaction counts)
-//   warp 1        tensor-memory allocator and MMA issuer (one elected lane):
-//                 4 x tcgen05.mma.cta_group::1.kind::f16 (M128 N128 K16) per
-//                 stage into one of two TMEM accumulators, tcgen05.commit;
-//                 K-major and MN-major operands use the matching descriptors
-//   warps 2..9    epilogue: tcgen05.ld, dequantization (and the inverse
-//                 Householder of every BHQ block for grad_X), coalesced
-//                 16-byte stores of fp32 grad_X or int32 split-K partials
+// k_gemm and its epilogues are in fqt_gemm_core.cuh (warp roles there), the
+// CTA-pair instances and k_gemm_wide in fqt_gemm_pair.cu; here are the
+// single-CTA instances, the plans and the choice between them, k_reduce,
+// k_gradw, the padding sums and the adaptive groups' fix-up.
 // Every mbarrier wait is bounded; a wait that runs out records FQT_ETIMEOUT
 // and the CTA winds down.
 #include <cuda.h>

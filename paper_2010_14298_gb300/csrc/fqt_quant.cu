@@ -3,14 +3,19 @@
 //  k_range  : per-CTA (min, max) of a tensor and a non-finite flag (the
 //             dynamic range R(X) = max X - min X of Sec. 3.3); also clears
 //             the column-sum outputs the quantizer accumulates into.
-//  k_quant  : one templated kernel for
+//  k_fwd_codes : deterministic PTQ of the forward operands (Sec. 2.1).
+//  k_quant, k_quant2 : the one-pass gradient quantizers (k_quant2 stages its
+//             rows in shared memory), fused with the 8-bit stochastic PTQ Q_b1
+//             of App. E, for the shapes and workspaces that the passes of
+//             fqt_codes.cu leave to them (bhq_pass_order):
 //             KIND_PTQ  per-tensor stochastic quantizer (Sec. 3.3),
 //             KIND_PSQ  per-sample quantizer (Sec. 4.1),
-//             KIND_BHQ  block Householder quantizer (Sec. 4.2, App. D.4),
-//             KIND_DET  deterministic PTQ of the forward operands (Sec. 2.1),
-//             fused with the 8-bit stochastic PTQ Q_b1 of App. E.
+//             KIND_BHQ  block Householder quantizer (Sec. 4.2, App. D.4);
+//             KIND_DET  row sums of forward operands of odd widths.
+//  k_shift  : the power-of-two shift quantizer (Sec. 4.3).
+//  k_bhq_offsets : grad_X's offsets of fixed BHQ blocks.
 //
-// Thread mapping.  A row (sample) is handled by a team of TW consecutive
+// Thread mapping of k_quant.  A row (sample) is handled by a team of TW consecutive
 // threads; each thread owns OPT "octs" (8 consecutive columns) of the row,
 // octs cl, cl + TW, ...  Rows of a unit are spread over RL row lanes, RPL
 // rows per lane.  For BHQ a unit is one block of `block` rows and a CTA runs
