@@ -460,21 +460,24 @@ __global__ void __launch_bounds__(256) k_grp_layout(const int32_t *__restrict__ 
                                                     int32_t *perm, int32_t *gstart,
                                                     int32_t *gsize, unsigned *slots) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i > N) return;
   const int64_t G = *Gp;
+  int64_t e0 = 0, e1 = 0;
+  if (i < G) {
+    const double SG = (double)SGp->h + (double)SGp->l;
+    e0 = cum_size(i, N, G, SG, cincl);
+    e1 = cum_size(i + 1, N, G, SG, cincl);
+    if (e1 < e0) e1 = e0;
+  }
+  const int64_t k0 = i + e0, ns = e1 - e0;
+  // one past the last group of more than kSmallGroup rows
+  const unsigned lim =
+      __reduce_max_sync(0xffffffffu, ns + 1 > kSmallGroup ? (unsigned)i + 1u : 0u);
+  if (lim && (threadIdx.x & 31) == 0) atomicMax(slots + 1, lim);
+  if (i > N) return;
   if (i >= G) {
     gstart[i] = (int32_t)N;
     return;
   }
-  const double SG = (double)SGp->h + (double)SGp->l;
-  const int64_t e0 = cum_size(i, N, G, SG, cincl);
-  int64_t e1 = cum_size(i + 1, N, G, SG, cincl);
-  if (e1 < e0) e1 = e0;
-  const int64_t k0 = i + e0, ns = e1 - e0;
-  // one past the last group of more than kSmallGroup rows
-  const unsigned act = __activemask();
-  const unsigned lim = __reduce_max_sync(act, ns + 1 > kSmallGroup ? (unsigned)i + 1u : 0u);
-  if (lim && (threadIdx.x & 31) == __ffs(act) - 1) atomicMax(slots + 1, lim);
   gstart[i] = (int32_t)k0;
   perm[k0] = vals[i];
   for (int64_t t = 0; t < ns; ++t) perm[k0 + 1 + t] = vals[N - e1 + t];
