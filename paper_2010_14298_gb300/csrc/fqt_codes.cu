@@ -809,7 +809,8 @@ size_t sample_pass_bytes(int64_t N, int64_t C, int64_t rows_per_sample) {
 // it rounds the current one.  A block's w_j and scalars stay in registers
 // while the lane's rows belong to it.  A row's parts meet only in its row sums
 // (atomic when code_split > 1).  Units shrink with the tensor, down to 8 rows
-// and one slab, until there are enough for every warp of the GPU.
+// and one slab, until there are enough for every warp of the GPU (on the
+// smallest tensors down to 2 rows).
 // What bounds it: HBM on the largest tensors (802816 x 256 BHQ-5, 822 MB read
 // and as much written: 322 -> 305 us, 5.6 TB/s), the issue slots and the
 // integer pipe (two Philox streams) on those that L2 holds: packed operations,
@@ -1196,7 +1197,7 @@ static int codes_lpr(int C) {
 
 // Rows per unit and column parts of the code pass: about 64 units per SM
 // (four per warp), first by splitting wide rows into slabs, then by units of
-// 16 and 8 rows.
+// 16 and 8 rows, fewer where that leaves SMs idle.
 static void codes_plan(QuantArgs &a, int lpr, int num_sms, int *lg_urows, int lg_nb = 0) {
   const int nslab = (a.C + 16 * lpr - 1) / (16 * lpr);
   const int64_t target = (int64_t)num_sms * 64;
@@ -1204,6 +1205,14 @@ static void codes_plan(QuantArgs &a, int lpr, int num_sms, int *lg_urows, int lg
   auto units = [&]() { return ((a.N + (1 << lg) - 1) >> lg) * (int64_t)split; };
   while (split < nslab && units() < target) split *= 2;
   while (lg > 3 && units() < target) --lg;
+  // a small tensor: units of down to 2 rows (a warp's rows at a time at least)
+  // until there are eight per SM, but for blocks that a unit holds.  256 x 1008
+  // fp32 BHQ-5: 64 units of 8 rows on 8 SMs 11.4 us, 256 of 2 rows 5.7; 128 x
+  // 256 8.0 -> 4.6; 2471 x 208 8.3 -> 5.8
+  const int lg_min = std::max(1, 5 - (31 - __builtin_clz((unsigned)lpr)));
+  while (lg > lg_min && !(lg_nb && lg_nb <= 3) &&
+         units() < (int64_t)num_sms * 8)
+    --lg;
   // units of whole blocks hold what grad_X's offsets need: three per warp are
   // still enough (131072 x 64: code pass 21.9 -> 22.9 us without 3.7 + 2.5 for
   // k_bhq_offsets and its gap)
@@ -1224,9 +1233,12 @@ static cudaError_t launch_codes_t(const QuantArgs &a, const BhqBlock *bst, const
   auto kern = plain ? k_codes<T, LPR, MODE, true> : k_codes<T, LPR, MODE, false>;
   const size_t smem = sizeof(int) * (size_t)a.C;
   const int64_t nunits = ((a.N + (1 << lg_urows) - 1) >> lg_urows) * a.code_split;
-  // two CTAs of eight warps per SM (__launch_bounds__)
-  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((nunits + 7) / 8, 2 * num_sms));
-  kern<<<(int)grid, 256, smem, st>>>(a, bst, wsum, lg_nb, srec, rps, lg_urows);
+  // two CTAs of eight warps per SM (__launch_bounds__); four warps where the
+  // units would leave SMs idle
+  const int warps = nunits < (int64_t)num_sms * 8 ? 4 : 8;
+  const int64_t grid =
+      std::max<int64_t>(1, std::min<int64_t>((nunits + warps - 1) / warps, 2 * num_sms));
+  kern<<<(int)grid, 32 * warps, smem, st>>>(a, bst, wsum, lg_nb, srec, rps, lg_urows);
   return cudaGetLastError();
 }
 
