@@ -1164,6 +1164,9 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
     }
 #pragma unroll
     for (int u = 0; u < kFwdUnroll; ++u) {
+      // the lanes that take part in the row sums below, from all lanes of the
+      // warp (i0's trip count is the CTA's); the lanes of a row agree
+      const unsigned on = ROWS ? __ballot_sync(0xffffffffu, ok[u]) : 0u;
       if (!ok[u]) continue;
       uint32_t c[8];
 #pragma unroll
@@ -1182,9 +1185,8 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
         int v = 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) v += (int)c[j];
-        const unsigned act = __activemask();
         const int span = min(opr, 32);
-        for (int d = 1; d < span; d <<= 1) v += __shfl_xor_sync(act, v, d);
+        for (int d = 1; d < span; d <<= 1) v += __shfl_xor_sync(on, v, d);
         if ((lane & (span - 1)) == 0) atomicAdd(&row_sum[row[u]], v);
       }
     }
