@@ -1589,10 +1589,15 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
     }
     const bool conv_tile = cpw > 0;
     SplitPlan p = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true);
-    // the workspace holds the partials of at most 2.5 N slots: tiny images,
-    // which pad far beyond, take the splits that fit
-    if (conv_tile && 2 * Kt > 5 * Nr) {
-      const int64_t fit = plan_splits(C, D, (Nr * 5 + 1) / 2, a_bits, x_bits, nsm, true).splits;
+    // gemm_workspace_bytes counts the splits of N rows and of 2.5 N slots: tiny
+    // images, which pad far beyond, and plans in between that round to more
+    // splits than either (675 pixels in 960 slots: 15 against 14) take the
+    // splits that fit
+    const int64_t pad_bytes = conv ? C * qx->conv[4] * qx->conv[5] * 4 : 0;
+    if (conv_tile &&
+        (2 * Kt > 5 * Nr ||
+         (int64_t)kGemmOffset + p.splits * C * D * 4 + pad_bytes > (int64_t)ws_bytes)) {
+      const int64_t fit = plan_splits(C, D, (Nr * 5 + 1) / 2, a_bits, 8, nsm, true).splits;
       if (p.splits > fit) {
         p.ks_blocks = (p.kb_total + fit - 1) / fit;
         p.splits = (int)((p.kb_total + p.ks_blocks - 1) / p.ks_blocks);
@@ -1607,7 +1612,6 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
     const bool w_ok = use_gradw(wp, nsm) && conv && !conv_tile;
     if (conv && Nr > 0 && !w_ok && !conv_tile) return FQT_EUNSUPPORTED;
     // CTA pairs where their plan is faster and its partials fit the workspace
-    const int64_t pad_bytes = conv ? C * qx->conv[4] * qx->conv[5] * 4 : 0;
     bool pair = false;
     if (Nr > 0 && !w_ok && !bytes && C > BM) {
       const SplitPlan pp = plan_splits(C, D, Kt, a_bits, x_bits, nsm, true, true);

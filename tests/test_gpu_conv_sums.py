@@ -45,3 +45,22 @@ def test_conv_padding_sums(n, h, w, cin, cout):
     _, gi = fqt.linear_backward(q1, q1, qi, None, grad_x=False, ws=ws)
     assert fqt.sync_status(ws) == 0
     assert torch.equal(ge, gi)
+
+
+@pytest.mark.parametrize("n,h,w,cin,cout", [(5, 9, 15, 64, 256), (3, 19, 12, 64, 144),
+                                            (3, 39, 6, 64, 256)])
+def test_conv_grad_w_fits_its_workspace(n, h, w, cin, cout):
+    """Images whose padded slots would be cut into more splits than the
+    workspace of fqt_workspace_size holds: fewer splits, the same result."""
+    g = wl.rng(7)
+    x = g.uniform(-1, 1.5, (n, h, w, cin)).astype(np.float32)
+    X = torch.from_numpy(wl.im2col_nhwc(x, 3, 3, 1, 1)).cuda()
+    dH = torch.from_numpy(wl.random_grad(g, n * h * w, cout)).cuda()
+    _, q1 = fqt.quantize_grad(dH, fqt.PTQ, 8, 0, seed=1)
+    ws = fqt.Workspace(n * h * w, cout, 9 * cin)
+    qx = fqt.quantize_act(X, 8, ws=ws)
+    qi = fqt.quantize_act_conv(torch.from_numpy(x).cuda(), 3, 3, 1, 8, ws=ws)
+    _, ge = fqt.linear_backward(q1, q1, qx, None, grad_x=False, ws=ws)
+    _, gi = fqt.linear_backward(q1, q1, qi, None, grad_x=False, ws=ws)
+    assert fqt.sync_status(ws) == 0
+    assert torch.equal(ge, gi)
