@@ -44,19 +44,19 @@ static int int_attr(PyObject *o, int name, int32_t *out) {
   return PyErr_Occurred() ? -1 : 0;
 }
 
-/* the first two entries of a sequence of integers */
+/* the entries of a sequence of two integers */
 static int two_ints(PyObject *seq, int64_t *a, int64_t *b) {
   PyObject *f = PySequence_Fast(seq, "shape");
   if (!f) return -1;
-  int ok = PySequence_Fast_GET_SIZE(f) >= 2;
-  if (ok) {
+  if (PySequence_Fast_GET_SIZE(f) == 2) {
     *a = PyLong_AsLongLong(PySequence_Fast_GET_ITEM(f, 0));
     *b = PyLong_AsLongLong(PySequence_Fast_GET_ITEM(f, 1));
   } else {
-    PyErr_SetString(PyExc_ValueError, "a matrix is needed");
+    PyErr_Format(PyExc_ValueError, "a quantized tensor has two dimensions, not %zd",
+                 PySequence_Fast_GET_SIZE(f));
   }
   Py_DECREF(f);
-  return ok && !PyErr_Occurred() ? 0 : -1;
+  return PyErr_Occurred() ? -1 : 0;
 }
 
 /* A QTensor object as the C struct; NULL for None. */

@@ -1,0 +1,44 @@
+"""The native argument marshalling takes and refuses what QTensor.c_struct, the
+ctypes marshalling of the other calls, takes and refuses (no GPU: every call
+here is refused before the library would start a kernel)."""
+import types
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2010_14298_gb300 import fqt  # noqa: E402
+
+STREAM = types.SimpleNamespace(cuda_stream=0)
+
+
+def _qtensor(**fields):
+    q = fqt.QTensor.empty(4, 8, fqt.PTQ, 8, device="cpu")
+    for k, v in fields.items():
+        setattr(q, k, v)
+    return q
+
+
+def _marshal(q):
+    """A call that marshals q and that the library refuses (bits = 0)."""
+    return fqt.native().quantize_fwd(0, torch.zeros(4, 8), 0, 4, 8, 0, q,
+                                     torch.zeros(256, dtype=torch.uint8), 256, 0)
+
+
+def _same_refusal(q):
+    with pytest.raises(Exception) as ref:
+        q.c_struct()
+    with pytest.raises(ref.type):
+        _marshal(q)
+
+
+def test_a_whole_tensor_is_marshalled():
+    _qtensor().c_struct()
+    assert _marshal(_qtensor()) == 1  # FQT_EINVAL, from the library
+
+
+@pytest.mark.parametrize("fields", [
+    dict(codes=torch.zeros(2, 2, 8, dtype=torch.uint8)), dict(logical=(4, 8, 1)),
+    dict(codes=torch.zeros(32, dtype=torch.uint8)), dict(logical=(4,)), dict(logical=())])
+def test_codes_of_other_than_two_dimensions_are_refused(fields):
+    _same_refusal(_qtensor(**fields))
