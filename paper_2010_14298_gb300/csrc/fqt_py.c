@@ -25,15 +25,21 @@ static const char *const kNames[A_COUNT] = {
     "block", "rows_per_sample", "conv", "logical", "shape", "data_ptr"};
 static PyObject *g_name[A_COUNT];
 
-/* data_ptr() of a tensor (0 for None); -1 with an exception set on failure */
-static int tensor_ptr(PyObject *t, void **out) {
+/* data_ptr() of a tensor; -1 with an exception set on failure (AttributeError
+ * for None) */
+static int needed_ptr(PyObject *t, void **out) {
   *out = NULL;
-  if (t == Py_None) return 0;
   PyObject *v = PyObject_CallMethodNoArgs(t, g_name[A_DATA_PTR]);
   if (!v) return -1;
   *out = PyLong_AsVoidPtr(v);
   Py_DECREF(v);
   return PyErr_Occurred() ? -1 : 0;
+}
+
+/* the same with 0 for None */
+static int tensor_ptr(PyObject *t, void **out) {
+  *out = NULL;
+  return t == Py_None ? 0 : needed_ptr(t, out);
 }
 
 static int int_attr(PyObject *o, int name, int32_t *out) {
@@ -59,10 +65,9 @@ static int two_ints(PyObject *seq, int64_t *a, int64_t *b) {
   return PyErr_Occurred() ? -1 : 0;
 }
 
-/* A QTensor object as the C struct; NULL for None. */
+/* A QTensor object as the C struct (AttributeError for None). */
 static int fill(PyObject *q, fqt_qtensor *s, fqt_qtensor **out) {
   *out = NULL;
-  if (q == Py_None) return 0;
   memset(s, 0, sizeof(*s));
   void *p[A_POINTERS];
   PyObject *matrix = NULL; /* the codes whose shape is the tensor's */
@@ -70,7 +75,7 @@ static int fill(PyObject *q, fqt_qtensor *s, fqt_qtensor **out) {
   for (int i = 0; i < A_POINTERS && !bad; ++i) {
     PyObject *t = PyObject_GetAttr(q, g_name[i]);
     if (!t) { bad = 1; break; }
-    bad = tensor_ptr(t, &p[i]) != 0;
+    bad = (i == A_INV_S || i == A_ZERO ? needed_ptr(t, &p[i]) : tensor_ptr(t, &p[i])) != 0;
     if (!matrix && i <= A_CODES16 && t != Py_None) matrix = t;  /* keeps the reference */
     else Py_DECREF(t);
   }
@@ -123,6 +128,12 @@ static int fill(PyObject *q, fqt_qtensor *s, fqt_qtensor **out) {
   return 0;
 }
 
+/* The same for an operand that may be left out: NULL for None. */
+static int fill_optional(PyObject *q, fqt_qtensor *s, fqt_qtensor **out) {
+  *out = NULL;
+  return q == Py_None ? 0 : fill(q, s, out);
+}
+
 #define NARGS(k)                                                     \
   if (n != (k)) {                                                    \
     PyErr_SetString(PyExc_TypeError, "wrong number of arguments");   \
@@ -146,7 +157,7 @@ typedef struct {
 } Tail;
 
 static int tail(PyObject *const *a, Tail *t) {
-  if (tensor_ptr(a[0], &t->ws)) return -1;
+  if (needed_ptr(a[0], &t->ws)) return -1;
   t->bytes = PyLong_AsSize_t(a[1]);
   t->stream = PyLong_AsVoidPtr(a[2]);
   return PyErr_Occurred() ? -1 : 0;
@@ -196,8 +207,8 @@ static PyObject *py_quantize_grad_samples(PyObject *self, PyObject *const *a, Py
   const fqt_kind kind = (fqt_kind)INT(5);
   const int bits = INT(6);
   const uint64_t seed = PyLong_AsUnsignedLongLong(a[7]);
-  if (PyErr_Occurred() || tensor_ptr(a[0], &h) || fill(a[8], &s2, &q2) || fill(a[9], &s1, &q1) ||
-      tail(a + 10, &t))
+  if (PyErr_Occurred() || tensor_ptr(a[0], &h) || fill(a[8], &s2, &q2) ||
+      fill_optional(a[9], &s1, &q1) || tail(a + 10, &t))
     return NULL;
   CALL(fqt_quantize_grad_samples(h, dt, N, C, R, kind, bits, seed, q2, q1, t.ws, t.bytes,
                                  t.stream))
@@ -230,8 +241,8 @@ static PyObject *py_quantize_grad(PyObject *self, PyObject *const *a, Py_ssize_t
   const fqt_kind kind = (fqt_kind)INT(4);
   const int bits = INT(5), block = INT(6);
   const uint64_t seed = PyLong_AsUnsignedLongLong(a[7]);
-  if (PyErr_Occurred() || tensor_ptr(a[0], &h) || fill(a[8], &s2, &q2) || fill(a[9], &s1, &q1) ||
-      tail(a + 10, &t))
+  if (PyErr_Occurred() || tensor_ptr(a[0], &h) || fill(a[8], &s2, &q2) ||
+      fill_optional(a[9], &s1, &q1) || tail(a + 10, &t))
     return NULL;
   CALL(fqt_quantize_grad(h, dt, N, C, kind, bits, block, seed, q2, q1, t.ws, t.bytes, t.stream))
 }
@@ -243,8 +254,9 @@ static PyObject *py_linear_backward(PyObject *self, PyObject *const *a, Py_ssize
   fqt_qtensor s[4], *q[4];
   void *gx, *gw;
   Tail t;
-  for (int i = 0; i < 4; ++i)
-    if (fill(a[i], &s[i], &q[i])) return NULL;
+  if (fill(a[0], &s[0], &q[0])) return NULL;
+  for (int i = 1; i < 4; ++i)
+    if (fill_optional(a[i], &s[i], &q[i])) return NULL;
   if (tensor_ptr(a[4], &gx) || tensor_ptr(a[5], &gw) || tail(a + 6, &t)) return NULL;
   CALL(fqt_linear_backward(q[0], q[1], q[2], q[3], gx, gw, t.ws, t.bytes, t.stream))
 }

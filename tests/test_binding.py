@@ -42,3 +42,19 @@ def test_a_whole_tensor_is_marshalled():
     dict(codes=torch.zeros(32, dtype=torch.uint8)), dict(logical=(4,)), dict(logical=())])
 def test_codes_of_other_than_two_dimensions_are_refused(fields):
     _same_refusal(_qtensor(**fields))
+
+
+@pytest.mark.parametrize("fields", [dict(inv_s=None), dict(zero=None),
+                                    dict(codes=None, codes16=None)])
+def test_missing_arrays_are_refused(fields):
+    _same_refusal(_qtensor(**fields))
+
+
+def test_missing_operands_and_workspaces_are_refused():
+    ws = fqt.Workspace(4, 16, 16, device="cpu")
+    with pytest.raises(AttributeError):  # no W~
+        fqt.conv_grad_x_nhwc(_qtensor(), None, 1, 2, 2, 32, ws=ws, stream=STREAM,
+                             out=torch.zeros(1, 2, 2, 32))
+    ws.buf = None
+    with pytest.raises(AttributeError):
+        fqt.quantize_act(torch.zeros(4, 8), 0, ws=ws, out=_qtensor(), stream=STREAM)
