@@ -96,16 +96,15 @@ static int fill(PyObject *q, fqt_qtensor *s, fqt_qtensor **out) {
     return -1;
   PyObject *conv = PyObject_GetAttr(q, g_name[A_CONV]);
   if (!conv) return -1;
-  if (conv != Py_None) {
-    PyObject *f = PySequence_Fast(conv, "conv");
-    if (f && PySequence_Fast_GET_SIZE(f) == 8) {
-      for (int i = 0; i < 8; ++i)
-        s->conv[i] = (int32_t)PyLong_AsLong(PySequence_Fast_GET_ITEM(f, i));
-    } else if (f) {
-      PyErr_SetString(PyExc_ValueError, "conv holds eight integers");
-    }
-    Py_XDECREF(f);
+  const int given = PyObject_IsTrue(conv); /* None or empty: not a conv operand */
+  PyObject *f = given > 0 ? PySequence_Fast(conv, "conv") : NULL;
+  if (f && PySequence_Fast_GET_SIZE(f) <= 8) {
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(f); ++i)
+      s->conv[i] = (int32_t)PyLong_AsLong(PySequence_Fast_GET_ITEM(f, i));
+  } else if (f) {
+    PyErr_SetString(PyExc_IndexError, "conv holds eight integers");
   }
+  Py_XDECREF(f);
   Py_DECREF(conv);
   if (PyErr_Occurred()) return -1;
   s->codes = p[A_CODES];

@@ -58,3 +58,16 @@ def test_missing_operands_and_workspaces_are_refused():
     ws.buf = None
     with pytest.raises(AttributeError):
         fqt.quantize_act(torch.zeros(4, 8), 0, ws=ws, out=_qtensor(), stream=STREAM)
+
+
+@pytest.mark.parametrize("conv", [(), [], (1, 2, 3), tuple(range(8))])
+def test_conv_geometries_are_taken(conv):
+    """An empty geometry is an ordinary matrix's, a short one ends in zeros."""
+    q = _qtensor(conv=conv)
+    q.c_struct()
+    assert _marshal(q) == 1
+
+
+@pytest.mark.parametrize("conv", [tuple(range(9)), (1.5,) * 8, ("a",)])
+def test_conv_geometries_that_do_not_fit_are_refused(conv):
+    _same_refusal(_qtensor(conv=conv))
