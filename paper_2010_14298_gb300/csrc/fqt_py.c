@@ -99,7 +99,7 @@ static int fill(PyObject *q, fqt_qtensor *s, fqt_qtensor **out) {
   const int given = PyObject_IsTrue(conv); /* None or empty: not a conv operand */
   PyObject *f = given > 0 ? PySequence_Fast(conv, "conv") : NULL;
   if (f && PySequence_Fast_GET_SIZE(f) <= 8) {
-    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(f); ++i)
+    for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(f) && !PyErr_Occurred(); ++i)
       s->conv[i] = (int32_t)PyLong_AsLong(PySequence_Fast_GET_ITEM(f, i));
   } else if (f) {
     PyErr_SetString(PyExc_IndexError, "conv holds eight integers");
