@@ -11,6 +11,7 @@ from __future__ import annotations
 import ctypes
 import importlib.machinery
 import importlib.util
+import operator
 import os
 import threading
 from dataclasses import dataclass
@@ -169,6 +170,13 @@ def _dtype_code(t: torch.Tensor) -> int:
     if t.dtype == torch.bfloat16:
         return BF16
     raise TypeError(f"unsupported dtype {t.dtype}")
+
+
+def _seed(seed) -> int:
+    """An integer modulo 2^64 (no tensor: reading it would wait for the device)."""
+    if isinstance(seed, torch.Tensor):
+        raise TypeError("the seed is an integer, not a tensor")
+    return operator.index(seed) & (2 ** 64 - 1)
 
 
 class Workspace:
@@ -386,7 +394,7 @@ def quantize_grad(dH: torch.Tensor, kind: int, bits: int, block: int = 0,
     if with_b1 and q_b1 is None:
         q_b1 = QTensor.empty(N, C, PTQ, 8, 0, False, True, dH.device)
     st = native().quantize_grad(dH, _dtype_code(dH), N, C, kind, bits,
-                                block if kind == BHQ else 0, int(seed) & (2 ** 64 - 1), q_b2,
+                                block if kind == BHQ else 0, _seed(seed), q_b2,
                                 q_b1 if with_b1 else None, ws.buf, ws.nbytes,
                                 _raw_stream(stream))
     if st:
@@ -411,7 +419,7 @@ def quantize_grad_samples(dH: torch.Tensor, rows_per_sample: int, kind: int, bit
     if with_b1 and q_b1 is None:
         q_b1 = QTensor.empty(N, C, PTQ, 8, 0, False, True, dH.device)
     st = native().quantize_grad_samples(dH, _dtype_code(dH), N, C, rows_per_sample, kind, bits,
-                                        int(seed) & (2 ** 64 - 1), q_b2,
+                                        _seed(seed), q_b2,
                                         q_b1 if with_b1 else None, ws.buf, ws.nbytes,
                                         _raw_stream(stream))
     if st:

@@ -3,6 +3,7 @@ ctypes marshalling of the other calls, takes and refuses (no GPU: every call
 here is refused before the library would start a kernel)."""
 import types
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -71,3 +72,23 @@ def test_conv_geometries_are_taken(conv):
 @pytest.mark.parametrize("conv", [tuple(range(9)), (1.5,) * 8, ("a",)])
 def test_conv_geometries_that_do_not_fit_are_refused(conv):
     _same_refusal(_qtensor(conv=conv))
+
+
+@pytest.mark.parametrize("samples", [False, True])
+@pytest.mark.parametrize("seed", [1.9, "7", None, torch.tensor(7), torch.tensor([7])])
+def test_seeds_that_are_no_integers_are_refused(seed, samples):
+    """A tensor too: reading it would wait for the device."""
+    dH = torch.zeros(4, 64)
+    kw = dict(seed=seed, ws=fqt.Workspace(4, 64, 16, device="cpu"), stream=STREAM,
+              q_b2=fqt.QTensor.empty(4, 64, fqt.PTQ, 8, device="cpu"), with_b1=False)
+    with pytest.raises(TypeError):
+        if samples:
+            fqt.quantize_grad_samples(dH, 2, fqt.PTQ, 9, **kw)
+        else:
+            fqt.quantize_grad(dH, fqt.PTQ, 9, **kw)
+
+
+@pytest.mark.parametrize("seed", [0, -1, 2 ** 64 - 1, 2 ** 70 + 3, True, np.int64(-5),
+                                  np.uint64(2 ** 64 - 1)])
+def test_integer_seeds_are_taken_modulo_2_64(seed):
+    assert fqt._seed(seed) == int(seed) % 2 ** 64
