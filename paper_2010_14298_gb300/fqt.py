@@ -149,13 +149,16 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 # The raw handle of the current device's current stream (building the stream
-# object that torch.cuda.current_stream() returns took 2.9 us per call).
-_current_raw_stream = torch._C._cuda_getCurrentRawStream
-_current_device = torch._C._cuda_getDevice
+# object that torch.cuda.current_stream() returns took 2.9 us per call); a
+# PyTorch built without CUDA lacks the two functions.
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _raw_stream(stream) -> int:
     if stream is None:
+        if _current_raw_stream is None or _current_device is None:
+            return torch.cuda.current_stream().cuda_stream
         return _current_raw_stream(_current_device())
     return stream.cuda_stream
 

@@ -1,6 +1,9 @@
 """The native argument marshalling takes and refuses what QTensor.c_struct, the
 ctypes marshalling of the other calls, takes and refuses (no GPU: every call
 here is refused before the library would start a kernel)."""
+import os
+import subprocess
+import sys
 import types
 
 import numpy as np
@@ -10,6 +13,7 @@ torch = pytest.importorskip("torch")
 
 from paper_2010_14298_gb300 import fqt  # noqa: E402
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 STREAM = types.SimpleNamespace(cuda_stream=0)
 
 
@@ -92,3 +96,14 @@ def test_seeds_that_are_no_integers_are_refused(seed, samples):
                                   np.uint64(2 ** 64 - 1)])
 def test_integer_seeds_are_taken_modulo_2_64(seed):
     assert fqt._seed(seed) == int(seed) % 2 ** 64
+
+
+def test_the_module_imports_without_torchs_cuda_bindings():
+    """A PyTorch built without CUDA lacks the raw-stream functions."""
+    code = ("import torch\n"
+            "for n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    delattr(torch._C, n)\n"
+            "from paper_2010_14298_gb300 import fqt\n"
+            "assert fqt.status_string(0) == 'ok'\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
