@@ -1,9 +1,11 @@
 """Builds the CUDA library paper_2010_14298_gb300/_lib/libfqt.so for sm_103a.
 
 Each translation unit is compiled by nvcc in parallel, then linked into one
-shared object with a plain C ABI (include/fqt.h); the Python binding's native
-marshalling (csrc/fqt_py.c) is a small extension module linked against it.  Run as a script or call
-``build()``; an up-to-date library is not rebuilt.
+shared object with a plain C ABI (include/fqt.h).  The Python binding's native
+marshalling (csrc/fqt_py.c) is a small extension module linked against it, named
+for the interpreter it is built for; where it cannot be built (no C compiler, no
+Python.h) the binding marshals through ctypes.  Run as a script or call
+``build()``; what is up to date is not rebuilt.
 """
 from __future__ import annotations
 
@@ -13,6 +15,7 @@ import shutil
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -20,7 +23,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIBDIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(LIBDIR, "libfqt.so")
-PYEXT = os.path.join(LIBDIR, "_fqt_py.so")
+# another interpreter finds no extension module under its own name
+PYEXT = os.path.join(LIBDIR, "_fqt_py" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["fqt_quant.cu", "fqt_codes.cu", "fqt_group.cu", "fqt_gemm.cu", "fqt_gemm_pair.cu", "fqt_conv.cu",
            "fqt_api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -35,26 +39,59 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
-def _inputs():
-    files = [os.path.join(CSRC, s) for s in SOURCES]
-    files += [os.path.join(CSRC, f) for f in os.listdir(CSRC)
-              if f.endswith((".cuh", ".h", ".c"))]
-    files.append(os.path.join(INCLUDE, "fqt.h"))
-    files.append(os.path.abspath(__file__))
-    return files
+def _fresh(target, inputs) -> bool:
+    if not os.path.exists(target):
+        return False
+    t = os.path.getmtime(target)
+    inputs = [*inputs, os.path.join(INCLUDE, "fqt.h"), os.path.abspath(__file__)]
+    return all(os.path.getmtime(f) <= t for f in inputs)
+
+
+def library_up_to_date() -> bool:
+    return _fresh(LIB, [os.path.join(CSRC, s) for s in SOURCES]
+                  + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))])
+
+
+def extension_up_to_date() -> bool:
+    return _fresh(PYEXT, [os.path.join(CSRC, "fqt_py.c")])
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(PYEXT):
+    return library_up_to_date() and extension_up_to_date()
+
+
+def build_extension() -> bool:
+    """Builds the extension module; a warning and False where it cannot be."""
+    tmp = PYEXT + f".tmp{os.getpid()}"
+    cmd = [shutil.which("gcc") or shutil.which("cc") or "gcc", "-O2", "-std=c11", "-shared",
+           "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+           os.path.join(CSRC, "fqt_py.c"), "-o", tmp, "-L", LIBDIR, "-l:libfqt.so",
+           "-Wl,-rpath,$ORIGIN"]
+    try:
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        why = (r.stdout + r.stderr or f"exit status {r.returncode}") if r.returncode else ""
+    except OSError as e:
+        why = str(e)
+    if why:
+        if os.path.exists(PYEXT):  # of other sources: not to be loaded
+            os.remove(PYEXT)
+        warnings.warn("the Python extension module was not built, the binding marshals through "
+                      f"ctypes:\n{why}", RuntimeWarning, stacklevel=2)
         return False
-    t = min(os.path.getmtime(LIB), os.path.getmtime(PYEXT))
-    return all(os.path.getmtime(f) <= t for f in _inputs())
+    os.replace(tmp, PYEXT)
+    return True
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and up_to_date():
-        return LIB
     os.makedirs(LIBDIR, exist_ok=True)
+    if force or not library_up_to_date():
+        _build_library(verbose)
+    if force or not extension_up_to_date():
+        build_extension()
+    return LIB
+
+
+def _build_library(verbose: bool) -> None:
     nvcc = _nvcc()
     objs = []
 
@@ -78,16 +115,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
-    tmp = PYEXT + f".tmp{os.getpid()}"
-    cmd = [shutil.which("gcc") or "gcc", "-O2", "-std=c11", "-shared", "-fPIC",
-           "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
-           os.path.join(CSRC, "fqt_py.c"), "-o", tmp, "-L", LIBDIR, "-l:libfqt.so",
-           "-Wl,-rpath,$ORIGIN"]
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(f"building the Python extension failed:\n{r.stdout}\n{r.stderr}")
-    os.replace(tmp, PYEXT)
-    return LIB
 
 
 if __name__ == "__main__":

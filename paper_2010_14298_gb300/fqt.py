@@ -1,8 +1,9 @@
 """Binding of the C ABI in include/fqt.h.
 
-Argument marshalling only, by the extension module ``_lib/_fqt_py.so`` for the
-calls of a training step and by ctypes for the others: every step of the hot
-path runs in the CUDA library ``_lib/libfqt.so``.  PyTorch provides device memory and streams.
+Argument marshalling only, by the extension module ``_lib/_fqt_py*.so`` for the
+calls of a training step and by ctypes for the others (and for all of them where
+the extension module cannot be built): every step of the hot path runs in the
+CUDA library ``_lib/libfqt.so``.  PyTorch provides device memory and streams.
 There is no CPU fallback: if the library is missing or no GPU is present the
 calls raise.
 """
@@ -63,7 +64,7 @@ def load(build_if_missing: bool = True):
         if _lib is not None:
             return _lib
         path = _build.LIB
-        if not (os.path.exists(path) and os.path.exists(_build.PYEXT)):
+        if not os.path.exists(path):
             if not build_if_missing:
                 raise FileNotFoundError(f"{path} is not built")
             _build.build()
@@ -121,19 +122,44 @@ def load(build_if_missing: bool = True):
         return lib
 
 
+class _CtypesCalls:
+    """The calls of the extension module, marshalled through ctypes."""
+
+    def __init__(self, lib):
+        self._lib = lib
+
+    def __getattr__(self, name):
+        f = getattr(self._lib, "fqt_" + name)
+        return lambda *args: f(*map(_c_arg, args))
+
+    def quantize_fwd(self, weight, *args):
+        return getattr(self, "quantize_weight" if weight else "quantize_act")(*args)
+
+
+def _c_arg(a):
+    if isinstance(a, torch.Tensor):
+        return ctypes.c_void_p(a.data_ptr())
+    return ctypes.byref(a.c_struct()) if isinstance(a, QTensor) else a
+
+
 def native():
-    """The extension module that marshals the calls of a training step."""
+    """The calls of a training step: the extension module that marshals them
+    natively (built when absent), or the same calls through ctypes where it
+    cannot be built."""
     global _native
     if _native is None:
-        load()
+        lib = load()
         with _lock:
             if _native is None:
-                loader = importlib.machinery.ExtensionFileLoader("_fqt_py", _build.PYEXT)
-                spec = importlib.util.spec_from_file_location("_fqt_py", _build.PYEXT,
-                                                              loader=loader)
-                mod = importlib.util.module_from_spec(spec)
-                loader.exec_module(mod)
-                _native = mod
+                if os.path.exists(_build.PYEXT) or _build.build_extension():
+                    loader = importlib.machinery.ExtensionFileLoader("_fqt_py", _build.PYEXT)
+                    spec = importlib.util.spec_from_file_location("_fqt_py", _build.PYEXT,
+                                                                  loader=loader)
+                    mod = importlib.util.module_from_spec(spec)
+                    loader.exec_module(mod)
+                    _native = mod
+                else:
+                    _native = _CtypesCalls(lib)
     return _native
 
 

@@ -4,14 +4,16 @@ here is refused before the library would start a kernel)."""
 import os
 import subprocess
 import sys
+import sysconfig
 import types
+from shutil import which
 
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2010_14298_gb300 import fqt  # noqa: E402
+from paper_2010_14298_gb300 import build, fqt  # noqa: E402
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 STREAM = types.SimpleNamespace(cuda_stream=0)
@@ -107,3 +109,49 @@ def test_the_module_imports_without_torchs_cuda_bindings():
             "assert fqt.status_string(0) == 'ok'\n")
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+# --- the extension module is built for one interpreter, and can be absent ---
+def test_the_extension_module_serves_the_calls_here():
+    """Built by this interpreter, under a name that no other one loads."""
+    assert isinstance(fqt.native(), types.ModuleType)
+    assert build.PYEXT.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+@pytest.fixture
+def no_extension(monkeypatch, tmp_path):
+    """The library is built, the extension module is not and cannot be."""
+    build.build()
+    monkeypatch.setattr(build, "PYEXT", str(tmp_path / "_fqt_py.so"))
+    monkeypatch.setattr(build.shutil, "which",
+                        lambda name, *a: None if name in ("cc", "gcc") else which(name, *a))
+    monkeypatch.setenv("PATH", str(tmp_path))
+    monkeypatch.setattr(fqt, "_native", None)
+
+
+def test_build_leaves_a_whole_library_without_a_c_compiler(no_extension):
+    with pytest.warns(RuntimeWarning):
+        assert build.build() == build.LIB
+
+
+def test_the_library_loads_without_the_extension_module(no_extension, monkeypatch):
+    monkeypatch.setattr(fqt, "_lib", None)
+    monkeypatch.setattr(build, "build", lambda *a, **k: pytest.fail("the library was rebuilt"))
+    assert fqt.load(build_if_missing=False).fqt_workspace_size(4, 8, 16) > 0
+
+
+def test_the_calls_are_made_through_ctypes_without_the_extension_module(no_extension):
+    want = fqt.workspace_size(1000, 64, 576)
+    with pytest.warns(RuntimeWarning):
+        calls = fqt.native()
+    assert calls.workspace_size(1000, 64, 576) == want
+    assert _marshal(_qtensor()) == 1
+    _same_refusal(_qtensor(logical=(4, 8, 1)))
+    q, ws = _qtensor(), fqt.Workspace(4, 16, 16, device="cpu")
+    with pytest.raises(fqt.FqtError) as e:  # k = 5 is not built
+        fqt.conv_grad_x_nhwc(q, q, 1, 2, 2, 32, k=5, ws=ws, stream=STREAM,
+                             out=torch.zeros(1, 2, 2, 32))
+    assert e.value.status in (1, 2)
+    with pytest.raises(fqt.FqtError) as e:  # W~ of other rows than dH's columns
+        fqt.linear_backward(q, None, None, q, grad_w=False, ws=ws, stream=STREAM)
+    assert e.value.status in (1, 2, 6)
