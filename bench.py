@@ -20,7 +20,8 @@ is needed between steps.
 The reference arm times the CPU oracle on a bounded sample of the same
 workload (every layer at batch 1) on all host cores.  The other workloads
 (the linear layer, the ResNet-18 and ResNet-50 layer3 convs, the transformer
-FFN pair) and the method's variants are reported as extras.
+FFN pair) and the method's variants are reported as extras, in the file that
+holds the per-layer times and the rooflines (--details).
 """
 from __future__ import annotations
 
@@ -379,6 +380,24 @@ def roofline_of(call: str, rows, hbm_peak: float, bf16_peak: float):
     return out
 
 
+# Parts of the result that go to a file: with them the line is 24 KB long, and a
+# log that keeps its last few KB loses the headline at its start.
+DETAILS = ("rooflines", "per_layer_ms", "slowest_layers", "extras")
+
+
+def report(result: dict, path: str) -> None:
+    """Prints the result as one JSON line and writes its details to `path`."""
+    details = {k: result[k] for k in DETAILS if k in result}
+    line = {k: v for k, v in result.items() if k not in DETAILS}
+    try:
+        with open(path, "w") as f:
+            json.dump(details, f, indent=1)
+        line["details"] = path
+    except OSError as e:
+        line["details"] = f"not written: {e}"
+    print(json.dumps(line), flush=True)
+
+
 def run_gpu(args):
     import torch
     import torch.distributed as dist
@@ -528,7 +547,7 @@ def run_gpu(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         result["cpu_baseline"] = cpu_baseline(args.cpu_batch)
     if rank == 0:
-        print(json.dumps(result), flush=True)
+        report(result, args.details)
     if world > 1:
         dist.destroy_process_group()
 
@@ -966,6 +985,8 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-extras", dest="extras", action="store_false",
                     help="skip the other workloads and the variants")
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for the per-layer times, the rooflines and the extras")
     ap.add_argument("--extra-steps", type=int, default=10,
                     help="timed rounds per call of the other workloads")
     args = ap.parse_args()
