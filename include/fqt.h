@@ -372,6 +372,20 @@ FQT_API fqt_status fqt_debug_wait_timeout(void *workspace, size_t ws_bytes,
 FQT_API fqt_status fqt_debug_mma_peak(int kind, int64_t iters, double *ops_out,
                                       void *workspace, size_t ws_bytes, void *stream);
 
+/* The kernel that this host thread's last contraction was dispatched to, for
+ * tests that aim at one: which = 0 for grad_X or the forward, 1 for grad_W (or
+ * a raw integer product).  out holds five entries:
+ *   [0] 0 none yet, 1 single CTAs, 2 CTA pairs, 3 wide column tiles (at most
+ *       128 rows of grad_W), 4 one exact chunk per CTA (implicit im2col rows of
+ *       more than 64 pixels);
+ *   [1] grad_X: form of the integer parts, 0 int32, 1 fp32 or int32 by the
+ *       tile, 2 fp32; else 0;
+ *   [2] splits of the reduction;
+ *   [3] 1 if the contraction dequantizes grad_W itself (one split);
+ *   [4] wide tiles: taps of a kernel row that share their pixels, or 0.
+ * Has no counterpart in the paper. */
+FQT_API fqt_status fqt_debug_last_plan(int which, int32_t *out);
+
 /* Static description of a status code. */
 FQT_API const char *fqt_status_string(fqt_status status);
 

@@ -549,6 +549,14 @@ fqt_status fqt_debug_mma_peak(int kind, int64_t iters, double *ops_out, void *wo
                         reinterpret_cast<cudaStream_t>(stream));
 }
 
+fqt_status fqt_debug_last_plan(int which, int32_t *out) {
+  if ((which != 0 && which != 1) || !out) return FQT_EINVAL;
+  const LastPlan &p = last_plan(which);
+  const int32_t v[5] = {p.kernel, p.form, p.splits, p.fused, p.row_taps};
+  memcpy(out, v, sizeof(v));
+  return FQT_OK;
+}
+
 size_t fqt_conv_grad_x_workspace_size(int64_t cin) { return conv_grad_x_ws_bytes(cin); }
 
 fqt_status fqt_conv_grad_x_nhwc(const fqt_qtensor *q_b2, const fqt_qtensor *qw, int64_t n,

@@ -382,6 +382,10 @@ static GemmKernel gemm_kernel(int mode, int nb, int form) {
   return nullptr;
 }
 
+static thread_local LastPlan g_last_plan[2];
+
+const LastPlan &last_plan(int which) { return g_last_plan[which]; }
+
 // Launches the contraction of fp16 carrier operands: A is M x K (stored
 // M x K if a_kmajor, else K x M), B is the K x N operand (stored N x K if
 // b_kmajor, else K x N).  Partials: out is splits x M x N int32.  grad_X:
@@ -420,6 +424,8 @@ static fqt_status run_gemm(const void *A, int a_kmajor, int a_bits, const void *
   if (!ok) return cuda_fail(cudaErrorInvalidValue, "tensor map encode");
   GemmKernel kern = pair ? gemm_pair_kernel(mode, nb, form) : gemm_kernel(mode, nb, form);
   if (!kern) return FQT_EUNSUPPORTED;
+  g_last_plan[partial] = {wide ? PLAN_WIDE : pair ? PLAN_PAIR : PLAN_SINGLE, partial ? 0 : form,
+                          p.splits, g.fuse, wide ? g.taps : 0};
   const bool four = !partial && form == 2;  // GemmLayout: four epilogue sets
   using LP = GemmLayout<1, 0, 1, true>;
   const int threads = partial && pair ? LP::threads
@@ -962,6 +968,7 @@ static fqt_status run_gradw(const uint16_t *X16, const uint16_t *Q16, int64_t K,
   const cudaError_t ea =
       cudaFuncSetAttribute(k_gradw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
   if (ea != cudaSuccess) return cuda_fail(ea, "grad_W shared-memory attribute");
+  g_last_plan[1] = {PLAN_GRADW, 0, p.splits, 0, 0};
   const int nsm = device_sm_count();
   const int grid = p.splits < nsm ? p.splits : nsm;
   k_gradw<<<grid, kWThreads, p.smem, st>>>(tx, tq, w);

@@ -108,6 +108,13 @@ int device_sm_count();
 // FQT_ECUDA, or FQT_OK for cudaSuccess.
 fqt_status cuda_fail(cudaError_t e, const char *where);
 
+// What a contraction was dispatched to (fqt_debug_last_plan), per host thread.
+enum { PLAN_SINGLE = 1, PLAN_PAIR = 2, PLAN_WIDE = 3, PLAN_GRADW = 4 };
+struct LastPlan {
+  int32_t kernel, form, splits, fused, row_taps;
+};
+const LastPlan &last_plan(int which);
+
 size_t gemm_workspace_bytes(int64_t N, int64_t C, int64_t D);
 size_t debug_workspace_bytes(int64_t M, int64_t N, int64_t K);
 fqt_status grad_w_fixed_scratch(const fqt_qtensor *qa, const fqt_qtensor *qx,

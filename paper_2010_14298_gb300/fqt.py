@@ -114,6 +114,8 @@ def load(build_if_missing: bool = True):
         lib.fqt_debug_int_gemm.restype = i32
         lib.fqt_debug_int_gemm_u8.argtypes = [P, i32, P, i32, i64, i64, i64, P, P, sz, P]
         lib.fqt_debug_int_gemm_u8.restype = i32
+        lib.fqt_debug_last_plan.argtypes = [i32, ctypes.POINTER(ctypes.c_int32)]
+        lib.fqt_debug_last_plan.restype = i32
         lib.fqt_status_string.argtypes = [i32]
         lib.fqt_status_string.restype = ctypes.c_char_p
         lib.fqt_last_cuda_error.argtypes = []
@@ -601,6 +603,14 @@ def debug_mma_peak(kind: int, iters: int, ws: Workspace, stream=None) -> float:
     _check(load().fqt_debug_mma_peak(kind, iters, ctypes.byref(ops), ws.ptr, ws.nbytes,
                                      _stream(stream)), "fqt_debug_mma_peak")
     return ops.value
+
+
+def debug_last_plan(grad_w: bool = False) -> dict:
+    """What this thread's last grad_X (or forward) or grad_W was dispatched to."""
+    out = (ctypes.c_int32 * 5)()
+    _check(load().fqt_debug_last_plan(int(grad_w), out), "fqt_debug_last_plan")
+    kernel = ("none", "single", "pair", "wide", "gradw")[out[0]]
+    return dict(kernel=kernel, form=out[1], splits=out[2], fused=bool(out[3]), row_taps=out[4])
 
 
 def status_string(code: int) -> str:

@@ -228,3 +228,18 @@ def test_sample_and_nhwc_refusals_without_gpu():
     assert lib.fqt_conv_grad_x_nhwc(ctypes.byref(q2), ctypes.byref(qw), 2, 8, 8, 32, 3, 1, out, p,
                                      64, None) == 6  # workspace too small
     del raw
+
+
+def test_last_plan_without_gpu():
+    """No contraction was dispatched yet in this thread; other slots than the two
+    and no place for the answer are refused."""
+    import threading
+    from paper_2010_14298_gb300 import fqt
+    seen = []
+    t = threading.Thread(target=lambda: seen.append(fqt.debug_last_plan(grad_w=True)))
+    t.start()
+    t.join()
+    assert seen == [dict(kernel="none", form=0, splits=0, fused=False, row_taps=0)]
+    out = (ctypes.c_int32 * 5)()
+    assert fqt.load().fqt_debug_last_plan(2, out) == 1
+    assert fqt.load().fqt_debug_last_plan(0, None) == 1

@@ -24,7 +24,7 @@ def test_conv_column_sums(n, h, w, c, dtype):
     X = torch.from_numpy(wl.im2col_nhwc(x.float().numpy(), 3, 3, 1, 1))
     ws = fqt.Workspace(n * h * w, c, 16)
     qe = fqt.quantize_act(X.cuda(), 8)
-    for _ in range(2):  # the second call finds the counter as the first left it
+    for _ in range(2):  # the second call finds the first one's sums in the workspace
         qi = fqt.quantize_act_conv(x.cuda(), 3, 3, 1, 8, ws=ws)
         assert fqt.sync_status(ws) == 0
         assert torch.equal(qi.col_sum[:-1], qe.col_sum)
