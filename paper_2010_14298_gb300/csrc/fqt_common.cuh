@@ -71,8 +71,9 @@ __device__ __forceinline__ uint32_t u16_of(const uint4 &w, int i) {
 
 // Stochastic rounding of v >= 0 onto 0..B (Sec. 3.3): the probability
 // frac(v) is realised in 16-bit fixed point, code = (floor(v 2^16) + u) >> 16.
-// sr_code16 takes v * 2^16 (scaling by 2^16 is exact, so callers may fold it
-// into their scale factor).
+// sr_code16 takes v * 2^16.  (The product v is scaled and not its scale factor
+// s = B / R, which would overflow from 2^112 on, that is for ranges R below
+// 5e-32, and gave code B for every entry of such a row or tensor.)
 // floor(v16) is read off the fp32 bits (integer shift of the significand by
 // the exponent, no conversion instruction): v16 is capped at 2^24 - 1, which
 // leaves every code unchanged (a capped v gives code B either way), so the

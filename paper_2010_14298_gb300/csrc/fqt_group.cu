@@ -587,7 +587,6 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
   const uint32_t B2 = (1u << a.bits) - 1u;
   const uint32_t og2 = (B2 + 1u) >> 1;
   const float s_g1 = affine_scale(gmin, gmax, 255u);
-  const float s_g1_16 = __fmul_rn(s_g1, 65536.0f);
   const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
   if (blockIdx.x == 0 && tid == 0 && has_b1) {
     a.inv1[0] = __fdiv_rn(1.0f, s_g1);
@@ -648,8 +647,8 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
       const uint4 w1 = philox_oct((uint64_t)src * (uint64_t)CO + (uint64_t)o, 1u, key);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const float vv = __fmul_rn(__fsub_rn(x[j], gmin), s_g1_16);
-        c[j] = sr_code16(vv, u16_of(w1, j), 255u);
+        const float vv = __fmul_rn(__fsub_rn(x[j], gmin), s_g1);
+        c[j] = sr_code(vv, u16_of(w1, j), 255u);
         rs1 += (int)c[j];
         cs[j] += (int)c[j];
       }
@@ -762,8 +761,8 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
           const uint4 w1 = philox_oct((uint64_t)src[r] * (uint64_t)CO + (uint64_t)o, 1u, key);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float vv = __fmul_rn(__fsub_rn(x[r][j], gmin), s_g1_16);
-            c[j] = sr_code16(vv, u16_of(w1, j), 255u);
+            const float vv = __fmul_rn(__fsub_rn(x[r][j], gmin), s_g1);
+            c[j] = sr_code(vv, u16_of(w1, j), 255u);
             rs1 += (int)c[j];
             cs[j] += (int)c[j];
           }
@@ -973,8 +972,8 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
           const uint4 w1 = philox_oct((uint64_t)src * (uint64_t)CO + (uint64_t)o, 1u, key);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float vv = __fmul_rn(__fsub_rn(x[j], gmin), s_g1_16);
-            c[j] = sr_code16(vv, u16_of(w1, j), 255u);
+            const float vv = __fmul_rn(__fsub_rn(x[j], gmin), s_g1);
+            c[j] = sr_code(vv, u16_of(w1, j), 255u);
             rs1 += (int)c[j];
             cs[j] += (int)c[j];
           }
@@ -1125,7 +1124,6 @@ __global__ void __launch_bounds__(256) k_bhq_groups_big(const QuantArgs a) {
   const uint32_t B2 = (1u << a.bits) - 1u;
   const uint32_t og2 = (B2 + 1u) >> 1;
   const float s_g1 = affine_scale(gmin, gmax, 255u);
-  const float s_g1_16 = __fmul_rn(s_g1, 65536.0f);
   const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
   PhiloxKeys key;
 #pragma unroll
@@ -1264,8 +1262,8 @@ __global__ void __launch_bounds__(256) k_bhq_groups_big(const QuantArgs a) {
         const uint4 w1 = philox_oct((uint64_t)src * (uint64_t)CO + (uint64_t)o, 1u, key);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const float vv = __fmul_rn(__fsub_rn(x[j], gmin), s_g1_16);
-          c[j] = sr_code16(vv, u16_of(w1, j), 255u);
+          const float vv = __fmul_rn(__fsub_rn(x[j], gmin), s_g1);
+          c[j] = sr_code(vv, u16_of(w1, j), 255u);
           rs1 += (int)c[j];
           cs[j] += (int)c[j];
         }

@@ -218,7 +218,6 @@ __global__ void __launch_bounds__(NTMAX) k_quant(const QuantArgs a) {
   const uint32_t B2 = (1u << a.bits) - 1u;
   const float s_g2 = affine_scale(gmin, gmax, B2);    // PTQ / DET scale
   const float s_g1 = affine_scale(gmin, gmax, 255u);  // Q_b1 scale
-  const float s_g1_16 = __fmul_rn(s_g1, 65536.0f);
   const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
   if (blockIdx.x == 0 && tid == 0) {
     if (KIND == KIND_PTQ || KIND == KIND_DET) {
@@ -600,7 +599,6 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
   const uint32_t B2 = (1u << a.bits) - 1u;
   const float s_g2 = affine_scale(gmin, gmax, B2);
   const float s_g1 = affine_scale(gmin, gmax, 255u);
-  const float s_g1_16 = __fmul_rn(s_g1, 65536.0f);
   const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
   if (blockIdx.x == 0 && tid == 0) {
     if (KIND == KIND_PTQ) {
@@ -769,7 +767,6 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
         }
         z2 = seg_reduce(tmin, LPR, OpMin());
       }
-      const float s2_16 = __fmul_rn(s2, 65536.0f);
       int rs2 = 0, rs1 = 0;
 #pragma unroll
       for (int k = 0; k < kMaxOct; ++k) {
@@ -783,11 +780,11 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
           float v;
           if (KIND == KIND_BHQ) {
             const float t = fmaf(-c_row, wrow[o * 8 + j], __fmul_rn(s2, x[k][j]));
-            v = __fmul_rn(__fsub_rn(t, z2), 65536.0f);
+            v = __fsub_rn(t, z2);
           } else {
-            v = __fmul_rn(__fsub_rn(x[k][j], z2), s2_16);  // = v 2^16 exactly
+            v = __fmul_rn(__fsub_rn(x[k][j], z2), s2);
           }
-          c[j] = sr_code16(v, u16_of(w2, j), B2);
+          c[j] = sr_code(v, u16_of(w2, j), B2);
           rs2 += (int)c[j];
         }
         if (a.c2) store_codes8(a.c2 + row * (int64_t)C + o * 8, c);
@@ -796,8 +793,8 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
           const uint4 w1 = philox_oct(q, 1u, key);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float v = __fmul_rn(__fsub_rn(x[k][j], gmin), s_g1_16);
-            c[j] = sr_code16(v, u16_of(w1, j), 255u);
+            const float v = __fmul_rn(__fsub_rn(x[k][j], gmin), s_g1);
+            c[j] = sr_code(v, u16_of(w1, j), 255u);
             rs1 += (int)c[j];
           }
           if (a.c1) store_codes8(a.c1 + row * (int64_t)C + o * 8, c);
@@ -933,7 +930,6 @@ __global__ void __launch_bounds__(256) k_shift(const QuantArgs a) {
   if (!(M > 0.0f) || !isfinite(s)) s = 1.0f;
   const float inv = __fdiv_rn(1.0f, s);
   const float s_g1 = affine_scale(gmin, gmax, 255u);
-  const float s_g1_16 = __fmul_rn(s_g1, 65536.0f);
   const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
   if (blockIdx.x == 0 && tid == 0) {
     a.sscale[0] = __fmul_rn(inv, 0.0625f);
@@ -1002,8 +998,8 @@ __global__ void __launch_bounds__(256) k_shift(const QuantArgs a) {
         const uint4 w1 = philox_oct(qi, 1u, key);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const float vv = __fmul_rn(__fsub_rn(x[q][j], gmin), s_g1_16);
-          c[j] = sr_code16(vv, u16_of(w1, j), 255u);
+          const float vv = __fmul_rn(__fsub_rn(x[q][j], gmin), s_g1);
+          c[j] = sr_code(vv, u16_of(w1, j), 255u);
           rs1 += (int)c[j];
           cs1[q][j] += (int)c[j];
         }

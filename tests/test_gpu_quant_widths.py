@@ -162,3 +162,29 @@ def test_grad_w_reduction_shapes(n, c, d):
     got = gw.double().cpu().numpy()
     floor = 1e-3 * np.abs(ref).max(axis=1, keepdims=True)
     assert (np.abs(got - ref) / np.maximum(np.abs(ref), floor)).max() <= 1e-3
+
+
+@pytest.mark.parametrize("n,c,kind,block,small", [
+    (200, 136, orc.PTQ, 0, False), (200, 136, orc.PSQ, 0, False), (200, 136, orc.PSQ, 0, True),
+    (200, 136, orc.BHQ, 16, False), (200, 136, orc.BHQ, 16, True), (200, 16, orc.BHQ, 2, False),
+    (200, 64, orc.BHQ, 16, False), (200, 64, orc.BHQ, 0, False), (300, 256, orc.BHQ, 0, False),
+    (200, 64, orc.SHIFT, 0, False)])
+@pytest.mark.parametrize("scale", [1e-31, 1e-33, 1e-36])
+def test_tiny_ranges(n, c, kind, block, small, scale):
+    """Ranges whose scale B / R is far above 2^112: the codes of every kernel are
+    the oracle's (adaptive groups: of Q_b1, whose rows no grouping orders)."""
+    dH = (wl.random_grad(wl.rng(5), n, c, 0.0, 0.0) * np.float32(scale)).astype(np.float32)
+    ws = fqt.Workspace(n, c, 16)
+    if small:
+        ws = fqt.Workspace(1, 16, 16)
+        ws.nbytes = 256 + 32768  # the header and the range partials
+    q2, q1 = fqt.quantize_grad(to_dev(dH, "f32"), kind, 5, block, 7, ws=ws)
+    assert fqt.sync_status(ws) == 0
+    ref = orc.quantize_grad(dH, orc.PTQ, 8, 0, 7, orc.STREAM_B1)
+    assert np.array_equal(q1.to_numpy()["codes"], ref["codes"])
+    if kind != orc.BHQ:
+        ref = orc.quantize_grad(dH, kind, 5, block, 7, orc.STREAM_B2)
+        assert np.array_equal(q2.to_numpy()["codes"], ref["codes"])
+    elif block:
+        ref = orc.quantize_grad(dH, kind, 5, block, 7, orc.STREAM_B2, want_v=True)
+        _check_bhq_codes(q2.to_numpy()["codes"], ref["codes"], ref["v"], 7)
