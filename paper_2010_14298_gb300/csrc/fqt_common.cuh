@@ -389,7 +389,10 @@ __device__ __forceinline__ HhConst hh_const(int n) {
 
 // The block scalars s1, s2 of App. D.4, rho = 1/sqrt(nb) and kappa = 1/(1 -
 // rho) of a block of nrows rows, from the lead row's norm np and range and
-// twice the next norm (all zero for a zero block).
+// twice the next norm (all zero for a zero block).  They grow as 1 / lambda:
+// where subnormal gradients take one past fp32, those rows count as zeros (an
+// infinite scale gave z' = -inf and NaN in grad_X): s2 = 0, the limit of lambda2
+// -> 0, and with s1 out of range too a zero block.
 struct BhqScale {
   float s1, s2, rho, kap;
 };
@@ -406,9 +409,12 @@ __device__ __forceinline__ BhqScale bhq_scale(float np, float lam1, float lam2, 
       const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
       r.s1 = fB2 * n6 / (c1 * den);
       r.s2 = fB2 * n6 / (c2 * den);
-    } else {
-      r.s1 = fB2 * sqrtf(Nf) / lam1;
     }
+    if (!(lam2 > 0.0f) || !isfinite(r.s2)) {
+      r.s1 = fB2 * sqrtf(Nf) / lam1;
+      r.s2 = 0.0f;
+    }
+    if (!isfinite(r.s1)) return {0.0f, 0.0f, 0.0f, 0.0f};
     if (nrows > 1) {
       r.rho = 1.0f / sqrtf(Nf);
       r.kap = 1.0f / (1.0f - r.rho);
@@ -424,17 +430,17 @@ static __device__ __noinline__ BhqScale bhq_scale_f64(float np, float lam1, floa
   if (np > 0.0f) {
     if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
     const double Nd = (double)nrows, B = (double)((1u << bits) - 1u);
-    double s1, s2 = 0.0;
     if (lam2 > 0.0f) {
       const double c1 = cbrt((double)lam1), c2 = cbrt((double)lam2);
       const double den = c1 * c1 * pow(Nd, -1.0 / 3.0) + c2 * c2 * pow(Nd, 2.0 / 3.0);
-      s1 = B * pow(Nd, 1.0 / 6.0) / (c1 * den);
-      s2 = B * pow(Nd, 1.0 / 6.0) / (c2 * den);
-    } else {  // limit lambda2 -> 0: the other rows are zero
-      s1 = B * sqrt(Nd) / (double)lam1;
+      r.s1 = (float)(B * pow(Nd, 1.0 / 6.0) / (c1 * den));
+      r.s2 = (float)(B * pow(Nd, 1.0 / 6.0) / (c2 * den));
     }
-    r.s1 = (float)s1;
-    r.s2 = lam2 > 0.0f ? (float)s2 : 0.0f;
+    if (!(lam2 > 0.0f) || !isfinite(r.s2)) {  // limit lambda2 -> 0: the other rows are zero
+      r.s1 = (float)(B * sqrt(Nd) / (double)lam1);
+      r.s2 = 0.0f;
+    }
+    if (!isfinite(r.s1)) return {0.0f, 0.0f, 0.0f, 0.0f};
     if (nrows > 1) {
       const double rho = 1.0 / sqrt(Nd);
       r.rho = (float)rho;

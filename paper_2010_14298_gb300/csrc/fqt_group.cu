@@ -624,6 +624,7 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
       float lam1 = __fsub_rn(mm.y, mm.x);
       if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
       s1f = (float)B2 * sqrtf(1.0f) / lam1;
+      if (!isfinite(s1f)) s1f = 0.0f;  // (see bhq_scale)
     }
     float t[8];
     float tmin = INFINITY;
@@ -904,25 +905,8 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
     const float lam2 = 2.0f * l2;
     const float np = fmaxf(fabsf(pmin), fabsf(pmax));
     // ---- group scalars s1, s2 (App. D.4) and the reflection ----
-    float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
-    if (np > 0.0f) {
-      float lam1 = __fsub_rn(pmax, pmin);
-      if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
-      const float Nf = (float)nb;
-      if (lam2 > 0.0f) {
-        const float c1 = cbrtf(lam1), c2 = cbrtf(lam2);
-        const float n3 = cbrtf(Nf), n6 = sqrtf(n3);
-        const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
-        s1f = (float)B2 * n6 / (c1 * den);
-        s2f = (float)B2 * n6 / (c2 * den);
-      } else {
-        s1f = (float)B2 * sqrtf(Nf) / lam1;
-      }
-      if (nb > 1) {
-        rho = 1.0f / sqrtf(Nf);
-        kap = 1.0f / (1.0f - rho);
-      }
-    }
+    const BhqScale sc = bhq_scale(np, __fsub_rn(pmax, pmin), lam2, nb, (float)B2);
+    const float s1f = sc.s1, s2f = sc.s2, rho = sc.rho, kap = sc.kap;
     // w_j = sum_k e_k s_k h_kj, e_lead = kap (rho - 1), e_small = kap rho
     const float el = kap * (rho - 1.0f), es = kap * rho;
     float w[8];
@@ -1196,23 +1180,8 @@ __global__ void __launch_bounds__(256) k_bhq_groups_big(const QuantArgs a) {
   for (int j = 0; j < 8; ++j) xl[j] = lead_s[o * 8 + j];
   const float lam2 = 2.0f * l2;
   const float np = fmaxf(fabsf(pmin), fabsf(pmax));
-  float s1f = 0.0f, s2f = 0.0f, rho = 0.0f, kap = 0.0f;
-  if (np > 0.0f) {
-    float lam1 = __fsub_rn(pmax, pmin);
-    if (!(lam1 > 0.0f)) lam1 = 2.0f * np;
-    const float Nf = (float)nb;
-    if (lam2 > 0.0f) {
-      const float c1 = cbrtf(lam1), c2 = cbrtf(lam2);
-      const float n3 = cbrtf(Nf), n6 = sqrtf(n3);
-      const float den = c1 * c1 / n3 + c2 * c2 * n3 * n3;
-      s1f = (float)B2 * n6 / (c1 * den);
-      s2f = (float)B2 * n6 / (c2 * den);
-    } else {
-      s1f = (float)B2 * sqrtf(Nf) / lam1;
-    }
-    rho = 1.0f / sqrtf(Nf);
-    kap = 1.0f / (1.0f - rho);
-  }
+  const BhqScale sc = bhq_scale(np, __fsub_rn(pmax, pmin), lam2, nb, (float)B2);
+  const float s1f = sc.s1, s2f = sc.s2, rho = sc.rho, kap = sc.kap;
   const float el = kap * (rho - 1.0f), es = kap * rho;
   float w[8];
 #pragma unroll

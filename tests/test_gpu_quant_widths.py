@@ -188,3 +188,29 @@ def test_tiny_ranges(n, c, kind, block, small, scale):
     elif block:
         ref = orc.quantize_grad(dH, kind, 5, block, 7, orc.STREAM_B2, want_v=True)
         _check_bhq_codes(q2.to_numpy()["codes"], ref["codes"], ref["v"], 7)
+
+
+@pytest.mark.parametrize("n,c,block", [(50, 48, 1), (50, 64, 4), (50, 48, 16), (200, 64, 16),
+                                       (77, 64, 32), (777, 64, 128), (61, 1040, 16), (200, 16, 2),
+                                       (300, 64, 0), (300, 256, 0)])
+@pytest.mark.parametrize("scale", [1e-37, 1e-39, 1e-43])
+def test_bhq_of_subnormal_gradients(n, c, block, scale):
+    """Blocks whose scales s1, s2 = O(B / lambda) overflow fp32 hold zeros, so
+    that their rows of grad_X are zeros and not NaN."""
+    g = wl.rng(8)
+    dH = (wl.random_grad(g, n, c, 0.0, 0.0) * np.float32(scale)).astype(np.float32)
+    dH[: n // 4] = 0.0
+    X = to_dev(g.standard_normal((n, 32)).astype(np.float32), "f32")
+    W = to_dev(g.standard_normal((c, 32)).astype(np.float32), "f32")
+    ws = fqt.Workspace(n, c, 32)
+    q2, q1 = fqt.quantize_grad(to_dev(dH, "f32"), orc.BHQ, 5, block, 7, ws=ws)
+    gx, gw = fqt.linear_backward(q2, q1, fqt.quantize_act(X, 8), fqt.quantize_weight(W, 8), ws=ws)
+    assert fqt.sync_status(ws) == 0
+    for t in (q2.inv_s, q2.zero, *([] if block == 1 else [q2.hz, q2.hr])):
+        assert torch.isfinite(t).all()
+    codes = q2.to_numpy()["codes"].astype(np.int64)
+    assert np.array_equal(q2.row_sum.cpu().numpy(), codes.sum(1))
+    # |grad_X| <= c max|dH| max|W| (1 + 1 / B), with room for the transform
+    bound = 4.0 * c * float(np.abs(dH).max()) * float(W.abs().max())
+    assert torch.isfinite(gx).all() and float(gx.abs().max()) <= bound
+    assert torch.isfinite(gw).all()
