@@ -1143,6 +1143,9 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
   const int opr = cols / 8;
   const int rl = tid / opr, o = tid - rl * opr;
   const bool lane_on = rl < rpi;
+  // ROWS: the lanes of this lane's row in its warp, which agree on every ok[u]
+  const int span = min(opr, 32);
+  const unsigned row_lanes = (0xffffffffu >> (32 - span)) << (lane & ~(span - 1));
   int cs[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) cs[j] = 0;
@@ -1160,9 +1163,6 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
     }
 #pragma unroll
     for (int u = 0; u < kFwdUnroll; ++u) {
-      // the lanes that take part in the row sums below, from all lanes of the
-      // warp (i0's trip count is the CTA's); the lanes of a row agree
-      const unsigned on = ROWS ? __ballot_sync(0xffffffffu, ok[u]) : 0u;
       if (!ok[u]) continue;
       uint32_t c[8];
 #pragma unroll
@@ -1181,8 +1181,10 @@ __global__ void __launch_bounds__(kFwdMaxThreads)
         int v = 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) v += (int)c[j];
-        const int span = min(opr, 32);
-        for (int d = 1; d < span; d <<= 1) v += __shfl_xor_sync(on, v, d);
+        if (span == 32)
+          v = __reduce_add_sync(0xffffffffu, v);
+        else
+          for (int d = 1; d < span; d <<= 1) v += __shfl_xor_sync(row_lanes, v, d);
         if ((lane & (span - 1)) == 0) atomicAdd(&row_sum[row[u]], v);
       }
     }
