@@ -676,8 +676,10 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
 
   // One group of up to kSmall rows per sub-warp (n rows from k0; none: n = 0),
   // its rows in registers: the arithmetic and the order of every sum are those
-  // of a group on a whole warp below.
+  // of a group on a whole warp of four rows per step below.  Only rows of 64
+  // columns come here: the registers of wider ones cost more than it gives.
   constexpr int kSmall = kSmallGroup;
+  constexpr bool kSub = RS == kSmall;
   auto do_small = [&](int64_t k0, int n) {
     const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)n);
     int64_t src[kSmall];
@@ -723,10 +725,8 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
     float w[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      // the rows r of a sub-warp in order, then the sub-warps r % RS
-      const float csm = RS == 4   ? x[1][j] + (x[2][j] + x[3][j])
-                        : RS == 2 ? x[2][j] + (x[1][j] + x[3][j])
-                                  : (x[1][j] + x[2][j]) + x[3][j];
+      // as on a whole warp: a row per sub-warp, the sub-warps in pairs
+      const float csm = x[1][j] + (x[2][j] + x[3][j]);
       w[j] = fmaf(es, __fmul_rn(sc.s2, csm), el * __fmul_rn(sc.s1, x[0][j]));
     }
     ff d[kSmall], R[kSmall];
@@ -788,9 +788,7 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
     }
     if (a.hz && n > 0) {
       auto total = [&](const ff (&q)[kSmall]) {
-        return RS == 4   ? ff_add(ff_add(q[0], q[1]), ff_add(q[2], q[3]))
-               : RS == 2 ? ff_add(ff_add(q[0], q[2]), ff_add(q[1], q[3]))
-                         : ff_add(ff_add(ff_add(q[0], q[1]), q[2]), q[3]);
+        return ff_add(ff_add(q[0], q[1]), ff_add(q[2], q[3]));
       };
       const HhConst hc = hh_const(n);
       const ff rsd = ff_mul(hc.rho, total(d)), rsR = ff_mul(hc.rho, total(R));
@@ -810,7 +808,6 @@ __global__ void __launch_bounds__(256, LPR == 8 ? 2 : 3) k_bhq_groups(const Quan
     }
   };
 
-  constexpr bool kSub = RS == 4;  // (wider rows: the registers cost more than it gives)
   // A warp takes slots of groups from a queue (one ahead): single groups
   // while there are any of more than kSmallGroup rows (a warp each, the
   // largest first), then RS consecutive groups: all single rows -> one step,

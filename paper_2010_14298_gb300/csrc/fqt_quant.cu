@@ -8,7 +8,8 @@
 //             rows in shared memory), fused with the 8-bit stochastic PTQ Q_b1
 //             of App. E, for the shapes and workspaces that the passes of
 //             fqt_codes.cu leave to them (bhq_pass_order):
-//             KIND_PTQ  per-tensor stochastic quantizer (Sec. 3.3),
+//             KIND_PTQ  per-tensor stochastic quantizer (Sec. 3.3; k_quant,
+//                       rows of more than 8192 columns),
 //             KIND_PSQ  per-sample quantizer (Sec. 4.1),
 //             KIND_BHQ  block Householder quantizer (Sec. 4.2, App. D.4);
 //             KIND_DET  row sums of forward operands of odd widths.
@@ -540,6 +541,7 @@ __device__ __forceinline__ V seg_reduce(V v, int LPR, Op op) {
 
 template <int KIND, typename T>
 __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
+  static_assert(KIND == KIND_PSQ || KIND == KIND_BHQ, "PTQ takes the code pass");
   extern __shared__ __align__(128) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int C = a.C, CO = a.CO;
@@ -597,18 +599,11 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
     return;
   }
   const uint32_t B2 = (1u << a.bits) - 1u;
-  const float s_g2 = affine_scale(gmin, gmax, B2);
   const float s_g1 = affine_scale(gmin, gmax, 255u);
   const bool has_b1 = a.c1 != nullptr || a.f1 != nullptr;
-  if (blockIdx.x == 0 && tid == 0) {
-    if (KIND == KIND_PTQ) {
-      a.inv2[0] = __fdiv_rn(1.0f, s_g2);
-      a.zero2[0] = __fmul_rn(s_g2, gmin);
-    }
-    if (has_b1) {
-      a.inv1[0] = __fdiv_rn(1.0f, s_g1);
-      a.zero1[0] = __fmul_rn(s_g1, gmin);
-    }
+  if (blockIdx.x == 0 && tid == 0 && has_b1) {
+    a.inv1[0] = __fdiv_rn(1.0f, s_g1);
+    a.zero1[0] = __fmul_rn(s_g1, gmin);
   }
   int32_t *const csum_g = has_b1 ? a.csum1 : a.csum2;
   const bool want_cs = csum_g != nullptr;
@@ -731,7 +726,7 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
           for (int j = 0; j < 8; ++j) x[k][j] = 0.0f;
         }
       }
-      float s2 = s_g2, z2 = gmin, c_row = 0.0f;
+      float s2, z2, c_row = 0.0f;
       const float *wrow = wcol;
       if (KIND == KIND_PSQ) {
         float2 mm = make_float2(INFINITY, -INFINITY);
@@ -748,7 +743,7 @@ __global__ void __launch_bounds__(kQ2Threads) k_quant2(const QuantArgs a) {
         mm = seg_reduce(mm, LPR, OpMinMax());
         s2 = affine_scale(mm.x, mm.y, B2);
         z2 = mm.x;
-      } else if (KIND == KIND_BHQ) {
+      } else {
         const int bb = rv ? r / nb : 0;
         const float *bp = bpar + bb * 8;
         const bool lead = rv && (r - bb * nb) == __float_as_int(bp[4]);
@@ -1677,7 +1672,9 @@ cudaError_t launch_quant2(const QuantArgs &a, bool bf16, int grid, size_t smem,
 template <int KIND, typename T>
 static cudaError_t launch_quant_t(const QuantArgs &a, int nth, int grid,
                                   size_t smem, cudaStream_t st) {
-  auto fn = nth <= 256 ? k_quant<KIND, T, 256> : k_quant<KIND, T, 1024>;
+  auto fn = k_quant<KIND, T, 1024>;
+  if constexpr (KIND != KIND_PTQ)  // (rows of up to 8192 columns take the code pass)
+    if (nth <= 256) fn = k_quant<KIND, T, 256>;
   cudaError_t e = cudaFuncSetAttribute(
       fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

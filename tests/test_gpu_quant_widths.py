@@ -82,7 +82,7 @@ def test_bhq_passes_equal_the_one_pass_quantizer(n, c, block, dtype):
         assert torch.equal(getattr(a1, f), getattr(b1, f)), f
 
 
-@pytest.mark.parametrize("c", WIDTHS + [8192])
+@pytest.mark.parametrize("c", WIDTHS + [8192, 8200])
 @pytest.mark.parametrize("kind,bits,dtype", [(orc.PTQ, 8, "f32"), (orc.PSQ, 8, "bf16"),
                                              (orc.PSQ, 4, "f32")])
 def test_affine_widths(c, kind, bits, dtype):
