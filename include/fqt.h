@@ -264,7 +264,8 @@ FQT_API fqt_status fqt_linear_backward(const fqt_qtensor *q_b2,
  * (columns (ky, kx, c_in)), codes_f16 and col_sum.  Needs k = 3, pad = 1,
  * h, w >= 2, w <= 128, cin % 32 == 0, cout % 64 == 0 and one exact chunk
  * (9 cout <= 2^(26 - b - bw)); else FQT_EUNSUPPORTED.  `workspace`: at least
- * fqt_conv_grad_x_workspace_size(cin) bytes (status word and tables).
+ * fqt_conv_grad_x_workspace_size(cin) bytes, of which the status word is used
+ * (the rest held tables that the kernel now forms on chip; the size is kept).
  */
 FQT_API size_t fqt_conv_grad_x_workspace_size(int64_t cin);
 FQT_API fqt_status fqt_conv_grad_x_nhwc(const fqt_qtensor *q_b2, const fqt_qtensor *qw,

@@ -447,6 +447,9 @@ static size_t conv_geometry(ConvXArgs &g) {
   return 1024 + 2 * (size_t)g.b_stride + (size_t)g.a_stages * g.a_bytes + kCvTailBytes;
 }
 
+// The status word is all that is used.  An earlier kernel kept two class tables
+// of C_in floats here; callers allocate, and smaller workspaces are refused, as
+// for it.
 size_t conv_grad_x_ws_bytes(int64_t cin) {
   return kGemmOffset + 2 * (size_t)kCvClasses * (size_t)(cin > 0 ? cin : 0) * sizeof(float) + 256;
 }

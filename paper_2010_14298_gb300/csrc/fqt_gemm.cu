@@ -1628,9 +1628,11 @@ fqt_status linear_backward(const fqt_qtensor *q_b2, const fqt_qtensor *q_b1,
     }
     // At most one tile of rows: wide tiles, where their plan is ahead by 10%
     // and its partials fit; an implicit im2col operand of kw = 2 to 4 taps a
-    // row then reads its pixels once per kernel row.  An explicit operand is
-    // read from HBM, which both plans wait for (64 x 576 over 131072 rows: 41
-    // and 42 us).
+    // row then reads its pixels once per kernel row.  An explicit operand gains
+    // nothing at 64 x 576 over 131072 rows (41 and 42 us with the reduction): its
+    // time is counted as at least that of reading it, which keeps such shapes
+    // here.  (That is not what they wait for: 168 MB at 60% of the DRAM peak, the
+    // tensor pipe at 25%, each CTA's chain of 69 K blocks at 0.5 us.)
     int wide = 0, row_taps = 0;
     if (Nr > 0 && !w_ok && !bytes && C <= BM && D > BN) {
       SplitPlan wp;
