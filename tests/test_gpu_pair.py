@@ -27,7 +27,8 @@ def _product(a, b):
 @pytest.mark.parametrize("n,c,d", [(2100, 528, 4112), (2063, 1008, 4096), (4097, 512, 2320),
                                    (12500, 272, 1296)])
 @pytest.mark.parametrize("kind,bits,block", [(wl.PTQ, 8, 0), (wl.PSQ, 5, 0), (wl.BHQ, 5, 16),
-                                             (wl.BHQ, 4, 64), (wl.BHQ, 8, 16)])
+                                             (wl.BHQ, 4, 64), (wl.BHQ, 8, 16), (wl.BHQ, 5, 4),
+                                             (wl.BHQ, 5, 8), (wl.BHQ, 5, 32)])
 def test_backward_pair_edges(n, c, d, kind, bits, block):
     from paper_2010_14298_gb300 import fqt
     if block * c > 65536:
@@ -44,8 +45,9 @@ def test_backward_pair_edges(n, c, d, kind, bits, block):
     px, pw = fqt.debug_last_plan(), fqt.debug_last_plan(grad_w=True)
     # (the int32 form takes pairs from eight K blocks on: not of 272 columns)
     assert px["kernel"] == ("single" if c == 272 and (kind, bits) == (wl.BHQ, 8) else "pair")
-    if kind == wl.BHQ:  # of 1008 columns some tiles leave the fp32 form
-        assert px["form"] == (0 if bits == 8 else 1 if c == 1008 else 2)
+    if kind == wl.BHQ:  # wide rows and large blocks leave less room for row offsets in fp32
+        narrow = {528: 1, 1008: 0} if block == 32 else {1008: 1}
+        assert px["form"] == (0 if bits == 8 else narrow.get(c, 2))
     if d > 4000:
         assert pw["kernel"] == "pair" and pw["fused"]
     h2, h1, hx, hw = q2.to_numpy(), q1.to_numpy(), qx.to_numpy(), qw.to_numpy()
@@ -85,3 +87,23 @@ def test_conv_grad_w_pair_edges(n, h, w, c, cout):
     assert fqt.debug_last_plan(grad_w=True)["kernel"] == "pair"
     assert _rel(ge, _product(orc.dequant(q1.to_numpy()).T, orc.dequant(qx.to_numpy()))) <= 1e-3
     assert torch.equal(gi, ge)
+
+
+@pytest.mark.parametrize("n,c,d,kernel", [(2100, 1024, 4112, "pair"), (4100, 256, 6160, "pair"),
+                                          (1638, 64, 12880, "wide"), (300, 128, 30656, "wide")])
+@pytest.mark.parametrize("bits", [5, 8])
+def test_shifted_codes_grad_w(n, c, d, kernel, bits):
+    """The shift quantizer's wide codes (exact chunks of one to eight K blocks)."""
+    from paper_2010_14298_gb300 import fqt
+    g = wl.rng(3 + n)
+    dH = torch.from_numpy(wl.random_grad(g, n, c)).cuda()
+    X = torch.from_numpy(g.uniform(-1, 1, (n, d)).astype(np.float32)).cuda()
+    qx = fqt.quantize_act(X, 8)
+    qs, _ = fqt.quantize_grad(dH, fqt.SHIFT, bits, 0, seed=3, with_b1=False)
+    ws = fqt.Workspace(n, c, d)
+    _, gw = fqt.linear_backward(qs, None, qx, None, grad_x=False, ws=ws)
+    assert fqt.sync_status(ws) == 0
+    assert fqt.debug_last_plan(grad_w=True)["kernel"] == kernel
+    a = qs.shift16.double() * qs.shift_scale[0].double()
+    x = torch.from_numpy(orc.dequant(qx.to_numpy())).cuda()
+    assert _rel(gw, (a.T @ x).cpu().numpy()) <= 1e-3
